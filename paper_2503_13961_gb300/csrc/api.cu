@@ -22,7 +22,7 @@ struct bgt_handle {
   bgt_config cfg;
   int device = 0;
   long long Pcap = 0, Fcap = 0, Kcap = 0, Kbcap = 0, Bcap = 0;
-  int Tcap = 0, Vcap = 0, Mcap = 0, nblk_cap = 0;
+  int Tcap = 0, Vcap = 0, Mcap = 0;
   void *arena = nullptr;
   size_t arena_bytes = 0;
   bgt::Work w{};
@@ -88,11 +88,11 @@ void carve(bgt_handle *h, char *base, size_t *total) {
   w.pid = c.take<int>(P);
   w.vis_seen = c.take<unsigned long long>(h->Mcap);
   w.puv = c.take<float2>(P);
-  w.pix_gidx = c.take<int>(P);
   w.T_final = c.take<float>(P);
   w.n_contrib = c.take<int>(P);
-  w.blk_cnt = c.take<int>(2 * (long long)h->nblk_cap);
-  w.blk_off = c.take<long long>(2 * ((long long)h->nblk_cap + 1));
+  const long long id_blocks = (P + bgt::kIdPixels - 1) / bgt::kIdPixels;
+  w.pix_mask = c.take<uint2>(id_blocks * (bgt::kIdPixels / 32));
+  w.blk_off = c.take<int2>(id_blocks);
   w.counters = c.take<int>(16);
   w.stats = c.take<unsigned long long>(8);
   w.status = c.take<int>(1);
@@ -121,7 +121,7 @@ void carve(bgt_handle *h, char *base, size_t *total) {
   w.b_tcount = c.take<int>(T + 1);
   w.b_tstart = c.take<long long>(T + 1);
   w.b_tfill = c.take<int>(T + 1);
-  const long long naux = std::max<long long>(std::max<long long>(T, h->nblk_cap), h->Mcap) / 4096 + 4;
+  const long long naux = std::max<long long>(T, h->Mcap) / 4096 + 4;
   w.scan_aux = c.take<long long>(2 * naux);
   w.scan_aux2 = w.scan_aux ? w.scan_aux + naux : nullptr;
   w.big_list = c.take<int>(2 * (long long)T + 2);
@@ -150,7 +150,6 @@ void carve(bgt_handle *h, char *base, size_t *total) {
   w.pg_rec = c.take<float4>(4 * F);
   w.pb_rec = c.take<float4>(2 * F);
   w.Fcap = F;
-  w.nblk = h->nblk_cap;
   w.views = h->d_views;
   w.view_pix_off = h->d_offs;
   w.view_tile_off = h->d_offs + (h->Vcap + 1);
@@ -251,6 +250,7 @@ bgt_status setup_call(bgt_handle *h, const bgt_scene *sc, const bgt_camera *cams
   p.raster_prims = h->raster_prims;
   p.bwd_dequeue = h->bwd_dequeue;
   p.chain_bps = h->chain_bps;
+  p.nsub_inv = ~0ull / (2ull * c.tess_level * c.tess_level) + 1ull;
   return BGT_OK;
 }
 
@@ -275,18 +275,14 @@ cudaError_t enqueue_fwd(bgt_handle *h, const bgt::Params &p, const bgt::Scene &s
   mark(h, 0, st);
   if (p.stats) cudaMemsetAsync(w.stats, 0, 8 * sizeof(unsigned long long), st);
   cudaMemsetAsync(w.zbuf, 0xff, sizeof(unsigned long long) * (size_t)p.P, st);
-  cudaMemsetAsync(w.g_tcount, 0, tb, st);
   cudaMemsetAsync(w.g_tfill, 0, tb, st);
-  cudaMemsetAsync(w.b_tcount, 0, tb, st);
   cudaMemsetAsync(w.b_tfill, 0, tb, st);
-  cudaMemsetAsync(w.counters, 0, 16 * sizeof(int), st);
   int k = 0;
   mark(h, 1, st);
   k += bgt::launch_raster(p, s, w, st);
   mark(h, 2, st);
-  k += bgt::launch_resolve(p, s, w, st);
+  k += bgt::launch_ids(p, s, w, st);
   mark(h, 3, st);
-  k += bgt::launch_prim_cov(p, s, w, st);
   k += bgt::launch_generate(p, s, w, st);
   mark(h, 4, st);
   k += bgt::launch_binning(p, w, st);
@@ -402,7 +398,6 @@ bgt_status bgt_create(const bgt_config *cfg, bgt_handle **out) {
   h->Mcap = cfg->max_prims;
   // tiles of all views at the smallest tile size: sum (W/8+1)(H/8+1) <= P (1/64 + 1/8) + 2 V
   h->Tcap = (int)(h->Pcap * 9 / 64 + 2ll * h->Vcap + 1);
-  h->nblk_cap = (int)((h->Pcap + 127) / 128);  // warp chunks of 128 pixels (sub-primitive generation)
   size_t total = 0;
   carve(h, nullptr, &total);
   cudaError_t e = cudaMalloc(&h->arena, total);
@@ -868,7 +863,11 @@ bgt_status bgt_get_stage(bgt_handle *h, int which, void *dst, long long bytes, l
   float *tmp = nullptr;
   switch (which) {
     case 0: src = h->w.pid; need = 4 * P; break;
-    case 1: src = h->w.puv; need = 8 * P; break;
+    case 1:
+      src = h->w.puv;
+      need = 8 * P;
+      bgt::launch_scatter_uv(p, h->w, (int)F, st);
+      break;
     case 2:
     case 3:
     case 10: {

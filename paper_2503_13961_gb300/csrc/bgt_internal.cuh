@@ -35,6 +35,8 @@ constexpr int kStatusBlendOverflow = 32;  // reserved (blend-record overflow fal
 constexpr int kRecChunk = 32;
 constexpr int kFillChunk = 8;
 
+constexpr int kIdPixels = 2048;  // pixels of a block of the I_id / compaction passes
+
 struct View {                 // one camera and its place in the batch (128 B)
   float R[9];                 // world -> camera rotation, row-major
   float t[3];
@@ -62,6 +64,7 @@ struct Params {
   // scheduling (bgt_tuning): primitives per rasterizer warp and block, warp
   // blocks per backward dequeue, persistent blocks per SM of the chain kernels
   int raster_prims, bwd_dequeue, chain_bps;
+  unsigned long long nsub_inv;  // floor((2^64 - 1) / nsub) + 1, nsub = 2 L^2: see prim_of
 };
 
 struct Scene {                // device pointers, caller-owned
@@ -106,10 +109,10 @@ struct Work {
   unsigned long long *zbuf;   // [P] depth key of the nearest flat triangle
   int *pid;                   // [P] I_id, -1 background
   unsigned long long *vis_seen;  // [M] views (bit v - v0) a primitive owns pixels in, for the visibility measures
-  float2 *puv;                // [P] I_uv (u, v)
-  int *pix_gidx;              // [P] gaussian index of a foreground pixel, else -1
-  int *blk_cnt;               // [2][nblk] foreground / boundary pixels per warp chunk of 128 pixels
-  long long *blk_off;         // [2][nblk + 1] their exclusive prefix sums (totals last)
+  float2 *puv;                // [P] I_uv (u, v), filled from g_uv when the stage buffer is read
+  uint2 *pix_mask;            // [P / 32] foreground and boundary bits of 32 consecutive pixels
+  int2 *blk_off;              // [P / kIdPixels] foreground / boundary pixels of each block of k_ids, then
+                              // their exclusive prefix sums
   int *counters;              // [16] F, Nb, K, Kb, queue heads...
   int *status;                // [1]
   // per primitive
@@ -176,7 +179,6 @@ struct Work {
   float4 *pb_rec;             // [Fcap][2] boundary point: (dl/dS, dl/dr_b), (u, v, 0, 0)
   unsigned long long *stats;  // [8] work units of the last profiled call (see Stat)
   long long Fcap;
-  int nblk;
 };
 
 // Work units counted by the blending kernels when Params::stats is set:
@@ -189,7 +191,7 @@ constexpr int kIndexBits = 27;  // Gaussian index field of a pair key (<= 134M G
 constexpr unsigned long long kIndexMask = (1ull << kIndexBits) - 1ull;
 
 enum Counter { kF = 0, kNb = 1, kK = 2, kKb = 3, kQueueFwd = 4, kQueueBwd = 5, kQueueSort = 6, kBigCount = 7,
-               kRecChunks = 8, kFillChunks = 9, kWalkCount = 10, kQueueWalk = 11, kMidCount = 12 };
+               kRecChunks = 8, kFillChunks = 9, kWalkCount = 10, kQueueWalk = 11, kMidCount = 12, kIdsDone = 13 };
 
 // ---------------------------------------------------------------------------
 // small helpers
@@ -355,6 +357,41 @@ __device__ inline long long edge_fn(int ax, int ay, int bx, int by, int px, int 
 __device__ inline bool owns_zero_edge(int ax, int ay, int bx, int by) {
   const int dx = bx - ax, dy = by - ay;
   return (dy < 0) || (dy == 0 && dx > 0);
+}
+
+// lattice vertices of the largest tessellation level, and the slot of vertex (a, b) in their order
+constexpr int kMaxVerts = (kMaxTess + 1) * (kMaxTess + 2) / 2;
+__device__ inline int vslot(int a, int b, int L) { return a * (L + 1) - a * (a - 1) / 2 + b; }
+
+__device__ inline void slot_to_ab(int vi, int L, int &a, int &b) {
+  int rem = vi;
+  a = 0;
+  while (rem >= L + 1 - a) {
+    rem -= L + 1 - a;
+    a++;
+  }
+  b = rem;
+}
+
+// Bernstein weights of the level-L lattice vertices in shared memory, written by the whole block
+// (the caller synchronizes)
+template <int N>
+__device__ inline void tabulate_lattice(int L, float *sB) {
+  constexpr int NCP = (N + 1) * (N + 2) / 2;
+  for (int vi = threadIdx.x; vi < (L + 1) * (L + 2) / 2; vi += blockDim.x) {
+    int a, b;
+    slot_to_ab(vi, L, a, b);
+    float Bw[NCP];
+    lattice_bernstein<N>(lattice_frac(a, L), lattice_frac(b, L), lattice_frac(L - a - b, L), Bw);
+#pragma unroll
+    for (int t = 0; t < NCP; t++) sB[vi * NCP + t] = Bw[t];
+  }
+}
+
+// primitive of a flat triangle's id, id / (2 L^2): the high word of id times ceil(2^64 / (2 L^2)),
+// exact for every 32-bit id (the product's excess is below id * 512 / 2^64 < 1 / 512)
+__device__ inline unsigned prim_of(unsigned gid, unsigned long long nsub_inv) {
+  return (unsigned)__umul64hi((unsigned long long)gid, nsub_inv);
 }
 
 // sub-triangle s = 2 (a L + b) + down of the level-L lattice
@@ -690,7 +727,7 @@ __device__ inline unsigned long long plain_depth_key(float depth) {
 // ---------------------------------------------------------------------------
 // host-side launchers; each returns the number of kernels it enqueued
 int launch_raster(const Params &p, const Scene &s, const Work &w, cudaStream_t st);
-int launch_resolve(const Params &p, const Scene &s, const Work &w, cudaStream_t st);
+int launch_ids(const Params &p, const Scene &s, const Work &w, cudaStream_t st);
 int launch_generate(const Params &p, const Scene &s, const Work &w, cudaStream_t st);
 int launch_binning(const Params &p, const Work &w, cudaStream_t st);
 cudaError_t configure_composite();  // opt the blending kernels into > 48 KB shared memory
@@ -698,7 +735,7 @@ cudaError_t configure_binning();    // the same for the per-tile sort
 int launch_composite_fwd(const Params &p, const Work &w, float *image, cudaStream_t st);
 int launch_composite_bwd(const Params &p, const Work &w, const float *dimage, cudaStream_t st);
 int launch_chain(const Params &p, const Scene &s, const Work &w, const Grads &g, cudaStream_t st);
-int launch_prim_cov(const Params &p, const Scene &s, const Work &w, cudaStream_t st);
+void launch_scatter_uv(const Params &p, const Work &w, int F, cudaStream_t st);
 int launch_l1_grad(const float *img, const float *target, long long n, float scale, float *dimg,
                    float *loss, cudaStream_t st);
 int launch_l2_dssim_grad(const float *img, const float *gt, int n_views, const int *sizes, float lambda,

@@ -5,8 +5,8 @@
 // 64-bit edge functions on a 1/256-pixel grid, and the nearest one per pixel
 // is kept by a 64-bit atomicMin on (~bits(1/z) << 32 | sub-triangle id), 1/z
 // the perspective-correct interpolation sum(e_i / z_i) / area2 (the nearest
-// surface has the largest 1/z). The resolve pass turns the winning key into
-// I_id and perspective-correct I_uv.
+// surface has the largest 1/z). subprim.cu turns the winning keys into I_id
+// and the perspective-correct I_uv of the foreground pixels.
 //
 // Grid: one block row per view (blockIdx.y), warps take primitives of that
 // view two at a time. Per block, the Bernstein weights of the (L+1)(L+2)/2
@@ -31,20 +31,7 @@ namespace bgt {
 namespace {
 
 constexpr int kRasterWarps = 4;
-constexpr int kMaxVerts = (kMaxTess + 1) * (kMaxTess + 2) / 2;
 constexpr int kSpan32 = 32000;    // box spans (1/256 px) below which edge functions fit 32 bits
-
-__device__ inline int vslot(int a, int b, int L) { return a * (L + 1) - a * (a - 1) / 2 + b; }
-
-__device__ inline void slot_to_ab(int vi, int L, int &a, int &b) {
-  int rem = vi;
-  a = 0;
-  while (rem >= L + 1 - a) {
-    rem -= L + 1 - a;
-    a++;
-  }
-  b = rem;
-}
 
 __device__ __forceinline__ float to_f32(int x) { return __int2float_rn(x); }
 __device__ __forceinline__ float to_f32(long long x) { return __ll2float_rn(x); }
@@ -121,14 +108,7 @@ __global__ void __launch_bounds__(kRasterWarps * 32, N <= 2 ? 8 : 6) k_raster(Pa
   const int NV = (L + 1) * (L + 2) / 2;
   const int up_count = L * (L + 1) / 2;
   const int nsub = 2 * L * L;
-  for (int vi = threadIdx.x; vi < NV; vi += blockDim.x) {
-    int a, b;
-    slot_to_ab(vi, L, a, b);
-    float Bw[NCP];
-    lattice_bernstein<N>(lattice_frac(a, L), lattice_frac(b, L), lattice_frac(L - a - b, L), Bw);
-#pragma unroll
-    for (int t = 0; t < NCP; t++) sB[vi * NCP + t] = Bw[t];
-  }
+  tabulate_lattice<N>(L, sB);
   for (int ti = threadIdx.x; ti < L * L; ti += blockDim.x) {
     int a, down, rem;
     if (ti < up_count) {
@@ -219,76 +199,6 @@ __global__ void __launch_bounds__(kRasterWarps * 32, N <= 2 ? 8 : 6) k_raster(Pa
   }
 }
 
-// Resolve: the winning key of each pixel -> I_id and perspective-correct
-// I_uv. Persistent blocks tabulate the lattice Bernstein weights once (the
-// raster's table, same operations) and recompute the winning flat triangle's
-// three vertices from it with the primitive's control points in registers.
-template <int N>
-__global__ void __launch_bounds__(256) k_resolve(Params p, Scene s, Work w) {
-  constexpr int NCP = (N + 1) * (N + 2) / 2;
-  __shared__ float sB[kMaxVerts * NCP];
-  const int L = p.L, nsub = 2 * L * L;
-  const int NV = (L + 1) * (L + 2) / 2;
-  for (int vi = threadIdx.x; vi < NV; vi += blockDim.x) {
-    int a, b;
-    slot_to_ab(vi, L, a, b);
-    float Bw[NCP];
-    lattice_bernstein<N>(lattice_frac(a, L), lattice_frac(b, L), lattice_frac(L - a - b, L), Bw);
-#pragma unroll
-    for (int t = 0; t < NCP; t++) sB[vi * NCP + t] = Bw[t];
-  }
-  __syncthreads();
-  for (int pix = blockIdx.x * blockDim.x + threadIdx.x; pix < p.P; pix += gridDim.x * blockDim.x) {
-    const unsigned long long key = w.zbuf[pix];
-    if (key == ~0ull) {
-      w.pid[pix] = -1;
-      w.puv[pix] = make_float2(0.f, 0.f);
-      continue;
-    }
-    const unsigned int gid = (unsigned int)(key & 0xffffffffu);
-    const int prim = (int)(gid / (unsigned int)nsub);
-    const int sid = (int)(gid - (unsigned int)prim * (unsigned int)nsub);
-    if (prim >= p.M) {
-      atomicOr(w.status, kStatusBadPrim);
-      w.pid[pix] = -1;
-      continue;
-    }
-    const int view = find_view(w.view_pix_off, p.V, pix);
-    const View &vw = w.views[view];
-    const float *cp = s.ctrl + (size_t)prim * NCP * 3;
-    float c[3 * NCP];
-#pragma unroll
-    for (int k = 0; k < 3 * NCP; k++) c[k] = __ldg(cp + k);
-    int va[3], vb[3];
-    subtri_verts(L, sid, va, vb);
-    RVert r[3];
-#pragma unroll
-    for (int k = 0; k < 3; k++) r[k] = vertex_from_weights<N>(sB + vslot(va[k], vb[k], L) * NCP, c, vw, p.near_z);
-    long long area2 = edge_fn(r[0].X, r[0].Y, r[1].X, r[1].Y, r[2].X, r[2].Y);
-    if (area2 < 0) {
-      RVert t = r[1]; r[1] = r[2]; r[2] = t;
-      int x = va[1]; va[1] = va[2]; va[2] = x;
-      x = vb[1]; vb[1] = vb[2]; vb[2] = x;
-      area2 = -area2;
-    }
-    const int local = pix - vw.pix_off;
-    const int qy = local / vw.W, qx = local - qy * vw.W;
-    const int Px = qx * 256, Py = qy * 256;
-    const long long e0 = edge_fn(r[1].X, r[1].Y, r[2].X, r[2].Y, Px, Py);
-    const long long e1 = edge_fn(r[2].X, r[2].Y, r[0].X, r[0].Y, Px, Py);
-    const long long e2 = edge_fn(r[0].X, r[0].Y, r[1].X, r[1].Y, Px, Py);
-    const float af = (float)area2;
-    const float w0 = ((float)e0 / af) / r[0].Z;
-    const float w1 = ((float)e1 / af) / r[1].Z;
-    const float w2 = ((float)e2 / af) / r[2].Z;
-    const float ws = (w0 + w1) + w2;
-    const float u = (w0 * (float)va[0] + w1 * (float)va[1] + w2 * (float)va[2]) / (ws * (float)L);
-    const float v = (w0 * (float)vb[0] + w1 * (float)vb[1] + w2 * (float)vb[2]) / (ws * (float)L);
-    w.pid[pix] = prim;
-    w.puv[pix] = make_float2(u, v);
-  }
-}
-
 }  // namespace
 
 int launch_raster(const Params &p, const Scene &s, const Work &w, cudaStream_t st) {
@@ -297,16 +207,6 @@ int launch_raster(const Params &p, const Scene &s, const Work &w, cudaStream_t s
   const int per_block = kRasterWarps * p.raster_prims;
   const dim3 grid((unsigned)((p.M + per_block - 1) / per_block), (unsigned)p.V);
   dispatch_degree(p.n, [&](auto d) { k_raster<decltype(d)::value><<<grid, kRasterWarps * 32, 0, st>>>(p, s, w); });
-  return 1;
-}
-
-int launch_resolve(const Params &p, const Scene &s, const Work &w, cudaStream_t st) {
-  if (p.P == 0) return 0;
-  int sms = 0, dev = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int blocks = min((p.P + 255) / 256, (sms > 0 ? sms : 152) * 8);
-  dispatch_degree(p.n, [&](auto d) { k_resolve<decltype(d)::value><<<blocks, 256, 0, st>>>(p, s, w); });
   return 1;
 }
 
