@@ -121,9 +121,6 @@ void carve(bgt_handle *h, char *base, size_t *total) {
   w.b_tcount = c.take<int>(T + 1);
   w.b_tstart = c.take<long long>(T + 1);
   w.b_tfill = c.take<int>(T + 1);
-  const long long naux = std::max<long long>(T, h->Mcap) / 4096 + 4;
-  w.scan_aux = c.take<long long>(2 * naux);
-  w.scan_aux2 = w.scan_aux ? w.scan_aux + naux : nullptr;
   w.big_list = c.take<int>(2 * (long long)T + 2);
   w.tile_desc = c.take<int4>(2 * (long long)T + 2);
   // headers 3/4 of the capacity, fill units 1/64 (fills are per primitive-cache miss: ~1 in 13
@@ -271,12 +268,9 @@ void mark(bgt_handle *h, int i, cudaStream_t st) {
 
 cudaError_t enqueue_fwd(bgt_handle *h, const bgt::Params &p, const bgt::Scene &s, float *images, cudaStream_t st) {
   const bgt::Work &w = h->w;
-  const size_t tb = sizeof(int) * (size_t)(p.tiles + 1);
   mark(h, 0, st);
   if (p.stats) cudaMemsetAsync(w.stats, 0, 8 * sizeof(unsigned long long), st);
   cudaMemsetAsync(w.zbuf, 0xff, sizeof(unsigned long long) * (size_t)p.P, st);
-  cudaMemsetAsync(w.g_tfill, 0, tb, st);
-  cudaMemsetAsync(w.b_tfill, 0, tb, st);
   int k = 0;
   mark(h, 1, st);
   k += bgt::launch_raster(p, s, w, st);

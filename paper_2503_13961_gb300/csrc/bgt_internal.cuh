@@ -137,7 +137,6 @@ struct Work {
   int *g_tcount, *g_tfill;    // [tiles + 1] per-tile pair counts / fill cursors
   int *b_tcount, *b_tfill;
   long long *g_tstart, *b_tstart;  // [tiles + 1] exclusive prefix sums (64-bit: no wrap)
-  long long *scan_aux, *scan_aux2; // scratch of the two tile-count (and chunk-count) scans
   int *big_list;              // [2 tiles] segments too long for one warp to sort
   int4 *tile_desc;            // [2 tiles] (view, x0 | y0 << 16, W | H << 16, view pixel offset),
                               // (Gaussian list start, length, boundary list start, length)
@@ -191,7 +190,7 @@ constexpr int kIndexBits = 27;  // Gaussian index field of a pair key (<= 134M G
 constexpr unsigned long long kIndexMask = (1ull << kIndexBits) - 1ull;
 
 enum Counter { kF = 0, kNb = 1, kK = 2, kKb = 3, kQueueFwd = 4, kQueueBwd = 5, kQueueSort = 6, kBigCount = 7,
-               kRecChunks = 8, kFillChunks = 9, kWalkCount = 10, kQueueWalk = 11, kMidCount = 12, kIdsDone = 13 };
+               kRecChunks = 8, kFillChunks = 9, kWalkCount = 10, kQueueWalk = 11, kIdsDone = 12 };
 
 // ---------------------------------------------------------------------------
 // small helpers
@@ -750,7 +749,7 @@ int launch_edge_prior(const Params &p, const Work &w, const float *edges, float 
                       cudaStream_t st);
 int launch_visibility(const Params &p, const Work &w, const int *view_off, int *view_count,
                       unsigned long long *cell_mask, cudaStream_t st);
-int launch_exclusive_scan(const int *in, long long *out, int n, long long *aux, cudaStream_t st);
-int launch_bin_sort_only(const Params &p, const Work &w, cudaStream_t st);
+// exclusive prefix sums (n + 1 values, the last the total) of two count arrays (16-byte aligned)
+int launch_scan_pair(const int *in0, long long *out0, const int *in1, long long *out1, int n, cudaStream_t st);
 
 }  // namespace bgt

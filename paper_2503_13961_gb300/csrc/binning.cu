@@ -7,95 +7,175 @@
 // index): the first digit is the whole tile id (a counting sort: per-tile
 // counts from the generation pass, an exclusive scan, one scatter), the
 // remaining 64 bits (36-bit depth key = FP32 depth bits and 5 finer bits,
-// 27-bit Gaussian index) are sorted inside each tile in shared memory. Keys
-// are unique, so the order is fully determined.
+// 27-bit Gaussian index) are sorted inside each tile by a network held in
+// registers. Keys are unique, so the order is fully determined.
 // Boundary keys are (primitive, boundary index).
+#include <cooperative_groups.h>
+
+#include <algorithm>
+
 #include "bgt_internal.cuh"
 
 namespace bgt {
 
 namespace {
 
-constexpr int kScanThreads = 256;
-constexpr int kScanItems = 16;
+// Scans of the per-tile and per-primitive counts: one launch of one cluster of
+// thread blocks. Every block sums its range of the counts, the blocks read
+// each other's sums from distributed shared memory behind one cluster
+// barrier, and each then scans its range; 8 blocks above kScanOne elements,
+// one below (a barrier less). No block waits for another but at that barrier.
+// A reduce, a scan of the block sums and a down-sweep as launches of their own took
+// ~10 us per array in the small calls, where every launch of the serial chain
+// costs 2-4 us whatever it does.
+constexpr int kScanThreads = 1024;
+constexpr int kScanItems = 4;
 constexpr int kScanChunk = kScanThreads * kScanItems;
+constexpr int kScanOne = 2 * kScanChunk;
+constexpr int kScanCluster = 8;
 
-// block-wide exclusive scan of one value per thread; returns the block total
-__device__ inline long long block_excl_scan(long long v, long long &total, long long *s_warp) {
-  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  long long x = v;
+// warp-inclusive sums of two values
+__device__ __forceinline__ void warp_scan2(long long &a, long long &b) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const long long y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) s_warp[wp] = x;
-  __syncthreads();
-  if (wp == 0) {
-    long long a = lane < nw ? s_warp[lane] : 0;
-    for (int o = 1; o < 32; o <<= 1) {
-      const long long y = __shfl_up_sync(0xffffffffu, a, o);
-      if (lane >= o) a += y;
+    const long long x = __shfl_up_sync(0xffffffffu, a, o), y = __shfl_up_sync(0xffffffffu, b, o);
+    if (lane >= o) {
+      a += x;
+      b += y;
     }
-    s_warp[lane] = a;
-  }
-  __syncthreads();
-  total = s_warp[nw - 1];
-  const long long res = (wp ? s_warp[wp - 1] : 0) + x - v;
-  __syncthreads();
-  return res;
-}
-
-__global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const int *in, int n, long long *aux) {
-  __shared__ long long s_warp[32];
-  const int base = blockIdx.x * kScanChunk;
-  long long sum = 0;
-  for (int k = 0; k < kScanItems; k++) {
-    const int i = base + k * kScanThreads + threadIdx.x;
-    if (i < n) sum += in[i];
-  }
-  long long total;
-  block_excl_scan(sum, total, s_warp);
-  if (threadIdx.x == 0) aux[blockIdx.x] = total;
-}
-
-__global__ void __launch_bounds__(kScanThreads) k_scan_top(long long *aux, int nb) {
-  __shared__ long long s_warp[32];
-  __shared__ long long s_carry;
-  if (threadIdx.x == 0) s_carry = 0;
-  __syncthreads();
-  for (int base = 0; base < nb; base += kScanThreads) {
-    const int i = base + threadIdx.x;
-    const long long v = i < nb ? aux[i] : 0;
-    long long tot;
-    const long long ex = block_excl_scan(v, tot, s_warp);
-    if (i < nb) aux[i] = ex + s_carry;
-    __syncthreads();
-    if (threadIdx.x == 0) s_carry += tot;
-    __syncthreads();
   }
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_down(const int *in, long long *out, int n,
-                                                            const long long *aux) {
-  __shared__ long long s_warp[32];
-  // each thread owns kScanItems consecutive elements
-  const int base = blockIdx.x * kScanChunk + threadIdx.x * kScanItems;
-  int v[kScanItems];
-  long long sum = 0;
+// exclusive scan over the block of two values per thread; tot: the block's sums
+__device__ inline void block_scan2(long long &a, long long &b, longlong2 &tot, longlong2 *s_warp) {
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  const long long a0 = a, b0 = b;
+  warp_scan2(a, b);
+  __syncthreads();  // s_warp is free
+  if (lane == 31) s_warp[wp] = make_longlong2(a, b);
+  __syncthreads();
+  const longlong2 v = s_warp[lane];  // 32 warps
+  longlong2 inc = v;
+  warp_scan2(inc.x, inc.y);
+  tot.x = __shfl_sync(0xffffffffu, inc.x, 31);
+  tot.y = __shfl_sync(0xffffffffu, inc.y, 31);
+  a += __shfl_sync(0xffffffffu, inc.x - v.x, wp) - a0;
+  b += __shfl_sync(0xffffffffu, inc.y - v.y, wp) - b0;
+}
+
+// Exclusive prefix sums of two count arrays (16-byte aligned, as the outputs), the totals last. Returns
+// the totals on every thread.
+template <int CL>
+__device__ inline longlong2 scan_both(const int *in0, long long *out0, const int *in1, long long *out1, int n) {
+  __shared__ longlong2 s_warp[32], s_sum;
+  const int4 *p0 = reinterpret_cast<const int4 *>(in0), *p1 = reinterpret_cast<const int4 *>(in1);
+  // this block's range [lo, hi), a multiple of kScanChunk long but for the last
+  const int chunks = (n + kScanChunk - 1) / kScanChunk, per = (chunks + CL - 1) / CL * kScanChunk;
+  const int lo = min((int)blockIdx.x * per, n), hi = min(lo + per, n);
+  longlong2 run = make_longlong2(0, 0);
+  if constexpr (CL > 1) {
+    namespace cg = cooperative_groups;
+    long long a = 0, b = 0;
+#pragma unroll 4
+    for (int i = (lo >> 2) + threadIdx.x; i < hi >> 2; i += kScanThreads) {
+      const int4 x = p0[i], y = p1[i];
+      a += ((long long)x.x + x.y) + ((long long)x.z + x.w);
+      b += ((long long)y.x + y.y) + ((long long)y.z + y.w);
+    }
+    if ((int)threadIdx.x < (hi & 3) && hi > lo) {
+      a += in0[(hi & ~3) + threadIdx.x];
+      b += in1[(hi & ~3) + threadIdx.x];
+    }
+    longlong2 sum;
+    block_scan2(a, b, sum, s_warp);
+    if (threadIdx.x == 0) s_sum = sum;
+    const cg::cluster_group cl = cg::this_cluster();
+    cl.sync();
+    for (int k = 0; k < (int)blockIdx.x; k++) {
+      const longlong2 o = *cl.map_shared_rank(&s_sum, k);
+      run.x += o.x;
+      run.y += o.y;
+    }
+    cl.sync();  // no block leaves while its sum may still be read
+  }
+  for (int base = lo; base < hi; base += kScanChunk) {
+    const int i = base + (int)threadIdx.x * kScanItems;
+    int4 x = make_int4(0, 0, 0, 0), y = x;
+    if (i + 3 < hi) {
+      x = p0[i >> 2];
+      y = p1[i >> 2];
+    } else {
+      if (i < hi) { x.x = in0[i]; y.x = in1[i]; }
+      if (i + 1 < hi) { x.y = in0[i + 1]; y.y = in1[i + 1]; }
+      if (i + 2 < hi) { x.z = in0[i + 2]; y.z = in1[i + 2]; }
+    }
+    long long a = ((long long)x.x + x.y) + ((long long)x.z + x.w), b = ((long long)y.x + y.y) + ((long long)y.z + y.w);
+    longlong2 tot;
+    block_scan2(a, b, tot, s_warp);
+    a += run.x;
+    b += run.y;
+    const long long sa[4] = {a, a + x.x, a + x.x + x.y, a + x.x + x.y + x.z};
+    const long long sb[4] = {b, b + y.x, b + y.x + y.y, b + y.x + y.y + y.z};
+    if (i + 3 < hi) {
+      longlong2 *o0 = reinterpret_cast<longlong2 *>(out0 + i), *o1 = reinterpret_cast<longlong2 *>(out1 + i);
+      o0[0] = make_longlong2(sa[0], sa[1]);
+      o0[1] = make_longlong2(sa[2], sa[3]);
+      o1[0] = make_longlong2(sb[0], sb[1]);
+      o1[1] = make_longlong2(sb[2], sb[3]);
+    } else {
 #pragma unroll
-  for (int k = 0; k < kScanItems; k++) {
-    v[k] = (base + k < n) ? in[base + k] : 0;
-    sum += v[k];
+      for (int k = 0; k < 3; k++)
+        if (i + k < hi) {
+          out0[i + k] = sa[k];
+          out1[i + k] = sb[k];
+        }
+    }
+    run.x += tot.x;
+    run.y += tot.y;
   }
-  long long total;
-  long long run = block_excl_scan(sum, total, s_warp) + aux[blockIdx.x];
-#pragma unroll
-  for (int k = 0; k < kScanItems; k++) {
-    if (base + k < n) out[base + k] = run;
-    run += v[k];
+  if (hi == n && lo < n && threadIdx.x == 0) {  // the block of the last element holds the totals
+    out0[n] = run.x;
+    out1[n] = run.y;
   }
-  // the thread holding element n - 1 also writes out[n] = grand total
-  if (base < n && base + kScanItems >= n) out[n] = run;
+  return run;
+}
+
+template <int CL>
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(kScanThreads)
+    k_scan_pair(const int *in0, long long *out0, const int *in1, long long *out1, int n) {
+  scan_both<CL>(in0, out0, in1, out1, n);
+}
+
+// Tile list starts (exclusive sums of the Gaussian and boundary counts) and the
+// capacity check, by the block that holds the last tile
+template <int CL>
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(kScanThreads) k_tile_scan(Params p, Work w) {
+  const longlong2 total = scan_both<CL>(w.g_tcount, w.g_tstart, w.b_tcount, w.b_tstart, p.tiles);
+  const int chunks = (p.tiles + kScanChunk - 1) / kScanChunk, per = (chunks + CL - 1) / CL * kScanChunk;
+  if ((int)blockIdx.x == (p.tiles - 1) / per && threadIdx.x == 0) {
+    w.counters[kK] = (int)min(total.x, 0x7fffffffll);
+    w.counters[kKb] = (int)min(total.y, 0x7fffffffll);
+    if (total.x > p.max_pairs) atomicOr(w.status, kStatusPairOverflow);
+    if (total.y > p.max_bpairs) atomicOr(w.status, kStatusBoundaryOverflow);
+  }
+}
+
+// per-tile descriptor, so that the blending kernels read two records instead
+// of searching the view offsets and reading the list starts: [2t] geometry,
+// [2t + 1] (Gaussian list start, length, boundary list start, length); an
+// overflowed list (its slots were not all written) has length 0
+__device__ inline void tile_descriptor(const Params &p, const Work &w, int t) {
+  const int view = find_view(w.view_tile_off, p.V, t);
+  const View &vw = w.views[view];
+  const int lt = t - vw.tile_off;
+  const int ty = lt / vw.tiles_x, tx = lt - ty * vw.tiles_x;
+  w.tile_desc[2 * t] = make_int4(view, (int)((unsigned)(tx * p.tile) | ((unsigned)(ty * p.tile) << 16)),
+                                 (int)((unsigned)vw.W | ((unsigned)vw.H << 16)), vw.pix_off);
+  const bool g_over = w.g_tstart[p.tiles] > p.max_pairs, b_over = w.b_tstart[p.tiles] > p.max_bpairs;
+  const long long gs = w.g_tstart[t], bs = w.b_tstart[t];
+  w.tile_desc[2 * t + 1] = make_int4(g_over ? 0 : (int)gs, g_over ? 0 : (int)(w.g_tstart[t + 1] - gs),
+                                     b_over ? 0 : (int)bs, b_over ? 0 : (int)(w.b_tstart[t + 1] - bs));
 }
 
 // a slot in tile t's segment: the active lanes of the warp that want one in
@@ -123,87 +203,128 @@ __device__ inline void emit_rect(unsigned long long *keys, int *fill, const long
     }
 }
 
+// the pair keys, unsorted, into the second halves of the key arrays (the sort
+// writes the first), and the tiles' descriptors
 __global__ void k_emit(Params p, Work w) {
   const int F = w.counters[kF], Nb = w.counters[kNb];
   const int stride = gridDim.x * blockDim.x;
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < p.tiles; t += stride) tile_descriptor(p, w, t);
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < F; i += stride) {
     const uint2 rect = w.g_rect[i];
     if ((rect.x & 0xffff) > (rect.y & 0xffff)) continue;
     const View *vw = w.views + w.g_view[i];
     const unsigned long long dkey =
         ((unsigned long long)__float_as_uint(w.g_depth[i]) << 5) | (unsigned long long)w.g_dsub[i];
-    emit_rect(w.gkeys, w.g_tfill, w.g_tstart, p.max_pairs, __ldg(&vw->tile_off), __ldg(&vw->tiles_x),
+    emit_rect(w.gkeys + p.max_pairs, w.g_tfill, w.g_tstart, p.max_pairs, __ldg(&vw->tile_off), __ldg(&vw->tiles_x),
               rect, dkey << kIndexBits, (unsigned)i);
   }
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < Nb; i += stride) {
     const uint2 rect = w.b_rect[i];
     if ((rect.x & 0xffff) > (rect.y & 0xffff)) continue;
     const View *vw = w.views + w.b_view[i];
-    emit_rect(w.bkeys, w.b_tfill, w.b_tstart, p.max_bpairs, __ldg(&vw->tile_off), __ldg(&vw->tiles_x),
+    emit_rect(w.bkeys + p.max_bpairs, w.b_tfill, w.b_tstart, p.max_bpairs, __ldg(&vw->tile_off), __ldg(&vw->tiles_x),
               rect, (unsigned long long)(unsigned)w.b_prim[i] << 32, (unsigned)i);
   }
-}
-
-// per-tile descriptor, so that the blending kernels read two records instead
-// of searching the view offsets and reading the list starts: [2t] geometry,
-// [2t + 1] (Gaussian list start, length, boundary list start, length); an
-// overflowed list (its slots were not all written) has length 0
-__global__ void k_tile_desc(Params p, Work w) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= p.tiles) return;
-  const int view = find_view(w.view_tile_off, p.V, t);
-  const View &vw = w.views[view];
-  const int lt = t - vw.tile_off;
-  const int ty = lt / vw.tiles_x, tx = lt - ty * vw.tiles_x;
-  w.tile_desc[2 * t] = make_int4(view, (int)((unsigned)(tx * p.tile) | ((unsigned)(ty * p.tile) << 16)),
-                                 (int)((unsigned)vw.W | ((unsigned)vw.H << 16)), vw.pix_off);
-  const bool g_over = w.g_tstart[p.tiles] > p.max_pairs, b_over = w.b_tstart[p.tiles] > p.max_bpairs;
-  const long long gs = w.g_tstart[t], bs = w.b_tstart[t];
-  w.tile_desc[2 * t + 1] = make_int4(g_over ? 0 : (int)gs, g_over ? 0 : (int)(w.g_tstart[t + 1] - gs),
-                                     b_over ? 0 : (int)bs, b_over ? 0 : (int)(w.b_tstart[t + 1] - bs));
-}
-
-__global__ void k_check_capacity(Params p, Work w) {
-  const long long K = w.g_tstart[p.tiles], Kb = w.b_tstart[p.tiles];
-  w.counters[kK] = (int)(K < 0x7fffffffll ? K : 0x7fffffffll);
-  w.counters[kKb] = (int)(Kb < 0x7fffffffll ? Kb : 0x7fffffffll);
-  if (K > p.max_pairs) atomicOr(w.status, kStatusPairOverflow);
-  if (Kb > p.max_bpairs) atomicOr(w.status, kStatusBoundaryOverflow);
 }
 
 // ---------------------------------------------------------------------------
 // per-tile sort
 // ---------------------------------------------------------------------------
-constexpr int kSortThreads = 256;
-constexpr int kSortCap = 4096;  // keys sorted in shared memory (32 KB)
+constexpr int kSortThreads = 128;
+constexpr int kSortWarps = kSortThreads / 32;
+constexpr int kRunCap = 512;                    // keys one warp sorts in registers (16 per lane)
+constexpr int kWarpSortCap = 2 * kRunCap;       // keys one warp sorts: two such runs, merged
+constexpr int kSortCap = kSortWarps * kWarpSortCap;  // keys one block sorts in shared memory
+constexpr int kFullKeys = 1 << 30;              // flag of a listed segment: its order needs all key bits
 
-__device__ void bitonic_smem(unsigned long long *s, int n) {
-  int N = 1;
-  while (N < n) N <<= 1;
-  for (int i = n + threadIdx.x; i < N; i += blockDim.x) s[i] = ~0ull;
-  __syncthreads();
-  // every thread takes compare-exchange pairs (i, i + j): pair p has
-  // i = (p with a zero bit inserted at j), so no thread idles on the
-  // upper half of a pair
-  for (int k = 2; k <= N; k <<= 1)
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int q = threadIdx.x; q < (N >> 1); q += blockDim.x) {
-        const int i = ((q & ~(j - 1)) << 1) | (q & (j - 1));
-        const unsigned long long a = s[i], b = s[i + j];
-        const bool up = (i & k) == 0;
-        if ((a > b) == up) {
-          s[i] = b;
-          s[i + j] = a;
-        }
-      }
-      __syncthreads();
-    }
+// position of key i in shared memory: one key of padding per 16, so that lanes
+// writing runs of consecutive keys (16 apart, say) hit distinct banks
+__host__ __device__ constexpr int padded(int i) { return i + (i >> 4); }
+constexpr int kWarpWords = padded(kWarpSortCap);  // a warp's words; every warp and block holds them twice
+constexpr int kSortBigSmem = 2 * kSortWarps * kWarpWords * (int)sizeof(unsigned);
+static_assert(kSortBigSmem >= padded(kSortCap) * (int)sizeof(unsigned long long), "the keys of a segment fit as well");
+
+__device__ __forceinline__ void key_order(unsigned &a, unsigned &b) {
+  const unsigned lo = min(a, b);
+  b = max(a, b);
+  a = lo;
 }
 
-// Stable block-wide LSD radix sort (8-bit digits) of a segment in global
-// memory, for segments larger than the shared-memory capacity. Digits that
-// are equal across the whole segment are skipped.
-__device__ void radix_global(unsigned long long *keys, unsigned long long *tmp, int n, int *s_hist,
+__device__ __forceinline__ void take_order(unsigned &k, unsigned o, bool upper) {
+  const unsigned lo = min(k, o), hi = max(k, o);
+  k = upper ? hi : lo;
+}
+
+__device__ __forceinline__ void take_order(unsigned long long &k, unsigned long long o, bool upper) {
+  k = (o < k) != upper ? o : k;
+}
+
+__device__ __forceinline__ void key_order(unsigned long long &a, unsigned long long &b) {
+  const bool swap = b < a;
+  const unsigned long long lo = swap ? b : a;
+  b = swap ? a : b;
+  a = lo;
+}
+
+// Batcher's odd-even merge network (1968) of E keys in one lane's registers:
+// stages p = 1, 2, .. E / 2, in each distances q = p, p / 2, .. 1
+template <int E, int P, int Q, class Key>
+__device__ __forceinline__ void odd_even_stage(Key (&k)[E]) {
+#pragma unroll
+  for (int i = Q % P; i + Q < E; i++)
+    if ((i - Q % P) % (2 * Q) < Q && i / (2 * P) == (i + Q) / (2 * P)) key_order(k[i], k[i + Q]);
+  if constexpr (Q > 1) odd_even_stage<E, P, Q / 2>(k);
+  else if constexpr (2 * P < E) odd_even_stage<E, 2 * P, 2 * P>(k);
+}
+
+// bitonic merge of a lane's keys: distances J, J / 2, .. 1
+template <int E, int J, class Key>
+__device__ __forceinline__ void halving_steps(Key (&k)[E]) {
+#pragma unroll
+  for (int e = 0; e < E; e++)
+    if (!(e & J)) key_order(k[e], k[e | J]);
+  if constexpr (J > 1) halving_steps<E, J / 2>(k);
+}
+
+// Sort of 32 E keys by one warp in registers, ascending, key i in lane i / E,
+// register i % E: every lane sorts its own keys (no shuffles), then lane groups of 2, 4, .. 32 merge
+// bitonically: a first step against the mirrored position of the other half
+// (so that every comparison is ascending), then halving distances, by
+// shuffles down to one lane and in registers inside it. 15 shuffle steps at
+// any E; neighbouring keys in one lane is what keeps them this few (keys 32
+// apart per lane need 35 at 512 keys).
+template <int E, class Key>
+__device__ __forceinline__ void warp_sort_regs(Key (&k)[E], int lane) {
+  if constexpr (E > 1) odd_even_stage<E, 1, 1>(k);
+#pragma unroll 1
+  for (int s = 2; s <= 32; s <<= 1) {
+    {
+      const bool upper = lane & (s >> 1);
+#pragma unroll
+      for (int e = 0; e < (E + 1) / 2; e++) {
+        const Key oa = __shfl_xor_sync(0xffffffffu, k[E - 1 - e], s - 1);
+        if (E > 1) {
+          const Key ob = __shfl_xor_sync(0xffffffffu, k[e], s - 1);
+          take_order(k[E - 1 - e], ob, upper);
+        }
+        take_order(k[e], oa, upper);
+      }
+    }
+#pragma unroll 1
+    for (int j = s >> 2; j >= 1; j >>= 1) {
+      const bool upper = lane & j;
+#pragma unroll
+      for (int e = 0; e < E; e++) take_order(k[e], __shfl_xor_sync(0xffffffffu, k[e], j), upper);
+    }
+    if constexpr (E > 1) halving_steps<E, E / 2>(k);
+  }
+}
+
+// Stable block-wide LSD radix sort (8-bit digits) of the segment `keys` in
+// global memory into `out`, for segments larger than the shared-memory
+// capacity; `keys` is scratch afterwards. Digits that are equal across the
+// whole segment are skipped.
+__device__ void radix_global(unsigned long long *keys, unsigned long long *out, int n, int *s_hist,
                              int *s_base, int *s_wcnt, unsigned long long *s_red) {
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, nw = kSortThreads / 32;
   // OR / AND over the segment to find constant digits
@@ -222,7 +343,7 @@ __device__ void radix_global(unsigned long long *keys, unsigned long long *tmp, 
   for (int i = 0; i < nw; i++) { vor |= s_red[i]; vand &= s_red[nw + i]; }
   __syncthreads();
   const unsigned long long varying = vor ^ vand;
-  unsigned long long *src = keys, *dst = tmp;
+  unsigned long long *src = keys, *dst = out;
   for (int shift = 0; shift < 64; shift += 8) {
     if (((varying >> shift) & 0xffull) == 0ull) continue;
     for (int d = threadIdx.x; d < 256; d += kSortThreads) s_hist[d] = 0;
@@ -259,19 +380,10 @@ __device__ void radix_global(unsigned long long *keys, unsigned long long *tmp, 
     }
     unsigned long long *t = src; src = dst; dst = t;
   }
-  if (src != keys)
-    for (int i = threadIdx.x; i < n; i += kSortThreads) keys[i] = src[i];
+  if (src != out)
+    for (int i = threadIdx.x; i < n; i += kSortThreads) out[i] = src[i];
   __syncthreads();
 }
-
-constexpr int kWarpSortCap = 512;  // keys a single warp sorts in its own shared memory (occupancy:
-                                   // 16 keys per lane in registers, 36 KB of shared memory per block)
-constexpr int kMidSortCap = 1024;  // longer segments up to this: one warp each in k_tile_sort_mid
-                                   // (32 keys per lane, 72 KB of shared memory per block)
-constexpr int kRadixMin = 129;     // segments from this length sort by radix, shorter ones by bitonic network
-// per warp: the keys (kWarpSortCap) and 256 radix bins
-constexpr int kTileSortSmem = (kSortThreads / 32) * (kWarpSortCap * (int)sizeof(unsigned long long) + 256 * 4);
-constexpr int kTileSortMidSmem = (kSortThreads / 32) * (kMidSortCap * (int)sizeof(unsigned long long) + 256 * 4);
 
 __device__ inline void segment_bounds(const Params &p, const Work &w, int item, bool &bnd, long long &s0,
                                       long long &s1) {
@@ -285,280 +397,414 @@ __device__ inline void segment_bounds(const Params &p, const Work &w, int item, 
   s1 = s1 < s0 ? s0 : (s1 > cap ? cap : s1);
 }
 
-__device__ inline void gather_boundary(const Work &w, long long s0, long long s1, int lane, int step) {
-  for (long long i = s0 + lane; i < s1; i += step) {
-    const unsigned long long k = w.bkeys[i];
-    w.bl_prim[i] = (int)(k >> 32);
-    w.bl_rec[i] = w.bR[(unsigned)(k & 0xffffffffu)];
-  }
-}
-
-// Bitonic sort of sk[0, N) (N a power of two, 64..kWarpSortCap) by one warp:
-// every stage is N / 2 independent compare-exchanges, 1 / 32 of them per lane.
-__device__ __forceinline__ void warp_bitonic_smem(unsigned long long *sk, int N, int lane) {
-  for (int k = 2; k <= N; k <<= 1)
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int t = lane; t < (N >> 1); t += 32) {
-        const int i = ((t & ~(j - 1)) << 1) | (t & (j - 1));  // i has bit j clear; its partner is i + j
-        const unsigned long long a = sk[i], b = sk[i + j];
-        if ((a > b) == ((i & k) == 0)) {
-          sk[i] = b;
-          sk[i + j] = a;
-        }
-      }
-      __syncwarp();
-    }
-}
-
-// Stable LSD radix sort (8-bit digits) of sk[0, n) (n <= 32 R) by
-// one warp on the key bits from lo_shift up: the keys sit in registers, key i
-// in lane i % 32, slot i / 32; each pass histograms the digit into `bins`,
-// scans it and scatters the keys back to sk in order, ranking equal digits of
-// a round with a match; digits that are equal over the whole segment are
-// skipped. Keys equal above lo_shift keep their input order.
-template <int R>  // n <= 32 R
-__device__ __forceinline__ void warp_radix_smem(unsigned long long *sk, unsigned *bins, int n, int lane,
-                                                int lo_shift) {
-  const int rounds = (n + 31) >> 5;
-  const unsigned lt = (1u << lane) - 1u;
-  unsigned long long key[R];
-  unsigned long long vor = 0ull, vand = ~0ull;
-#pragma unroll
-  for (int r = 0; r < R; r++) {
-    key[r] = 0ull;
-    if (r < rounds && r * 32 + lane < n) {
-      key[r] = sk[r * 32 + lane];
-      vor |= key[r];
-      vand &= key[r];
-    }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    vor |= __shfl_xor_sync(0xffffffffu, vor, o);
-    vand &= __shfl_xor_sync(0xffffffffu, vand, o);
-  }
-  const unsigned long long varying = vor ^ vand;
-  for (int shift = lo_shift; shift < 64; shift += 8) {
-    if (((varying >> shift) & 0xffull) == 0ull) continue;
-    for (int d = lane; d < 256; d += 32) bins[d] = 0u;
-    __syncwarp();
-#pragma unroll
-    for (int r = 0; r < R; r++)
-      if (r < rounds && r * 32 + lane < n) atomicAdd(&bins[(unsigned)(key[r] >> shift) & 0xffu], 1u);
-    __syncwarp();
-    // exclusive scan of the 256 bins: 8 consecutive bins per lane
-    unsigned c[8], tot = 0u;
-#pragma unroll
-    for (int q = 0; q < 8; q++) {
-      c[q] = bins[lane * 8 + q];
-      tot += c[q];
-    }
-    unsigned inc = tot;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned y = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += y;
-    }
-    unsigned run = inc - tot;
-#pragma unroll
-    for (int q = 0; q < 8; q++) {
-      bins[lane * 8 + q] = run;
-      run += c[q];
-    }
-    __syncwarp();
-    // stable scatter, one round of 32 keys at a time
-#pragma unroll
-    for (int r = 0; r < R; r++) {
-      if (r >= rounds) break;
-      const bool valid = r * 32 + lane < n;
-      const unsigned d = valid ? ((unsigned)(key[r] >> shift) & 0xffu) : 0x100u + lane;
-      const unsigned peers = __match_any_sync(0xffffffffu, d);
-      const unsigned base = valid ? bins[d] : 0u;
-      if (valid) sk[base + __popc(peers & lt)] = key[r];
-      __syncwarp();
-      if (valid && lane == 31 - __clz(peers)) bins[d] = base + __popc(peers);
-      __syncwarp();
-    }
-#pragma unroll
-    for (int r = 0; r < R; r++)
-      if (r < rounds && r * 32 + lane < n) key[r] = sk[r * 32 + lane];
-    __syncwarp();
-  }
-}
-
-// A segment staged in sk[0, n) (padded with ~0 to the power of two N) sorted
-// by one warp: boundary keys by radix on all bits; Gaussian keys by their
-// depth bits only (the index below them just breaks ties), and when a tie is
-// left in emission order (rare) the full keys go through the bitonic network,
-// so the order is the (tile, depth, index) order either way.
-template <int R>
-__device__ __forceinline__ void warp_sort_segment(unsigned long long *sk, unsigned *bins, int n, int N, bool bnd,
-                                                  int lane) {
-  if (bnd) {
-    warp_radix_smem<R>(sk, bins, n, lane, 0);
+// a sorted key to its place in the list; a boundary key's record beside it
+__device__ __forceinline__ void store_sorted(const Work &w, bool bnd, long long at, unsigned long long key) {
+  if (!bnd) {
+    w.gkeys[at] = key;
     return;
   }
-  warp_radix_smem<R>(sk, bins, n, lane, kIndexBits);
-  bool tie = false;
-  for (int i = lane; i + 1 < n; i += 32) tie |= ((sk[i] ^ sk[i + 1]) >> kIndexBits) == 0ull;
-  if (__any_sync(0xffffffffu, tie)) warp_bitonic_smem(sk, N, lane);
+  w.bkeys[at] = key;
+  w.bl_prim[at] = (int)(key >> 32);
+  w.bl_rec[at] = w.bR[(unsigned)(key & 0xffffffffu)];
 }
 
-// Warps take segments from a queue. Up to 32 keys: bitonic sort across the
-// lanes' registers; up to kWarpSortCap: bitonic sort (up to 128 keys) or
-// radix sort in the warp's shared memory; longer segments are listed for
-// k_tile_sort_mid (up to kMidSortCap keys) or k_tile_sort_big.
-__global__ void __launch_bounds__(kSortThreads, 3) k_tile_sort(Params p, Work w, int *big_list) {
-  extern __shared__ __align__(16) unsigned long long s_sort[];
+// How the 64-bit keys of one segment are sorted as 32-bit words, which one
+// compare-exchange of the network moves in two instructions instead of six (and
+// the network's code, a third of the size, stays in the instruction cache).
+//   Boundary keys: (primitive - least) << lo_bits | (index - least), the key
+//   itself shortened, when both ranges fit 31 bits together.
+//   Gaussian keys: the depth key less the least FP32 depth of the segment,
+//   cut to its upper bits, with the key's position in the segment below them.
+//   Depths that differ only in the cut bits, and ties of depth, may leave
+//   neighbours out of order: words that agree above their positions are
+//   exchanged by their full keys (groups of up to 3 on the room's tiles).
+// Segments that fit neither are sorted on all key bits.
+struct WordForm {
+  unsigned hi0, lo0;  // least high word; boundary keys: least low word
+  int shift;          // Gaussian keys: bits cut off; boundary keys: lo_bits
+  bool ok;
+};
+
+// least and greatest high word of a segment; boundary keys: low words too
+struct KeyRange {
+  unsigned hi0, hi1, lo0, lo1;
+};
+
+__device__ __forceinline__ KeyRange key_range(const unsigned long long *keys, int n, int first, int step) {
+  KeyRange r{0xffffffffu, 0u, 0xffffffffu, 0u};
+  for (int i = first; i < n; i += step) {
+    const unsigned long long k = keys[i];
+    const unsigned hi = (unsigned)(k >> 32), lo = (unsigned)k;
+    r.hi0 = min(r.hi0, hi);
+    r.hi1 = max(r.hi1, hi);
+    r.lo0 = min(r.lo0, lo);
+    r.lo1 = max(r.lo1, lo);
+  }
+  r.hi0 = __reduce_min_sync(0xffffffffu, r.hi0);
+  r.hi1 = __reduce_max_sync(0xffffffffu, r.hi1);
+  r.lo0 = __reduce_min_sync(0xffffffffu, r.lo0);
+  r.lo1 = __reduce_max_sync(0xffffffffu, r.lo1);
+  return r;
+}
+
+// pos_bits: bits of a position in the segment
+__device__ __forceinline__ WordForm word_form(const KeyRange &r, bool bnd, int pos_bits) {
+  WordForm f;
+  f.hi0 = r.hi0;
+  f.lo0 = r.lo0;
+  const unsigned span = r.hi1 - r.hi0;
+  if (bnd) {
+    f.shift = 32 - __clz((int)(r.lo1 - r.lo0));
+    f.ok = f.shift + 32 - __clz((int)span) <= 31;
+  } else {
+    f.ok = span < (1u << 27);  // depth key less (hi0 << 5) fits 32 bits
+    const int bits = 32 - __clz((int)((span << 5) | 31u));
+    f.shift = max(0, bits - (32 - pos_bits));
+  }
+  return f;
+}
+
+__device__ __forceinline__ unsigned key_word(const WordForm &f, bool bnd, unsigned long long key, int pos,
+                                             int pos_bits) {
+  const unsigned hi = (unsigned)(key >> 32) - f.hi0, lo = (unsigned)key;
+  // boundary shift is below 32 (both ranges within 31 bits), pos_bits between 5 and 13
+  return bnd ? (hi << f.shift) | (lo - f.lo0)
+             : ((((hi << 5) | (lo >> kIndexBits)) >> f.shift) << pos_bits) | (unsigned)pos;
+}
+
+__device__ __forceinline__ unsigned long long word_key(const WordForm &f, bool bnd, const unsigned long long *keys,
+                                                       unsigned word, int pos_bits) {
+  if (!bnd) return keys[word & ((1u << pos_bits) - 1u)];
+  const unsigned lo = word & ((1u << f.shift) - 1u);
+  return ((unsigned long long)((word >> f.shift) + f.hi0) << 32) | (unsigned long long)(lo + f.lo0);
+}
+
+constexpr int kFixPasses = 8;  // rounds of neighbour exchanges before a list is sorted on all bits
+
+// One round of exchanges (even, then odd neighbours) among the sorted words of a
+// Gaussian list that agree above their position bits, by the full keys; true
+// if any moved. SYNC separates the two halves and ends the round.
+template <class Sync>
+__device__ __forceinline__ bool exchange_ties(const unsigned long long *keys, unsigned *s, int n, int pos_bits, int first,
+                                              int step, Sync sync) {
+  const unsigned mask = (1u << pos_bits) - 1u;
+  bool moved = false;
+  for (int odd = 0; odd < 2; odd++) {
+    for (int i = 2 * first + odd; i + 1 < n; i += 2 * step) {
+      const unsigned a = s[padded(i)], b = s[padded(i + 1)];
+      if (((a ^ b) >> pos_bits) == 0u && keys[b & mask] < keys[a & mask]) {
+        s[padded(i)] = b;
+        s[padded(i + 1)] = a;
+        moved = true;
+      }
+    }
+    sync();
+  }
+  return moved;
+}
+
+// The words of keys[0, n), n <= 32 E, with positions from `first` on, sorted by one warp into s (padded
+// positions from `first` on). Not inlined: the two runs of a segment share the
+// code of a size, which has to stay in the instruction cache (a form of 32
+// words per lane beside it made the fetches the first stall).
+template <int E>
+__device__ __noinline__ void warp_sort_run(const unsigned long long *keys, unsigned *s, WordForm f, bool bnd, int first,
+                                           int n, int pos_bits) {
+  const int lane = threadIdx.x & 31;
+  unsigned k[E];
+#pragma unroll
+  for (int e = 0; e < E; e++) {
+    const int i = e * 32 + lane;
+    k[e] = i < n ? key_word(f, bnd, keys[i], first + i, pos_bits) : 0xffffffffu;  // padding: last in any order
+  }
+  warp_sort_regs<E>(k, lane);
+#pragma unroll
+  for (int e = 0; e < E; e++)
+    if (lane * E + e < n) s[padded(first + lane * E + e)] = k[e];
+}
+
+__device__ __forceinline__ void sort_run(const unsigned long long *keys, unsigned *s, const WordForm &f, bool bnd,
+                                         int first, int n, int pos_bits) {
+  if (n <= 32) warp_sort_run<1>(keys, s, f, bnd, first, n, pos_bits);
+  else if (n <= 64) warp_sort_run<2>(keys, s, f, bnd, first, n, pos_bits);
+  else if (n <= 128) warp_sort_run<4>(keys, s, f, bnd, first, n, pos_bits);
+  else if (n <= 256) warp_sort_run<8>(keys, s, f, bnd, first, n, pos_bits);
+  else warp_sort_run<16>(keys, s, f, bnd, first, n, pos_bits);
+}
+
+// Outputs [d0, d1) of the merge of the sorted runs s[a, a + na) and s[b, b + nb)
+// (distinct words) into out from position o on: the split of the first output
+// by binary search along its diagonal (merge path, Green et al. 2012), then
+// one word at a time.
+__device__ __forceinline__ void merge_part(const unsigned *s, int a, int na, int b, int nb, unsigned *out, int o, int d0,
+                                           int d1) {
+  if (d0 >= d1) return;
+  int lo = max(0, d0 - nb), hi = min(d0, na);
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (s[padded(a + mid)] < s[padded(b + d0 - 1 - mid)]) lo = mid + 1;
+    else hi = mid;
+  }
+  int i = a + lo, j = b + d0 - lo;
+  const int ie = a + na, je = b + nb;
+  unsigned x = i < ie ? s[padded(i)] : 0xffffffffu, y = j < je ? s[padded(j)] : 0xffffffffu;
+  for (int d = d0; d < d1; d++) {
+    const bool second = j < je && (i >= ie || y < x);
+    out[padded(o + d)] = second ? y : x;
+    const int next = second ? ++j : ++i;
+    const unsigned v = next < (second ? je : ie) ? s[padded(next)] : 0xffffffffu;
+    if (second) y = v;
+    else x = v;
+  }
+}
+
+// The words of keys[0, n), n <= kWarpSortCap, positions from `first` on, sorted by one warp; the result
+// is in s or t (returned), padded positions from `first` on.
+__device__ __forceinline__ unsigned *warp_sort_words(const unsigned long long *keys, unsigned *s, unsigned *t,
+                                                     const WordForm &f, bool bnd, int first, int n, int pos_bits) {
+  const int n0 = min(n, kRunCap), n1 = n - n0;
+  sort_run(keys, s, f, bnd, first, n0, pos_bits);
+  if (n1 > 0) sort_run(keys + n0, s, f, bnd, first + n0, n1, pos_bits);
+  __syncwarp();
+  if (n1 <= 0) return s;
+  const int lane = threadIdx.x & 31, part = (n + 31) >> 5;
+  merge_part(s, first, n0, first + n0, n1, t, first, min(lane * part, n), min(lane * part + part, n));
+  __syncwarp();
+  return t;
+}
+
+// position bits of a segment of n keys: one more position than keys for the padding word
+__device__ __forceinline__ int position_bits(int n) { return max(5, 32 - __clz(n)); }
+
+// A segment of n <= kWarpSortCap keys, sorted by one warp. False: it needs all key bits.
+__device__ __forceinline__ bool warp_sort_segment(const Work &w, const unsigned long long *keys, unsigned *sk, bool bnd,
+                                                  long long s0, int n, int lane) {
+  const int pos_bits = position_bits(n);
+  const WordForm f = word_form(key_range(keys, n, lane, 32), bnd, pos_bits);
+  if (!f.ok) return false;
+  unsigned *s = warp_sort_words(keys, sk, sk + kWarpWords, f, bnd, 0, n, pos_bits);
+  if (!bnd) {
+    int pass = 0;
+    while (__any_sync(0xffffffffu, exchange_ties(keys, s, n, pos_bits, lane, 32, [] { __syncwarp(); })))
+      if (++pass == kFixPasses) return false;
+  }
+  for (int i = lane; i < n; i += 32) store_sorted(w, bnd, s0 + i, word_key(f, bnd, keys, s[padded(i)], pos_bits));
+  __syncwarp();
+  return true;
+}
+
+// Warps take groups of `grab` segments from a queue (tiles' Gaussian lists,
+// then boundary lists), the lanes reading their bounds together, and sort the
+// ones of up to kWarpSortCap keys: up to two runs in registers, a power-of-two
+// number of words per lane, and a merge; longer ones, and those that need all
+// key bits, are listed for k_tile_sort_big. Bound: instruction fetch and issue.
+// One warp's radix sort of a segment in shared memory (four or five passes,
+// each ranking 32 keys per round by a match) took 118 us on one 800^2 view
+// and 0.77 ms on 64 mixed views (30 M keys); this network on 64-bit keys 25 us
+// and 1.05 ms (its code did not stay in the instruction cache), on 32-bit
+// words with up to 32 per lane 21 us and 0.58 ms, with the runs of 16 per lane
+// and the merge 20 us and 0.48 ms.
+__global__ void __launch_bounds__(kSortThreads, 6) k_tile_sort(Params p, Work w, int *big_list, int grab) {
+  __shared__ unsigned s_sort[2 * kSortWarps * kWarpWords];
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   const bool g_over = w.g_tstart[p.tiles] > p.max_pairs, b_over = w.b_tstart[p.tiles] > p.max_bpairs;
   const int items = 2 * p.tiles;
-  unsigned long long *sk = s_sort + wp * kWarpSortCap;
-  unsigned *bins = reinterpret_cast<unsigned *>(s_sort + (kSortThreads / 32) * kWarpSortCap) + wp * 256;
+  unsigned *sk = s_sort + 2 * wp * kWarpWords;
   for (;;) {
-    int item = 0;
-    if (lane == 0) item = atomicAdd(w.counters + kQueueSort, 1);
-    item = __shfl_sync(0xffffffffu, item, 0);
-    if (item >= items) break;
-    bool bnd;
-    long long s0, s1;
-    segment_bounds(p, w, item, bnd, s0, s1);
-    if (bnd ? b_over : g_over) continue;  // unwritten slots: nothing to sort
-    const int n = (int)(s1 - s0);
-    unsigned long long *keys = (bnd ? w.bkeys : w.gkeys) + s0;
-    if (n > kWarpSortCap) {  // listed for k_tile_sort_mid (from the top of the list) or k_tile_sort_big
-      if (lane == 0) {
-        if (n <= kMidSortCap) big_list[2 * p.tiles + 1 - atomicAdd(w.counters + kMidCount, 1)] = item;
-        else big_list[atomicAdd(w.counters + kQueueSort + 1, 1)] = item;
-      }
-      continue;
+    int base = 0;
+    if (lane == 0) base = atomicAdd(w.counters + kQueueSort, grab);
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (base >= items) break;
+    bool bnd = false;
+    long long s0 = 0, s1 = 0;
+    const int item = base + lane;
+    if (lane < grab && item < items) {
+      segment_bounds(p, w, item, bnd, s0, s1);
+      if (bnd ? b_over : g_over) s1 = s0;  // unwritten slots: nothing to sort
     }
-    if (n > 1 && n <= 32) {
-      unsigned long long key = lane < n ? keys[lane] : ~0ull;
-      for (int k = 2; k <= 32; k <<= 1)
-        for (int j = k >> 1; j > 0; j >>= 1) {
-          const unsigned long long other = __shfl_xor_sync(0xffffffffu, key, j);
-          const bool up = (lane & k) == 0;
-          const bool lower = (lane & j) == 0;
-          key = (lower == up) ? (key < other ? key : other) : (key < other ? other : key);
-        }
-      if (lane < n) keys[lane] = key;
-    } else if (n > 32) {
-      int N = 64;
-      while (N < n) N <<= 1;
-      for (int i = lane; i < N; i += 32) sk[i] = i < n ? keys[i] : ~0ull;
+    const int n_lane = (int)(s1 - s0);
+    if (n_lane > kWarpSortCap) big_list[atomicAdd(w.counters + kBigCount, 1)] = item;
+    unsigned todo = __ballot_sync(0xffffffffu, n_lane > 0 && n_lane <= kWarpSortCap);
+    while (todo) {
+      const int l = __ffs(todo) - 1;
+      todo &= todo - 1;
+      const int n = __shfl_sync(0xffffffffu, n_lane, l);
+      const long long at = __shfl_sync(0xffffffffu, s0, l);
+      const bool b = __shfl_sync(0xffffffffu, (int)bnd, l);
+      const unsigned long long *keys = (b ? w.bkeys + p.max_bpairs : w.gkeys + p.max_pairs) + at;
+      const bool ok = warp_sort_segment(w, keys, sk, b, at, n, lane);
+      if (!ok && lane == 0) big_list[atomicAdd(w.counters + kBigCount, 1)] = (base + l) | kFullKeys;
       __syncwarp();
-      if (n < kRadixMin) warp_bitonic_smem(sk, N, lane);
-      else warp_sort_segment<kWarpSortCap / 32>(sk, bins, n, N, bnd, lane);
-      for (int i = lane; i < n; i += 32) keys[i] = sk[i];
-      __syncwarp();
-    }
-    if (bnd) {
-      __syncwarp();
-      gather_boundary(w, s0, s1, lane, 32);
     }
   }
 }
 
-// Segments of kWarpSortCap + 1 .. kMidSortCap keys (listed from the top of
-// big_list): one warp each, as in k_tile_sort with 32 keys per lane.
-__global__ void __launch_bounds__(kSortThreads, 2) k_tile_sort_mid(Params p, Work w, const int *big_list) {
-  extern __shared__ __align__(16) unsigned long long s_mid[];
+// keys of s[base, base + len) below `key` (with ties: not above it), len a power of two
+template <class Key>
+__device__ __forceinline__ int rank_in_run(const Key *s, int base, int len, Key key, bool ties) {
+  int pos = 0;
+  for (int step = len >> 1; step > 0; step >>= 1) {
+    const Key v = s[padded(base + pos + step - 1)];
+    if (ties ? v <= key : v < key) pos += step;
+  }
+  const Key v = s[padded(base + pos)];
+  return pos + (int)(ties ? v <= key : v < key);
+}
+
+// 32 E keys of every warp of the block, in registers as loaded, sorted over
+// the block into s (padded positions): each warp sorts its own in registers,
+// then two merges (runs 0-1 and 2-3, then the two halves) in which each key,
+// kept in its register, finds its rank in the other run by binary search and
+// moves there. Equal keys (the padding) take the lower run's first, so that
+// every position is written. Ends behind a block barrier.
+template <int E, class Key>
+__device__ __forceinline__ void block_sort(Key (&k)[E], Key *s) {
+  constexpr int L = 32 * E;
+  static_assert(kSortWarps == 4, "two merge levels");
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  unsigned long long *sk = s_mid + wp * kMidSortCap;
-  unsigned *bins = reinterpret_cast<unsigned *>(s_mid + (kSortThreads / 32) * kMidSortCap) + wp * 256;
-  const int nmid = w.counters[kMidCount];
-  for (int it = blockIdx.x * (kSortThreads / 32) + wp; it < nmid; it += gridDim.x * (kSortThreads / 32)) {
-    bool bnd;
-    long long s0, s1;
-    segment_bounds(p, w, big_list[2 * p.tiles + 1 - it], bnd, s0, s1);
-    const int n = (int)(s1 - s0);
-    unsigned long long *keys = (bnd ? w.bkeys : w.gkeys) + s0;
-    int N = 64;
-    while (N < n) N <<= 1;
-    for (int i = lane; i < N; i += 32) sk[i] = i < n ? keys[i] : ~0ull;
-    __syncwarp();
-    warp_sort_segment<kMidSortCap / 32>(sk, bins, n, N, bnd, lane);
-    for (int i = lane; i < n; i += 32) keys[i] = sk[i];
-    __syncwarp();
-    if (bnd) gather_boundary(w, s0, s1, lane, 32);
+  warp_sort_regs<E>(k, lane);
+  int pos[E];
+#pragma unroll
+  for (int e = 0; e < E; e++) {
+    pos[e] = lane * E + e;
+    s[padded(wp * L + pos[e])] = k[e];
   }
+  for (int level = 0; level < 2; level++) {
+    const int len = L << level, run = wp >> level;
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < E; e++) pos[e] += rank_in_run(s, (run ^ 1) * len, len, k[e], run & 1);
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < E; e++) s[padded((run >> 1) * 2 * len + pos[e])] = k[e];
+  }
+  __syncthreads();
 }
 
-// Segments longer than kMidSortCap: one block each (bitonic in shared memory
-// up to kSortCap keys, stable radix sort in global memory beyond; a block
-// radix sort in shared memory measured slower on dense tiles).
-__global__ void __launch_bounds__(kSortThreads) k_tile_sort_big(Params p, Work w, const int *big_list,
-                                                               unsigned long long *gtmp, unsigned long long *btmp) {
-  __shared__ unsigned long long s_keys[kSortCap];
-  __shared__ int s_hist[256], s_base[256];
-  __shared__ int s_wcnt[(kSortThreads / 32) * 256];
-  __shared__ unsigned long long s_red[2 * (kSortThreads / 32)];
-  const int nbig = w.counters[kQueueSort + 1];
+// a segment of n <= 128 E keys on all key bits
+template <int E>
+__device__ __forceinline__ void block_sort_full(const Work &w, const unsigned long long *keys, unsigned long long *s,
+                                                bool bnd, long long s0, int n) {
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  unsigned long long k[E];
+#pragma unroll
+  for (int e = 0; e < E; e++) {
+    const int i = wp * 32 * E + e * 32 + lane;
+    k[e] = i < n ? keys[i] : ~0ull;
+  }
+  block_sort<E>(k, s);
+  for (int i = threadIdx.x; i < n; i += kSortThreads) store_sorted(w, bnd, s0 + i, s[padded(i)]);
+}
+
+// a segment of n <= kSortCap keys as 32-bit words: a quarter of them per warp,
+// then two merges by the block; false: it needs all key bits
+__device__ __forceinline__ bool block_sort_words(const Work &w, const unsigned long long *keys, unsigned *s,
+                                                 KeyRange *s_range, bool bnd, long long s0, int n) {
+  static_assert(kSortWarps == 4, "two merge levels");
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, pos_bits = position_bits(n);
+  KeyRange r = key_range(keys, n, threadIdx.x, kSortThreads);
+  if (lane == 0) s_range[wp] = r;
+  __syncthreads();
+  for (int q = 0; q < kSortWarps; q++) {
+    r.hi0 = min(r.hi0, s_range[q].hi0);
+    r.hi1 = max(r.hi1, s_range[q].hi1);
+    r.lo0 = min(r.lo0, s_range[q].lo0);
+    r.lo1 = max(r.lo1, s_range[q].lo1);
+  }
+  const WordForm f = word_form(r, bnd, pos_bits);
+  if (!f.ok) return false;
+  unsigned *t = s + kSortWarps * kWarpWords;
+  const int q = (n + kSortWarps - 1) / kSortWarps;  // <= kWarpSortCap, and all quarters on one side of kRunCap
+  const int c[5] = {0, min(q, n), min(2 * q, n), min(3 * q, n), n};
+  const int first = min(wp * q, n), mine = min(q, n - first);
+  // one or two runs per warp: which buffer holds the result is decided by q for all warps alike
+  sort_run(keys + first, s, f, bnd, first, min(mine, kRunCap), pos_bits);
+  if (q > kRunCap) {
+    const int n0 = min(mine, kRunCap), n1 = mine - n0, part = (mine + 31) >> 5;
+    if (n1 > 0) sort_run(keys + first + n0, s, f, bnd, first + n0, n1, pos_bits);
+    __syncwarp();
+    merge_part(s, first, n0, first + n0, n1, t, first, min(lane * part, mine), min(lane * part + part, mine));
+    unsigned *x = s; s = t; t = x;
+  }
+  __syncthreads();
+  {  // quarters 0-1 by the first half of the block, 2-3 by the second
+    const int h = wp >> 1, a = c[2 * h], b = c[2 * h + 1], e = c[2 * h + 2], part = (e - a + 63) >> 6;
+    const int d = ((int)threadIdx.x & 63) * part;
+    merge_part(s, a, b - a, b, e - b, t, a, min(d, e - a), min(d + part, e - a));
+  }
+  __syncthreads();
+  {
+    const int part = (n + kSortThreads - 1) / kSortThreads, d = (int)threadIdx.x * part;
+    merge_part(t, 0, c[2], c[2], n - c[2], s, 0, min(d, n), min(d + part, n));
+  }
+  __syncthreads();
+  if (!bnd) {
+    int pass = 0;
+    while (__syncthreads_or(exchange_ties(keys, s, n, pos_bits, threadIdx.x, kSortThreads, [] { __syncthreads(); })))
+      if (++pass == kFixPasses) return false;
+  }
+  for (int i = threadIdx.x; i < n; i += kSortThreads)
+    store_sorted(w, bnd, s0 + i, word_key(f, bnd, keys, s[padded(i)], pos_bits));
+  return true;
+}
+
+// Segments longer than kWarpSortCap and those that need all key bits: one
+// block each, in shared memory up to kSortCap keys, by a stable radix sort in
+// global memory beyond. On eight 1600 x 1200 views of the room (dense tiles)
+// a bitonic network of the block over 64-bit keys in shared memory took 1.62
+// ms, quarters sorted by the warps and merged on 32-bit words 0.78 ms.
+__global__ void __launch_bounds__(kSortThreads, 4) k_tile_sort_big(Params p, Work w, const int *big_list) {
+  extern __shared__ __align__(16) unsigned long long s_keys[];
+  __shared__ KeyRange s_range[kSortWarps];
+  const int nbig = w.counters[kBigCount];
   for (int b = blockIdx.x; b < nbig; b += gridDim.x) {
+    const int item = big_list[b];
+    const bool full = item & kFullKeys;
     bool bnd;
     long long s0, s1;
-    segment_bounds(p, w, big_list[b], bnd, s0, s1);
+    segment_bounds(p, w, item & ~kFullKeys, bnd, s0, s1);
     const int n = (int)(s1 - s0);
-    unsigned long long *keys = (bnd ? w.bkeys : w.gkeys) + s0;
-    unsigned long long *tmp = (bnd ? btmp : gtmp) + s0;
+    unsigned long long *keys = (bnd ? w.bkeys + p.max_bpairs : w.gkeys + p.max_pairs) + s0;
     if (n <= kSortCap) {
-      for (int i = threadIdx.x; i < n; i += kSortThreads) s_keys[i] = keys[i];
-      __syncthreads();
-      bitonic_smem(s_keys, n);
-      for (int i = threadIdx.x; i < n; i += kSortThreads) keys[i] = s_keys[i];
+      if (full || !block_sort_words(w, keys, reinterpret_cast<unsigned *>(s_keys), s_range, bnd, s0, n)) {
+        __syncthreads();
+        block_sort_full<kWarpSortCap / 32>(w, keys, s_keys, bnd, s0, n);
+      }
     } else {
-      radix_global(keys, tmp, n, s_hist, s_base, s_wcnt, s_red);
+      unsigned long long *s_red = s_keys;  // 2 per warp
+      int *s_hist = reinterpret_cast<int *>(s_keys + 2 * kSortWarps), *s_base = s_hist + 256;
+      unsigned long long *out = (bnd ? w.bkeys : w.gkeys) + s0;
+      radix_global(keys, out, n, s_hist, s_base, s_base + 256, s_red);
+      if (bnd)
+        for (int i = threadIdx.x; i < n; i += kSortThreads) store_sorted(w, true, s0 + i, out[i]);
     }
-    __syncthreads();
-    if (bnd) gather_boundary(w, s0, s1, threadIdx.x, kSortThreads);
     __syncthreads();
   }
 }
 
 }  // namespace
 
-int launch_exclusive_scan(const int *in, long long *out, int n, long long *aux, cudaStream_t st) {
-  // out[0..n) = exclusive prefix sums of in, out[n] = total
-  if (n <= 0) {
-    cudaMemsetAsync(out, 0, sizeof(long long), st);
-    return 0;
-  }
-  const int nb = (n + kScanChunk - 1) / kScanChunk;
-  k_scan_reduce<<<nb, kScanThreads, 0, st>>>(in, n, aux);
-  k_scan_top<<<1, kScanThreads, 0, st>>>(aux, nb);
-  k_scan_down<<<nb, kScanThreads, 0, st>>>(in, out, n, aux);
-  return 3;
+int launch_scan_pair(const int *in0, long long *out0, const int *in1, long long *out1, int n, cudaStream_t st) {
+  if (n <= kScanOne) k_scan_pair<1><<<1, kScanThreads, 0, st>>>(in0, out0, in1, out1, n);
+  else k_scan_pair<kScanCluster><<<kScanCluster, kScanThreads, 0, st>>>(in0, out0, in1, out1, n);
+  return 1;
 }
 
 cudaError_t configure_binning() {
-  cudaError_t e = cudaFuncSetAttribute(k_tile_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSortSmem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_tile_sort_mid, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSortMidSmem);
-  return e;
-}
-
-int launch_bin_sort_only(const Params &p, const Work &w, cudaStream_t st) {
-  k_emit<<<16 * 152, 256, 0, st>>>(p, w);
-  if (p.tiles <= 0) return 1;
-  cudaMemsetAsync(w.counters + kQueueSort, 0, 2 * sizeof(int), st);
-  cudaMemsetAsync(w.counters + kMidCount, 0, sizeof(int), st);
-  k_tile_sort<<<3 * 152, kSortThreads, kTileSortSmem, st>>>(p, w, w.big_list);
-  k_tile_sort_mid<<<2 * 152, kSortThreads, kTileSortMidSmem, st>>>(p, w, w.big_list);
-  k_tile_sort_big<<<4 * 152, kSortThreads, 0, st>>>(p, w, w.big_list, w.gkeys + p.max_pairs, w.bkeys + p.max_bpairs);
-  return 4;
+  return cudaFuncSetAttribute(k_tile_sort_big, cudaFuncAttributeMaxDynamicSharedMemorySize, kSortBigSmem);
 }
 
 int launch_binning(const Params &p, const Work &w, cudaStream_t st) {
-  int k = launch_exclusive_scan(w.g_tcount, w.g_tstart, p.tiles, w.scan_aux, st);
-  k += launch_exclusive_scan(w.b_tcount, w.b_tstart, p.tiles, w.scan_aux2, st);
-  k_check_capacity<<<1, 1, 0, st>>>(p, w);
-  k += 2;
-  if (p.tiles > 0) {
-    k_tile_desc<<<(p.tiles + 255) / 256, 256, 0, st>>>(p, w);
-    k++;
-  }
-  return k + launch_bin_sort_only(p, w, st);
+  if (p.tiles <= 0) return 0;
+  if (p.tiles <= kScanOne) k_tile_scan<1><<<1, kScanThreads, 0, st>>>(p, w);
+  else k_tile_scan<kScanCluster><<<kScanCluster, kScanThreads, 0, st>>>(p, w);
+  k_emit<<<16 * 152, 256, 0, st>>>(p, w);
+  // segments per dequeue: enough dequeues for every resident warp to take a few, so that long segments
+  // spread, and few enough that the queue's one counter is no bottleneck
+  const int blocks = 6 * 152, grab = std::max(1, std::min(32, 2 * p.tiles / (blocks * kSortWarps * 4)));
+  k_tile_sort<<<blocks, kSortThreads, 0, st>>>(p, w, w.big_list, grab);
+  k_tile_sort_big<<<4 * 152, kSortThreads, kSortBigSmem, st>>>(p, w, w.big_list);
+  return 4;
 }
 
 }  // namespace bgt

@@ -703,8 +703,7 @@ int launch_chain(const Params &p, const Scene &s, const Work &w, const Grads &g,
     cudaMemsetAsync(w.prim_gcnt, 0, sizeof(int) * (size_t)p.M, st);
     cudaMemsetAsync(w.prim_bcnt, 0, sizeof(int) * (size_t)p.M, st);
     k_prim_count<<<(sms > 0 ? sms : 152) * 8, 256, 0, st>>>(w);
-    k += 1 + launch_exclusive_scan(w.prim_gcnt, w.prim_gseg, p.M, w.scan_aux, st);
-    k += launch_exclusive_scan(w.prim_bcnt, w.prim_bseg, p.M, w.scan_aux2, st);
+    k += 1 + launch_scan_pair(w.prim_gcnt, w.prim_gseg, w.prim_bcnt, w.prim_bseg, p.M, st);
     cudaMemsetAsync(w.prim_gcnt, 0, sizeof(int) * (size_t)p.M, st);  // now the fill counters
     cudaMemsetAsync(w.prim_bcnt, 0, sizeof(int) * (size_t)p.M, st);
     if (with_cov) cudaMemsetAsync(w.prim_gcov, 0, sizeof(float) * 6 * (size_t)p.M, st);

@@ -101,6 +101,8 @@ __global__ void __launch_bounds__(kGenThreads) k_ids(Params p, Scene s, Work w, 
   for (int t = gtid; t < p.tiles; t += gthreads) {
     w.g_tcount[t] = 0;
     w.b_tcount[t] = 0;
+    w.g_tfill[t] = 0;
+    w.b_tfill[t] = 0;
   }
   if (gtid >= kQueueFwd && gtid < kIdsDone) w.counters[gtid] = 0;
   if (p.attr_res == 1)

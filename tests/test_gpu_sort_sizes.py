@@ -1,0 +1,47 @@
+"""The per-tile sort at the sizes where it changes form (runs of 32, 64, 128, 256 and 512 words per
+warp, two merged runs, the block's quarters, the radix sort beyond 4096 keys) and on depths that need
+each of its forms: spread depths, ties, depths closer than the words resolve, all equal (the index
+decides), and a range too wide for 32-bit words. Keys are integers: the list has to hold every Gaussian
+once, in ascending key order."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+SIZES = [1, 2, 31, 32, 33, 64, 65, 128, 129, 256, 257, 511, 512, 513, 700, 1023, 1024, 1025, 1500, 2047, 2048, 2049,
+         3000, 4095, 4096, 4097, 5000]
+
+
+def _depths(kind, n, rng):
+    if kind == "spread":
+        return rng.uniform(0.3, 60.0, n)
+    if kind == "ties":
+        return rng.choice(rng.uniform(2.0, 6.0, max(1, n // 3)), n)
+    if kind == "close":  # neighbouring floats, and one far away that takes the words' upper bits
+        d = np.float32(3.0) + np.arange(n, dtype=np.float32) * np.float32(2.4e-7)
+        d = rng.permutation(d)
+        d[0] = 900.0
+        return d
+    if kind == "equal":
+        return np.full(n, 4.25)
+    return 10.0 ** rng.uniform(-20, 20, n)  # "wide"
+
+
+@pytest.mark.parametrize("kind", ["spread", "ties", "close", "equal", "wide"])
+def test_one_tile_lists_of_every_size(scenes, kind):
+    from paper_2503_13961_gb300 import render as R
+    cap = max(SIZES)
+    rd = R.Renderer(degree=2, max_prims=1, max_views=1, max_pixels=cap, max_pairs=4 * cap, max_boundary_pairs=1024,
+                    tile_size=32)
+    for n in SIZES:
+        rng = np.random.default_rng(n)
+        g = scenes.random_gaussians(n, 32, 32, n)
+        g["depth"] = np.ascontiguousarray(_depths(kind, n, rng), np.float32)
+        out = rd.bin_sort(g, 32, 32)
+        rd.sync_status()
+        keys = out["keys"]
+        assert out["ranges"].tolist() == [0, n] and len(keys) == n, n
+        want = np.sort((((g["depth"].view(np.uint32).astype(np.uint64) << np.uint64(5)) | np.uint64(16))
+                        << np.uint64(27)) | np.arange(n, dtype=np.uint64))
+        assert np.array_equal(keys, want), (kind, n)
+    rd.close()
