@@ -290,18 +290,9 @@ cudaError_t enqueue_fwd(bgt_handle *h, const bgt::Params &p, const bgt::Scene &s
 cudaError_t enqueue_bwd(bgt_handle *h, const bgt::Params &p, const bgt::Scene &s, const float *dimg,
                         const bgt::Grads &g, cudaStream_t st) {
   const bgt::Work &w = h->w;
-  const size_t cp = sizeof(float) * (size_t)p.M * p.ncp * 3;
   mark(h, 7, st);
-  if (p.M > 0) {
-    cudaMemsetAsync(g.ctrl, 0, cp, st);
-    cudaMemsetAsync(g.color, 0, cp, st);
-    cudaMemsetAsync(g.opacity, 0, sizeof(float) * (size_t)p.M, st);
-    cudaMemsetAsync(g.r_b, 0, sizeof(float) * (size_t)p.M, st);
-    if (g.log_scale) cudaMemsetAsync(g.log_scale, 0, sizeof(float) * 3 * (size_t)p.M * p.ntex, st);
-    if (g.quat) cudaMemsetAsync(g.quat, 0, sizeof(float) * 4 * (size_t)p.M * p.ntex, st);
-    if (g.sh && p.sh_k > 0) cudaMemsetAsync(g.sh, 0, sizeof(float) * 3 * (size_t)p.M * p.sh_k, st);
-  }
-  int k = bgt::launch_composite_bwd(p, w, dimg, st);
+  int k = bgt::launch_clear_grads(p, w, g, st);
+  k += bgt::launch_composite_bwd(p, w, dimg, st);
   mark(h, 8, st);
   k += bgt::launch_chain(p, s, w, g, st);
   mark(h, 9, st);

@@ -733,6 +733,7 @@ cudaError_t configure_composite();  // opt the blending kernels into > 48 KB sha
 cudaError_t configure_binning();    // the same for the per-tile sort
 int launch_composite_fwd(const Params &p, const Work &w, float *image, cudaStream_t st);
 int launch_composite_bwd(const Params &p, const Work &w, const float *dimage, cudaStream_t st);
+int launch_clear_grads(const Params &p, const Work &w, const Grads &g, cudaStream_t st);
 int launch_chain(const Params &p, const Scene &s, const Work &w, const Grads &g, cudaStream_t st);
 void launch_scatter_uv(const Params &p, const Work &w, int F, cudaStream_t st);
 int launch_l1_grad(const float *img, const float *target, long long n, float scale, float *dimg,
@@ -749,7 +750,8 @@ int launch_edge_prior(const Params &p, const Work &w, const float *edges, float 
                       cudaStream_t st);
 int launch_visibility(const Params &p, const Work &w, const int *view_off, int *view_count,
                       unsigned long long *cell_mask, cudaStream_t st);
-// exclusive prefix sums (n + 1 values, the last the total) of two count arrays (16-byte aligned)
-int launch_scan_pair(const int *in0, long long *out0, const int *in1, long long *out1, int n, cudaStream_t st);
+// exclusive prefix sums (n + 1 values, the last the total) of two count arrays (16-byte aligned); clear:
+// the counts are zeroed behind their last use
+int launch_scan_pair(int *in0, long long *out0, int *in1, long long *out1, int n, bool clear, cudaStream_t st);
 
 }  // namespace bgt

@@ -143,8 +143,14 @@ __device__ inline longlong2 scan_both(const int *in0, long long *out0, const int
 
 template <int CL>
 __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(kScanThreads)
-    k_scan_pair(const int *in0, long long *out0, const int *in1, long long *out1, int n) {
+    k_scan_pair(int *in0, long long *out0, int *in1, long long *out1, int n, bool clear) {
   scan_both<CL>(in0, out0, in1, out1, n);
+  if (!clear) return;
+  // every count of the block's range was last read before its last block barrier, but for the final chunk's
+  __syncthreads();
+  const int chunks = (n + kScanChunk - 1) / kScanChunk, per = (chunks + CL - 1) / CL * kScanChunk;
+  const int lo = min((int)blockIdx.x * per, n), hi = min(lo + per, n);
+  for (int i = lo + (int)threadIdx.x; i < hi; i += kScanThreads) in0[i] = in1[i] = 0;
 }
 
 // Tile list starts (exclusive sums of the Gaussian and boundary counts) and the
@@ -784,9 +790,9 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_tile_sort_big(Params p, Wor
 
 }  // namespace
 
-int launch_scan_pair(const int *in0, long long *out0, const int *in1, long long *out1, int n, cudaStream_t st) {
-  if (n <= kScanOne) k_scan_pair<1><<<1, kScanThreads, 0, st>>>(in0, out0, in1, out1, n);
-  else k_scan_pair<kScanCluster><<<kScanCluster, kScanThreads, 0, st>>>(in0, out0, in1, out1, n);
+int launch_scan_pair(int *in0, long long *out0, int *in1, long long *out1, int n, bool clear, cudaStream_t st) {
+  if (n <= kScanOne) k_scan_pair<1><<<1, kScanThreads, 0, st>>>(in0, out0, in1, out1, n, clear);
+  else k_scan_pair<kScanCluster><<<kScanCluster, kScanThreads, 0, st>>>(in0, out0, in1, out1, n, clear);
   return 1;
 }
 

@@ -12,12 +12,13 @@
 // Two passes take these to the primitives: pass one (one thread per Gaussian,
 // one per boundary point) computes dl/dS_q and the other per-record
 // gradients and writes them, with the record's (u, v), into its primitive's
-// segment of a record array (segments from a count and a scan over the
-// primitives); pass two sums each primitive's records with their Bernstein
+// segment of a record array (segments from the counts that the blending
+// backward takes beside its work, and a scan over the primitives); pass two sums each primitive's records with their Bernstein
 // weights. A primitive covers a few pixels of a view, so records in pixel
 // order change primitive every two or so; grouped, a primitive's records of
 // all views are contiguous and its sums take a few atomics instead of one
 // per short run and value.
+#include <algorithm>
 #include <cstdint>
 
 #include "bgt_internal.cuh"
@@ -83,16 +84,13 @@ __device__ inline int stage_views(const Params &p, const Work &w, View *s_views)
   return nsv;
 }
 
+// the chain rule of the warp's Gaussian i (one per lane, below F)
 template <int N>
-__global__ void __launch_bounds__(256) k_chain_gauss(Params p, Scene s, Work w, Grads out) {
+__device__ __forceinline__ void chain_gauss(const Params &p, const Scene &s, const Work &w, const Grads &out,
+                                            const View *s_views, int nsv, int i, int F) {
   constexpr int m = SurfPoint<N>::M;
-  __shared__ View s_views[kStagedViews];
-  const int nsv = stage_views(p, w, s_views);
-  const int F = w.counters[kF];
   const int lane = threadIdx.x & 31;
-  const int warps_total = gridDim.x * (blockDim.x >> 5);
-  for (int base = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32; base < F; base += warps_total * 32) {
-    const int i = base + lane;
+  {
     bool active = i < F;
     int g = -1;
     float gS[3] = {0.f, 0.f, 0.f}, gcol[3] = {0.f, 0.f, 0.f}, gop = 0.f;
@@ -312,17 +310,13 @@ __global__ void __launch_bounds__(256) k_chain_sh(Params p, Scene s, Work w, Gra
   }
 }
 
+// the chain rule of the warp's boundary point i (one per lane, below Nb)
 template <int N>
-__global__ void __launch_bounds__(256) k_chain_bnd(Params p, Scene s, Work w, Grads out) {
+__device__ __forceinline__ void chain_bnd(const Params &p, const Scene &s, const Work &w, const View *s_views, int nsv,
+                                          int i, int Nb) {
   constexpr int m = SurfPoint<N>::M;
-  __shared__ View s_views[kStagedViews];
-  const int nsv = stage_views(p, w, s_views);
-  const int Nb = w.counters[kNb];
   const int lane = threadIdx.x & 31;
-  const int warps_total = gridDim.x * (blockDim.x >> 5);
-  for (int base = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32; base < Nb; base += warps_total * 32) {
-    const int i = base + lane;
-    if (i >= Nb) continue;
+  if (i < Nb) {
     const int g = w.b_prim[i];
     const float2 uv = w.b_uv[i];
     float gS[3] = {0.f, 0.f, 0.f}, grb = 0.f;
@@ -353,22 +347,77 @@ __global__ void __launch_bounds__(256) k_chain_bnd(Params p, Scene s, Work w, Gr
   }
 }
 
-// records per primitive: its Gaussians and its boundary points; the lanes of
-// a warp with the same primitive add their count with one atomic
-__global__ void k_prim_count(Work w) {
+// Pass one over the Gaussians, then the boundary points, 32 at a time per warp,
+// in one launch: the boundary points fill in where the Gaussians run out
+template <int N>
+__global__ void __launch_bounds__(256) k_chain(Params p, Scene s, Work w, Grads out) {
+  __shared__ View s_views[kStagedViews];
   const int F = w.counters[kF], Nb = w.counters[kNb];
+  const int ng = (F + 31) >> 5, groups = ng + ((Nb + 31) >> 5);
+  if ((int)(blockIdx.x * kChainWarps) >= groups) return;
+  const int nsv = stage_views(p, w, s_views);
   const int lane = threadIdx.x & 31;
-  const int stride = gridDim.x * blockDim.x;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < F + Nb; i += stride) {
-    const bool gs = i < F;
-    const int g = gs ? w.g_prim[i] : w.b_prim[i - F];
-    const unsigned peers = __match_any_sync(__activemask(), gs ? g : -1 - g);
-    if (lane == __ffs(peers) - 1) atomicAdd((gs ? w.prim_gcnt : w.prim_bcnt) + g, __popc(peers));
+  for (int q = blockIdx.x * kChainWarps + (threadIdx.x >> 5); q < groups; q += gridDim.x * kChainWarps) {
+    if (q < ng) chain_gauss<N>(p, s, w, out, s_views, nsv, q * 32 + lane, F);
+    else chain_bnd<N>(p, s, w, s_views, nsv, (q - ng) * 32 + lane, Nb);
   }
 }
 
+// n floats from p on cleared by the whole grid, 16 bytes at a time where p allows
+__device__ __forceinline__ void clear_floats(float *p, long long n) {
+  if (!p) return;
+  const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
+  const long long head = min(n, (long long)((16 - (reinterpret_cast<uintptr_t>(p) & 15)) & 15) / 4);
+  const long long n4 = (n - head) >> 2;
+  float4 *p4 = reinterpret_cast<float4 *>(p + head);
+  for (long long i = t0; i < n4; i += stride) p4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  const long long tail = head + 4 * n4;
+  if (t0 < head) p[t0] = 0.f;
+  if (tail + t0 < n) p[tail + t0] = 0.f;
+}
+
+// Everything the backward pass adds into, cleared in one launch: the gradient
+// arrays, the per-primitive record counters and dl/dSigma3D, the queue heads
+// (nine or more memsets, 2-3 us each in the serial chain of a small call). With maps
+// of leg resolution 1 the map gradients are written whole at the end.
+__global__ void __launch_bounds__(256) k_clear_grads(Params p, Work w, Grads g) {
+  const long long M = p.M;
+  clear_floats(g.ctrl, M * p.ncp * 3);
+  clear_floats(g.color, M * p.ncp * 3);
+  clear_floats(g.opacity, M);
+  clear_floats(g.r_b, M);
+  if (p.attr_res != 1) {
+    clear_floats(g.log_scale, 3 * M * p.ntex);
+    clear_floats(g.quat, 4 * M * p.ntex);
+  } else if (g.log_scale || g.quat) {
+    clear_floats(w.prim_gcov, 6 * M);
+  }
+  if (p.sh_k > 0) clear_floats(g.sh, 3 * M * p.sh_k);
+  clear_floats(reinterpret_cast<float *>(w.prim_gcnt), M);
+  clear_floats(reinterpret_cast<float *>(w.prim_bcnt), M);
+  if (blockIdx.x == 0 && threadIdx.x == 0) w.counters[kQueueBwd] = w.counters[kQueueWalk] = 0;
+}
+
 constexpr int kSumCols = 15;   // staged row: dl/dS (3), dl/do, dl/dc (3), dl/dSigma3D (6), dl/dr_b, primitive
-constexpr int kSumChunk = 256; // records per work item of the per-primitive sums
+constexpr int kSumChunk = 256; // most records per work item of the per-primitive sums
+
+// Work items of the per-primitive sums: chunks of the Gaussian records, then
+// of the boundary records; their length so that every warp of the grid gets
+// one (a primitive's sum is a chain of dependent steps: on one 800^2 view,
+// 310,000 records, chunks of 256 left half of the warps idle and took 63 us), a
+// multiple of the 32 records of a round.
+struct SumChunks {
+  int len, ng, count;
+};
+
+__device__ __forceinline__ SumChunks sum_chunks(int F, int Nb) {
+  SumChunks c;
+  const int warps = gridDim.x * (blockDim.x >> 5);
+  c.len = min(kSumChunk, ((F + Nb) / warps + 32) & ~31);
+  c.ng = (F + c.len - 1) / c.len;
+  c.count = c.ng + (Nb + c.len - 1) / c.len;
+  return c;
+}
 
 // Per-primitive sums of the records, which pass one left grouped by primitive:
 // dl/dp_a = sum_q B_a(u_q, v_q) dl/dS_q over the primitive's Gaussians and
@@ -380,7 +429,7 @@ constexpr int kSumChunk = 256; // records per work item of the per-primitive sum
 // Sigma3D) and sums them along the run of the current primitive, adding the
 // run's sum with one atomic when the primitive changes and at the chunk's end.
 template <int N>
-__global__ void __launch_bounds__(256) k_prim_sum(Params p, Work w, Grads out, int with_cov) {
+__global__ void __launch_bounds__(256, 3) k_prim_sum_rows(Work w, Grads out, int with_cov) {
   constexpr int m = SurfPoint<N>::M;
   constexpr int RS = (kSumCols + m) | 1;  // row stride (odd: conflict-free row writes)
   constexpr int NO = 6 * m + 8;           // outputs
@@ -423,12 +472,12 @@ __global__ void __launch_bounds__(256) k_prim_sum(Params p, Work w, Grads out, i
       atomicAdd(dst, acc[q]);
     }
   };
-  const long long ng = (F + kSumChunk - 1) / kSumChunk, nchunks = ng + (Nb + kSumChunk - 1) / kSumChunk;
+  const SumChunks sc = sum_chunks(F, Nb);
   const int warps_total = gridDim.x * (blockDim.x >> 5);
-  for (long long ck = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); ck < nchunks; ck += warps_total) {
-    const bool bnd = ck >= ng;
-    const long long r0 = (bnd ? ck - ng : ck) * kSumChunk;
-    const long long r1 = min(r0 + kSumChunk, (long long)(bnd ? Nb : F));
+  for (int ck = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); ck < sc.count; ck += warps_total) {
+    const bool bnd = ck >= sc.ng;
+    const long long r0 = (long long)(bnd ? ck - sc.ng : ck) * sc.len;
+    const long long r1 = min(r0 + sc.len, (long long)(bnd ? Nb : F));
     float acc[NQ];
 #pragma unroll
     for (int q = 0; q < NQ; q++) acc[q] = 0.f;
@@ -519,16 +568,17 @@ __global__ void __launch_bounds__(256) k_prim_sum(Params p, Work w, Grads out, i
   }
 }
 
-// The per-primitive sums of k_prim_sum for degrees whose outputs fit in
+// The per-primitive sums of k_prim_sum_rows for degrees whose outputs fit in
 // registers (6m + 8 <= 44 at degree 2): lane i owns record slot i of each
 // round of 32 and adds its record's weighted values to its own 6m + 8
 // accumulators over the rounds of a run of equal primitive; when the
 // primitive changes (and at the chunk's end) a reduce-scatter over the warp
 // (shuffle butterfly, 62 exchanges) leaves outputs 2i and 2i + 1 in lane i,
-// which adds them with one atomic each. Same sums as k_prim_sum, with a
-// shuffle exchange per run instead of a shared-memory pass per round.
+// which adds them with one atomic each. Same sums as k_prim_sum_rows, with a
+// shuffle exchange per run (~330 instructions) instead of a shared-memory pass
+// per round (~8 instructions per record).
 template <int N>
-__global__ void __launch_bounds__(256, 2) k_prim_sum_reg(Params p, Work w, Grads out) {
+__global__ void __launch_bounds__(256, 2) k_prim_sum_regs(Work w, Grads out) {
   constexpr int m = SurfPoint<N>::M;
   constexpr int NO = 6 * m + 8;
   static_assert(NO <= 64, "outputs beyond two per lane");
@@ -561,12 +611,12 @@ __global__ void __launch_bounds__(256, 2) k_prim_sum_reg(Params p, Work w, Grads
 #pragma unroll
     for (int i = 0; i < 64; i++) acc[i] = 0.f;
   };
-  const long long ng = (F + kSumChunk - 1) / kSumChunk, nchunks = ng + (Nb + kSumChunk - 1) / kSumChunk;
+  const SumChunks sc = sum_chunks(F, Nb);
   const int warps_total = gridDim.x * (blockDim.x >> 5);
-  for (long long ck = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); ck < nchunks; ck += warps_total) {
-    const bool bnd = ck >= ng;
-    const long long r0 = (bnd ? ck - ng : ck) * kSumChunk;
-    const long long r1 = min(r0 + kSumChunk, (long long)(bnd ? Nb : F));
+  for (int ck = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); ck < sc.count; ck += warps_total) {
+    const bool bnd = ck >= sc.ng;
+    const long long r0 = (long long)(bnd ? ck - sc.ng : ck) * sc.len;
+    const long long r1 = min(r0 + sc.len, (long long)(bnd ? Nb : F));
 #pragma unroll
     for (int i = 0; i < 64; i++) acc[i] = 0.f;
     int gcur = -1;
@@ -691,36 +741,44 @@ __global__ void k_prim_attr_grad(Params p, Scene s, Work w, Grads out) {
     for (int k = 0; k < 4; k++) out.quat[4 * (size_t)m + k] = gq[k];
 }
 
+// The form of the per-primitive sums at degrees 1 and 2: k_prim_sum_regs pays
+// per run of records of one primitive, k_prim_sum_rows per record. How many
+// records a primitive has is known on the device only; about 0.4 (an object) to
+// 1.1 (a room) per pixel are Gaussians and boundary points. 20,000 primitives:
+// 32 pixels per primitive 29 against 47 us (rows against registers), 52 46
+// against 70, 302 107 against 91, 1,600 337 against 184.
+constexpr long long kSumRegsFrom = 160;  // pixels per primitive
+
+int launch_clear_grads(const Params &p, const Work &w, const Grads &g, cudaStream_t st) {
+  const long long most = std::max(1ll, (long long)p.M * (3 * p.ncp + 3 * p.sh_k));  // floats, about
+  k_clear_grads<<<(int)std::min(most / 1024 + 1, 152ll * 8), 256, 0, st>>>(p, w, g);
+  return 1;
+}
+
 int launch_chain(const Params &p, const Scene &s, const Work &w, const Grads &g, cudaStream_t st) {
   int sms = 0, dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int grid = (sms > 0 ? sms : 152) * p.chain_bps;
+  if (sms <= 0) sms = 152;
+  const int grid = sms * p.chain_bps;
   int k = 0;
   const int with_cov = p.attr_res == 1 && (g.log_scale || g.quat);
-  if (p.M > 0) {
-    // segments of the per-primitive records
-    cudaMemsetAsync(w.prim_gcnt, 0, sizeof(int) * (size_t)p.M, st);
-    cudaMemsetAsync(w.prim_bcnt, 0, sizeof(int) * (size_t)p.M, st);
-    k_prim_count<<<(sms > 0 ? sms : 152) * 8, 256, 0, st>>>(w);
-    k += 1 + launch_scan_pair(w.prim_gcnt, w.prim_gseg, w.prim_bcnt, w.prim_bseg, p.M, st);
-    cudaMemsetAsync(w.prim_gcnt, 0, sizeof(int) * (size_t)p.M, st);  // now the fill counters
-    cudaMemsetAsync(w.prim_bcnt, 0, sizeof(int) * (size_t)p.M, st);
-    if (with_cov) cudaMemsetAsync(w.prim_gcov, 0, sizeof(float) * 6 * (size_t)p.M, st);
-  }
+  if (p.M == 0) return 0;
+  // segments of the per-primitive records from their counts (taken by the blending backward)
+  k += launch_scan_pair(w.prim_gcnt, w.prim_gseg, w.prim_bcnt, w.prim_bseg, p.M, true, st);
   dispatch_degree(p.n, [&](auto d) {
-    k_chain_gauss<decltype(d)::value><<<grid, 256, 0, st>>>(p, s, w, g);
-    k_chain_bnd<decltype(d)::value><<<grid, 256, 0, st>>>(p, s, w, g);
-    if (p.M > 0) {
-      if constexpr (SurfPoint<decltype(d)::value>::M <= 6)
-        k_prim_sum_reg<decltype(d)::value><<<(sms > 0 ? sms : 152) * 2, 256, 0, st>>>(p, w, g);
-      else
-        k_prim_sum<decltype(d)::value><<<(sms > 0 ? sms : 152) * 4, 256, 0, st>>>(p, w, g, with_cov);
+    constexpr int N = decltype(d)::value;
+    k_chain<N><<<grid, 256, 0, st>>>(p, s, w, g);
+    bool regs = false;
+    if constexpr (SurfPoint<N>::M <= 6) {
+      regs = p.P > kSumRegsFrom * (long long)p.M;
+      if (regs) k_prim_sum_regs<N><<<sms * 2, 256, 0, st>>>(w, g);
     }
-    if (p.sh_deg > 0) k_chain_sh<decltype(d)::value><<<grid, 256, 0, st>>>(p, s, w, g);
+    if (!regs) k_prim_sum_rows<N><<<sms * 4, 256, 0, st>>>(w, g, with_cov);
+    if (p.sh_deg > 0) k_chain_sh<N><<<grid, 256, 0, st>>>(p, s, w, g);
   });
-  k += (p.sh_deg > 0 ? 3 : 2) + (p.M > 0 ? 1 : 0);
-  if (p.attr_res == 1 && (g.log_scale || g.quat) && p.M > 0) {
+  k += p.sh_deg > 0 ? 3 : 2;
+  if (with_cov) {
     k_prim_attr_grad<<<(p.M + 255) / 256, 256, 0, st>>>(p, s, w, g);
     k++;
   }

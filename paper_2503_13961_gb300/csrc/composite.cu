@@ -870,6 +870,31 @@ __global__ void __launch_bounds__(TileCfg<T>::NT, TileCfg<T>::MINB_BWD) k_compos
   }
 }
 
+// Records per primitive of the chain rule's grouping, its Gaussians and its
+// boundary points, counted by the whole grid of the tile-list walk, which
+// mostly has no block to walk (a launch less; counted by the record replay's grid, whose
+// later blocks start only behind its first ones, it cost the replay 6 %);
+// the lanes of a warp with the same primitive add their count with one atomic.
+__device__ __forceinline__ void count_prim_records(const Work &w) {
+  const int F = w.counters[kF], n = F + w.counters[kNb];
+  const int lane = threadIdx.x & 31;
+  const int stride = gridDim.x * blockDim.x;
+  for (int i0 = blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += 4 * stride) {
+    int g[4];  // four loads in flight: the kernel's few warps leave their latency bare
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      const long long i = i0 + (long long)q * stride;
+      g[q] = i < F ? w.g_prim[i] : i < n ? -1 - w.b_prim[i - F] : 0x7fffffff;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      if (g[q] == 0x7fffffff) break;
+      const unsigned peers = __match_any_sync(__activemask(), g[q]);
+      if (lane == __ffs(peers) - 1) atomicAdd(g[q] >= 0 ? w.prim_gcnt + g[q] : w.prim_bcnt + (-1 - g[q]), __popc(peers));
+    }
+  }
+}
+
 // Backward pass of the warp blocks whose blend records did not fit (listed
 // by the forward pass): each warp re-walks its block's tile list back to
 // front from the last composited entry of its pixels. Every decision of the
@@ -894,6 +919,7 @@ __global__ void __launch_bounds__(TileCfg<T>::NT) k_composite_bwd_walk(Params p,
   __shared__ int s_wb[NW][kWalkSlots][PPT][32];    // its most influential boundary candidate
   float4 *sP = s_P[warp], *sQ = s_Q[warp], *sC = s_C[warp];
   int *sG = s_G[warp];
+  count_prim_records(w);
   const int nwalk = w.counters[kWalkCount];
   for (;;) {
     int q = 0;
@@ -1038,8 +1064,7 @@ int launch_bwd_t(const Params &p, const Work &w, const float *dimage, cudaStream
   if (grid > 0) {
     if (p.stats) k_composite_bwd<T, true><<<grid, TileCfg<T>::NT, sizeof(BwdShared<T>), st>>>(p, w, dimage);
     else k_composite_bwd<T, false><<<grid, TileCfg<T>::NT, sizeof(BwdShared<T>), st>>>(p, w, dimage);
-    // warp blocks whose records overflowed (none in the common case: the
-    // kernel reads the count and returns)
+    // the records per primitive, and the warp blocks whose blend records overflowed (none in the common case)
     k_composite_bwd_walk<T><<<sms * 3, TileCfg<T>::NT, 0, st>>>(p, w, dimage);  // 3 blocks per SM by registers
   }
   return grid > 0 ? 2 : 0;
@@ -1082,7 +1107,6 @@ cudaError_t configure_composite() {
 }
 
 int launch_composite_fwd(const Params &p, const Work &w, float *image, cudaStream_t st) {
-  cudaMemsetAsync(w.counters + kQueueFwd, 0, sizeof(int), st);
   const int sms = num_sms();
   if (p.tile == 8) return launch_fwd_t<8>(p, w, image, st, sms);
   if (p.tile == 32) return launch_fwd_t<32>(p, w, image, st, sms);
@@ -1090,8 +1114,6 @@ int launch_composite_fwd(const Params &p, const Work &w, float *image, cudaStrea
 }
 
 int launch_composite_bwd(const Params &p, const Work &w, const float *dimage, cudaStream_t st) {
-  cudaMemsetAsync(w.counters + kQueueBwd, 0, sizeof(int), st);
-  cudaMemsetAsync(w.counters + kQueueWalk, 0, sizeof(int), st);
   const int sms = num_sms();
   if (p.tile == 8) return launch_bwd_t<8>(p, w, dimage, st, sms);
   if (p.tile == 32) return launch_bwd_t<32>(p, w, dimage, st, sms);
