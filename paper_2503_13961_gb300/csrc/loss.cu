@@ -8,17 +8,34 @@
 // window (sigma 1.5, zero outside the image), C1 = 0.01^2, C2 = 0.03^2,
 // averaged over pixels and channels; L2 is the mean of (C - C_gt)^2.
 //
-// One CTA owns a 32 x 32 output tile of one view (views of any size, the
-// image layout of the renderer: concatenated [H][W][3] blocks). Its gradient needs SSIM's
-// partials a = ds/dmu_x, b = ds/d(F x^2), c = ds/d(F xy) on the tile plus a
-// 5-pixel halo (42 x 42), and those need the image on a 10-pixel halo
-// (52 x 52). Per channel: image values to shared memory; separable window
-// over the five moments (rows, then columns); SSIM and its partials (zero
-// at pixels outside the image, which are not in the mean); separable window
-// over the three partials; gradient = 2 w_l2 (x - y) - w_ssim (F a + 2 x F b
-// + y F c) with the symmetric window as its own adjoint. The halo is
-// recomputed by neighbouring CTAs instead of round-tripping the partials
-// through HBM: HBM traffic is the two images read and the gradient written.
+// One CTA owns a strip of kOutW columns and some rows of one view, all three
+// channels (views of any size, the image layout of the renderer: concatenated
+// [H][W][3] blocks), and streams down it kRows rows at a time. The gradient
+// needs SSIM's partials a = ds/dmu_x, b = ds/d(F (x^2 + y^2)), c = ds/d(F xy)
+// on a 5-pixel halo, and those the image on a 10-pixel halo. Per group of
+// rows: image values to a ring of rows in shared memory; the window along the
+// rows over the four moments (x, y, x^2 + y^2, xy: SSIM needs the squares
+// only in this sum); along the columns, one thread per column, into the sums
+// of the eleven rows that a row reaches, which stay in registers from group to
+// group; SSIM and its partials (zero at pixels outside the image, which are
+// not in the mean) where a row's sums are complete; the window over the three
+// partials the same way; gradient = 2 w_l2 (x - y) - w_ssim (F a + 2 x F b + y F
+// c) with the symmetric window as its own adjoint. HBM traffic is the two
+// images read and the gradient written.
+//
+// Streaming leaves a halo to recompute only beside a strip (64 of 54 columns)
+// and above a segment of rows: ~180 window FMAs per value, the square sum
+// included, against 288 for 32 x 32 tiles that recompute it on all sides
+// (52 x 52 -> 42 x 42 -> 32 x 32). Bound: issue (55 % of the slots busy at 12
+// warps per SM) and the FP32 pipe. 64 mixed views (97 M values) took 2.01 ms,
+// now 1.30; one 800^2 view 53 us, now 41. Three CTAs per SM spill the sums
+// (112 registers: 1.70 ms without loads in flight, 2.13 with).
+//
+// The moments are taken of x - 1/2 and y - 1/2 (pixels outside the image: -1/2):
+// variances and covariance do not move, and the cancellation in F x^2 -
+// (F x)^2 loses two bits less. Error of the
+// gradient against 64 bits on those views: 1.2e-5 of its norm, now 3.3e-6.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -29,30 +46,24 @@ namespace {
 
 constexpr int kR = 5;
 constexpr int kTaps = 2 * kR + 1;
-constexpr int kTW = 32, kTH = 32;                       // output tile
-constexpr int kAW = kTW + 2 * kR, kAH = kTH + 2 * kR;   // SSIM partials: 42 x 42
-constexpr int kIW = kTW + 4 * kR, kIH = kTH + 4 * kR;   // image values: 52 x 52
-// shared-memory row strides (in elements), odd so that threads walking down
-// rows hit distinct banks
-constexpr int kSI = kIW + 1, kSH1 = kAW + 1, kSA = kAW + 1, kSH2 = kTW + 1;
-constexpr int kI = kIH * kSI, kH1 = kIH * kSH1, kA = kAH * kSA, kH2 = kAH * kSH2;
-constexpr int kLossThreads = 256;
-constexpr int kLoadRows = (kIH + kLossThreads / 32 - 1) / (kLossThreads / 32);
-static_assert(kIW <= 64, "a region row is two loads per lane");
-// (x, y) pairs; windowed rows as pairs (x, y), (x^2, y^2) and singles xy;
-// partials as pairs (a, b) and singles c; second horizontal pass aliased on
-// the first one's buffer
-constexpr int kLossSmem = (int)(sizeof(float2) * (kI + 2 * kH1 + kA) + sizeof(float) * (kH1 + kA));
-static_assert(sizeof(float2) * kH2 + sizeof(float) * kH2 <= sizeof(float2) * 2 * kH1, "aliasing");
-static_assert(2 * kLossSmem + 2048 <= 232448, "two CTAs per SM");
-// register blocking: each thread filters a run of consecutive outputs and
-// loads every input of the run once (runs of 7 columns in the first
-// horizontal pass, 7 rows in the first vertical one, 8 columns and 4 rows in
-// the passes over the partials)
-constexpr int kRunH1 = 7, kRunV1 = 7, kRunH2 = 8, kRunV2 = 4;
-static_assert(kAW % kRunH1 == 0 && kAH % kRunV1 == 0 && kTW % kRunH2 == 0 && kTH % kRunV2 == 0, "runs tile");
-static_assert((kAW / kRunH1) * kIH <= 2 * kLossThreads && (kAH / kRunV1) * kAW <= kLossThreads &&
-              (kTW / kRunH2) * kAH <= kLossThreads && (kTH / kRunV2) * kTW <= kLossThreads, "work items");
+constexpr int kLossThreads = 192;                       // 3 channels x 64 columns
+constexpr int kOutW = 54, kPartW = kOutW + 2 * kR, kInW = kOutW + 4 * kR;  // columns: output, partials, image
+constexpr int kRows = 8;                                // rows per group
+constexpr int kRun = 8;                                 // columns a thread filters along a row
+constexpr int kRing = kRows + 2 * kR;                   // image rows held: an output row completes 10 rows behind
+static_assert(kLossThreads == 3 * kPartW && kPartW == kRun * (kLossThreads / 3 / kRows), "one item per thread and phase");
+// Shared-memory strides: one element of padding per 8, so that threads whose
+// runs start 8 apart hit distinct banks; the ring's rows 16 banks apart (a half
+// warp reads 8 runs of 2 rows), its channels 12 (three channels stored together)
+__host__ __device__ constexpr int pad8(int i) { return i + (i >> 3); }
+constexpr int kInStride = 88, kInPlane = kRing * kInStride + 6;  // float2 (x, y)
+constexpr int kPartStride = pad8(kPartW), kPartPlane = kRows * kPartStride;  // float4
+static_assert(pad8(kInW - 1) < kInStride && kInStride * 2 % 32 == 16, "ring row");
+constexpr int kLossSmem = (int)(sizeof(float2) * 3 * kInPlane + sizeof(float4) * 3 * kPartPlane);
+static_assert(2 * kLossSmem + 4096 <= 232448, "two CTAs per SM");
+constexpr int kExtra = 3 * kInW - kLossThreads;         // values of an image row beyond one per thread
+constexpr int kExtraLoads = (kExtra * kRows + kLossThreads - 1) / kLossThreads;
+constexpr float kShift = 0.5f;
 
 constexpr float kC1 = 0.01f * 0.01f;
 constexpr float kC2 = 0.03f * 0.03f;
@@ -83,17 +94,22 @@ __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
 
 struct LossView {
   long long off;       // first pixel of the view in the concatenated images
-  int W, H, tiles_x, tile0;
+  int W, H, strips, tile0;
   float w_l2, w_ssim;  // scale (1 - lambda) / N and scale lambda / N, N = 3 W H
 };
 
 struct LossArgs {
   const float *img, *gt;
   float *dimg, *loss;
-  int n_views;
+  int n_views, seg;    // seg: output rows of a CTA
   float g[kTaps];      // 1-D window weights
   f32x2 g2[kTaps];     // the same, each weight in both lanes
   LossView view[kMaxLossViews];
@@ -102,16 +118,11 @@ static_assert(sizeof(LossArgs) <= 4000, "kernel parameters");
 
 __global__ void __launch_bounds__(kLossThreads, 2) k_l2_dssim_grad(const __grid_constant__ LossArgs a) {
   extern __shared__ float4 sm4[];
-  float2 *sxy = reinterpret_cast<float2 *>(sm4);       // [kIH][kSI] (x, y)
-  float2 *h1p = sxy + kI;                              // [2][kIH][kSH1] rows of (x, y), (x^2, y^2)
-  float2 *pab = h1p + 2 * kH1;                         // [kAH][kSA] partials (a, b)
-  float *h1s = reinterpret_cast<float *>(pab + kA);    // [kIH][kSH1] rows of xy
-  float *pc = h1s + kH1;                               // [kAH][kSA] partial c
-  float2 *h2p = h1p;                                   // [kAH][kSH2] rows of (a, b)
-  float *h2s = reinterpret_cast<float *>(h1p + kH2);   // [kAH][kSH2] rows of c
+  float4 *part = sm4;                                             // [3][kRows][kPartStride] rows of moments / partials
+  float2 *ring = reinterpret_cast<float2 *>(sm4 + 3 * kPartPlane);  // [3][kRing][kInStride] (x, y)
   __shared__ float s_red[kLossThreads / 32];
 
-  // the view this tile belongs to: last view whose first tile is <= blockIdx.x
+  // the view this CTA belongs to: last view whose first tile is <= blockIdx.x
   int lo = 0, hi = a.n_views - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
@@ -121,207 +132,239 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_l2_dssim_grad(const __grid_
   const LossView &vw = a.view[lo];
   const int W = vw.W, H = vw.H;
   const int tile = blockIdx.x - vw.tile0;
-  const int x0 = (tile % vw.tiles_x) * kTW, y0 = (tile / vw.tiles_x) * kTH;
-  const size_t base = (size_t)vw.off;
+  const int x0 = (tile % vw.strips) * kOutW, y0 = (tile / vw.strips) * a.seg;
+  const int y1 = min(y0 + a.seg, H);
   const float w_l2 = vw.w_l2, w_ssim = vw.w_ssim;
   const int tid = threadIdx.x;
+  const int ch = tid / kPartW, col = tid % kPartW;    // column phases: channel and column
+  const int hrow = col / (kPartW / kRun), hrun = col % (kPartW / kRun);  // row phases: row and run of columns
+  float4 *pch = part + ch * kPartPlane;
+  const float2 *rch = ring + ch * kInPlane;
+
+  // loads: value e of an image row (pixel e / 3, channel e % 3) by thread e, the
+  // kExtra values beyond one per thread spread over the threads
+  const long long pitch = 3ll * W;
+  const long long origin = (vw.off + (long long)(y0 - 2 * kR) * W + x0 - 2 * kR) * 3;  // of the first image row's values
+  const int gx = x0 - 2 * kR + tid / 3;
+  const bool col_ok = gx >= 0 && gx < W;
+  const int slot_e = (tid % 3) * kInPlane + pad8(tid / 3);
+  float2 ld[kRows], lx[kExtraLoads];
+  auto load = [&](int i0) {  // image rows i0 .. i0 + kRows - 1 of the strip into registers
+#pragma unroll
+    for (int r = 0; r < kRows; r++) {
+      const int gy = y0 - 2 * kR + i0 + r;
+      ld[r] = make_float2(0.f, 0.f);
+      if (col_ok && gy >= 0 && gy < H) {
+        const long long o = origin + (i0 + r) * pitch + tid;
+        ld[r] = make_float2(__ldg(a.img + o), __ldg(a.gt + o));
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < kExtraLoads; k++) {
+      const int q = tid + k * kLossThreads, r = q / kExtra, e = kLossThreads + q % kExtra;
+      const int gy = y0 - 2 * kR + i0 + r, x = x0 - 2 * kR + e / 3;
+      lx[k] = make_float2(0.f, 0.f);
+      if (r < kRows && x >= 0 && x < W && gy >= 0 && gy < H) {
+        const long long o = origin + (i0 + r) * pitch + e;
+        lx[k] = make_float2(__ldg(a.img + o), __ldg(a.gt + o));
+      }
+    }
+  };
+
+  // sums of the rows begun: moments of rows i0 - 5 .. i0 + 4 (image rows of the strip), partials five rows behind
+  f32x2 m01[2 * kR], m23[2 * kR], fab[2 * kR];
+  float fc[2 * kR];
+#pragma unroll
+  for (int k = 0; k < 2 * kR; k++) {
+    m01[k] = m23[k] = fab[k] = 0ull;
+    fc[k] = 0.f;
+  }
   float acc = 0.f;
+  const int n_rows = y1 - y0 + 4 * kR;
+  load(0);
+  int base = 0;  // ring slot of image row i0
+  for (int i0 = 0; i0 < n_rows; i0 += kRows) {
+#pragma unroll
+    for (int r = 0; r < kRows; r++) {
+      int s = base + r;
+      s -= s >= kRing ? kRing : 0;
+      ring[slot_e + s * kInStride] = ld[r];
+    }
+#pragma unroll
+    for (int k = 0; k < kExtraLoads; k++) {
+      const int q = tid + k * kLossThreads, r = q / kExtra, e = kLossThreads + q % kExtra;
+      int s = base + r;
+      s -= s >= kRing ? kRing : 0;
+      if (r < kRows) ring[(e % 3) * kInPlane + s * kInStride + pad8(e / 3)] = lx[k];
+    }
+    __syncthreads();
+    if (i0 + kRows < n_rows) load(i0 + kRows);  // in flight over the phases below
 
-  for (int c = 0; c < 3; ++c) {
+    // along the rows: moments of kRun columns of one row
     {
-      // warp w loads rows w, w + 8, ... of the region; every load in flight
-      // at once, then the stores
-      const int warp = tid >> 5, lane = tid & 31;
-      float2 v[kLoadRows][2];
+      int s = base + hrow;
+      s -= s >= kRing ? kRing : 0;
+      const float2 *in = rch + s * kInStride + hrun * (kRun + 1);
+      f32x2 h01[kRun], h23[kRun];
 #pragma unroll
-      for (int k = 0; k < kLoadRows; ++k) {
-        const int r = warp + k * (kLossThreads / 32);
-        const int gy = y0 - 2 * kR + r;
-        const bool row_ok = r < kIH && gy >= 0 && gy < H;
-        const size_t row = (base + (size_t)(row_ok ? gy : 0) * W) * 3 + c;
+      for (int j = 0; j < kRun; j++) h01[j] = h23[j] = 0ull;
+      const f32x2 shift = pk(-kShift, -kShift);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int q = lane + 32 * h;
-          const int gx = x0 - 2 * kR + q;
-          v[k][h] = make_float2(0.f, 0.f);
-          if (row_ok && q < kIW && gx >= 0 && gx < W) {
-            v[k][h].x = __ldg(a.img + row + 3 * (size_t)gx);
-            v[k][h].y = __ldg(a.gt + row + 3 * (size_t)gx);
+      for (int i = 0; i < kRun + 2 * kR; i++) {
+        const f32x2 xy2 = add2(pk(in[i + (i >> 3)]), shift);
+        const float2 v = unpk(xy2);
+        const f32x2 sp = pk(fmaf(v.x, v.x, v.y * v.y), v.x * v.y);
+#pragma unroll
+        for (int j = 0; j < kRun; j++) {
+          const int t = i - j;
+          if (t >= 0 && t < kTaps) {
+            h01[j] = fma2(a.g2[t], xy2, h01[j]);
+            h23[j] = fma2(a.g2[t], sp, h23[j]);
           }
         }
       }
+      float4 *o = pch + hrow * kPartStride + hrun * (kRun + 1);
 #pragma unroll
-      for (int k = 0; k < kLoadRows; ++k) {
-        const int r = warp + k * (kLossThreads / 32);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int q = lane + 32 * h;
-          if (r < kIH && q < kIW) sxy[r * kSI + q] = v[k][h];
-        }
+      for (int j = 0; j < kRun; j++) {
+        const float2 u = unpk(h01[j]), v = unpk(h23[j]);
+        o[j] = make_float4(u.x, u.y, v.x, v.y);
       }
     }
     __syncthreads();
 
-    // rows: (x, y), (x^2, y^2) and xy under the 1-D window, runs of kRunH1 columns
-    for (int it = tid; it < (kAW / kRunH1) * kIH; it += kLossThreads) {
-      const int r = it % kIH, q0 = (it / kIH) * kRunH1;
-      f32x2 m01[kRunH1], m23[kRunH1];
-      float m4[kRunH1];
+    // along the columns: image row i0 + r completes the moments of row i0 + r - 5, in place
+    {
+      const int gxp = x0 - kR + col;
+      const bool x_ok = gxp >= 0 && gxp < W;
+      const bool own = col >= kR && col < kR + kOutW;
+      f32x2 s01[kRows + 2 * kR], s23[kRows + 2 * kR];
 #pragma unroll
-      for (int j = 0; j < kRunH1; ++j) {
-        m01[j] = m23[j] = 0ull;
-        m4[j] = 0.f;
+      for (int k = 0; k < 2 * kR; k++) {
+        s01[k] = m01[k];
+        s23[k] = m23[k];
       }
 #pragma unroll
-      for (int i = 0; i < kRunH1 + 2 * kR; ++i) {
-        const float2 v = sxy[r * kSI + q0 + i];
-        const f32x2 xy2 = pk(v);
-        const f32x2 sq2 = mul2(xy2, xy2);
-        const float xy = v.x * v.y;
+      for (int r = 0; r < kRows; r++) {
+        float4 *cell = pch + r * kPartStride + pad8(col);
+        const float4 h = *cell;
+        const f32x2 u = pk(h.x, h.y), v = pk(h.z, h.w);
 #pragma unroll
-        for (int j = 0; j < kRunH1; ++j) {
-          const int t = i - j;
-          if (t >= 0 && t < kTaps) {
-            m01[j] = fma2(a.g2[t], xy2, m01[j]);
-            m23[j] = fma2(a.g2[t], sq2, m23[j]);
-            m4[j] = fmaf(a.g[t], xy, m4[j]);
-          }
+        for (int t = 0; t < kTaps - 1; t++) {
+          s01[r + t] = fma2(a.g2[t], u, s01[r + t]);
+          s23[r + t] = fma2(a.g2[t], v, s23[r + t]);
         }
-      }
-#pragma unroll
-      for (int j = 0; j < kRunH1; ++j) {
-        h1p[r * kSH1 + q0 + j] = unpk(m01[j]);
-        h1p[kH1 + r * kSH1 + q0 + j] = unpk(m23[j]);
-        h1s[r * kSH1 + q0 + j] = m4[j];
-      }
-    }
-    __syncthreads();
-
-    // columns, then SSIM and its partials, runs of kRunV1 rows
-    if (tid < (kAH / kRunV1) * kAW) {
-      const int q = tid % kAW, r0 = (tid / kAW) * kRunV1;
-      f32x2 m01[kRunV1], m23[kRunV1];
-      float m4[kRunV1];
-#pragma unroll
-      for (int j = 0; j < kRunV1; ++j) {
-        m01[j] = m23[j] = 0ull;
-        m4[j] = 0.f;
-      }
-#pragma unroll
-      for (int i = 0; i < kRunV1 + 2 * kR; ++i) {
-        const int o = (r0 + i) * kSH1 + q;
-        const f32x2 u = pk(h1p[o]), w = pk(h1p[kH1 + o]);
-        const float z = h1s[o];
-#pragma unroll
-        for (int j = 0; j < kRunV1; ++j) {
-          const int t = i - j;
-          if (t >= 0 && t < kTaps) {
-            m01[j] = fma2(a.g2[t], u, m01[j]);
-            m23[j] = fma2(a.g2[t], w, m23[j]);
-            m4[j] = fmaf(a.g[t], z, m4[j]);
-          }
-        }
-      }
-      const int gx = x0 - kR + q;
-#pragma unroll
-      for (int j = 0; j < kRunV1; ++j) {
-        const int r = r0 + j, gy = y0 - kR + r;
-        float2 dab = make_float2(0.f, 0.f);
-        float dc = 0.f;
-        if (gy >= 0 && gy < H && gx >= 0 && gx < W) {
-          const float2 mu = unpk(m01[j]), sq = unpk(m23[j]);
-          const float mx = mu.x, my = mu.y;
+        s01[r + kTaps - 1] = mul2(a.g2[kTaps - 1], u);
+        s23[r + kTaps - 1] = mul2(a.g2[kTaps - 1], v);
+        const int gyp = y0 - 3 * kR + i0 + r;  // its row in the view
+        float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (x_ok && gyp >= 0 && gyp < H && gyp >= y0 - kR) {
+          const float2 mu = unpk(s01[r]), sp = unpk(s23[r]);
+          const float mx = mu.x + kShift, my = mu.y + kShift;
           const float l1 = 2.f * mx * my + kC1;
-          const float cs1 = 2.f * (m4[j] - mx * my) + kC2;
+          const float cs1 = 2.f * (sp.y - mu.x * mu.y) + kC2;
           const float l2 = mx * mx + my * my + kC1;
-          const float cs2 = (sq.x - mx * mx) + (sq.y - my * my) + kC2;
+          const float cs2 = (sp.x - (mu.x * mu.x + mu.y * mu.y)) + kC2;
           const float rD = __fdividef(1.f, l2 * cs2);  // D in [C1 C2, 4 (1 + C1) (2 + C2)]
           const float s = l1 * cs1 * rD;
-          const float dN = 2.f * my * (cs1 - l1);
-          const float dD = 2.f * mx * (cs2 - l2);
-          dab.x = (dN - s * dD) * rD;
-          dab.y = -s * l2 * rD;
-          dc = 2.f * l1 * rD;
-          if (r >= kR && r < kR + kTH && q >= kR && q < kR + kTW) {
-            const float2 v = sxy[(r + kR) * kSI + q + kR];
-            const float d = v.x - v.y;
-            acc += w_l2 * d * d + w_ssim * (1.f - s);
-          }
+          const float dN = 2.f * (my * cs1 - mu.y * l1);
+          const float dD = 2.f * (mx * cs2 - mu.x * l2);
+          d.x = (dN - s * dD) * rD;
+          d.y = -s * l2 * rD;
+          d.z = 2.f * l1 * rD;
+          if (own && gyp >= y0 && gyp < y1) acc += w_ssim * (1.f - s);
         }
-        pab[r * kSA + q] = dab;
-        pc[r * kSA + q] = dc;
+        *cell = d;
+      }
+#pragma unroll
+      for (int k = 0; k < 2 * kR; k++) {
+        m01[k] = s01[kRows + k];
+        m23[k] = s23[kRows + k];
       }
     }
     __syncthreads();
 
-    // rows of the partials, runs of kRunH2 columns
-    if (tid < (kTW / kRunH2) * kAH) {
-      const int r = tid % kAH, q0 = (tid / kAH) * kRunH2;
-      f32x2 fab[kRunH2];
-      float fc[kRunH2];
+    // along the rows of the partials (the last run's columns beyond kOutW read padding or the next
+    // row's values and are not used)
+    float4 h2[kRun];
+    {
+      const float4 *in = pch + hrow * kPartStride + hrun * (kRun + 1);
+      f32x2 hab[kRun];
+      float hc[kRun];
 #pragma unroll
-      for (int j = 0; j < kRunH2; ++j) {
-        fab[j] = 0ull;
-        fc[j] = 0.f;
+      for (int j = 0; j < kRun; j++) {
+        hab[j] = 0ull;
+        hc[j] = 0.f;
       }
 #pragma unroll
-      for (int i = 0; i < kRunH2 + 2 * kR; ++i) {
-        const f32x2 u = pk(pab[r * kSA + q0 + i]);
-        const float z = pc[r * kSA + q0 + i];
+      for (int i = 0; i < kRun + 2 * kR; i++) {
+        if (hrun * kRun + i >= kPartW) break;
+        const float4 d = in[i + (i >> 3)];
+        const f32x2 u = pk(d.x, d.y);
 #pragma unroll
-        for (int j = 0; j < kRunH2; ++j) {
+        for (int j = 0; j < kRun; j++) {
           const int t = i - j;
           if (t >= 0 && t < kTaps) {
-            fab[j] = fma2(a.g2[t], u, fab[j]);
-            fc[j] = fmaf(a.g[t], z, fc[j]);
+            hab[j] = fma2(a.g2[t], u, hab[j]);
+            hc[j] = fmaf(a.g[t], d.z, hc[j]);
           }
         }
       }
 #pragma unroll
-      for (int j = 0; j < kRunH2; ++j) {
-        h2p[r * kSH2 + q0 + j] = unpk(fab[j]);
-        h2s[r * kSH2 + q0 + j] = fc[j];
+      for (int j = 0; j < kRun; j++) {
+        const float2 u = unpk(hab[j]);
+        h2[j] = make_float4(u.x, u.y, hc[j], 0.f);
       }
+    }
+    __syncthreads();
+    {
+      float4 *o = pch + hrow * kPartStride + hrun * (kRun + 1);
+#pragma unroll
+      for (int j = 0; j < kRun; j++) o[j] = h2[j];
     }
     __syncthreads();
 
-    // columns of the partials and the gradient, runs of kRunV2 rows
-    if (tid < (kTH / kRunV2) * kTW) {
-      const int q = tid % kTW, r0 = (tid / kTW) * kRunV2;
-      f32x2 fab[kRunV2];
-      float fc[kRunV2];
+    // along the columns of the partials: row i0 + r completes output row i0 + r - 20
+    if (col < kOutW) {
+      const int gxo = x0 + col;
+      f32x2 sab[kRows + 2 * kR];
+      float sc[kRows + 2 * kR];
 #pragma unroll
-      for (int j = 0; j < kRunV2; ++j) {
-        fab[j] = 0ull;
-        fc[j] = 0.f;
+      for (int k = 0; k < 2 * kR; k++) {
+        sab[k] = fab[k];
+        sc[k] = fc[k];
       }
 #pragma unroll
-      for (int i = 0; i < kRunV2 + 2 * kR; ++i) {
-        const int o = (r0 + i) * kSH2 + q;
-        const f32x2 u = pk(h2p[o]);
-        const float z = h2s[o];
+      for (int r = 0; r < kRows; r++) {
+        const float4 h = pch[r * kPartStride + pad8(col)];
+        const f32x2 u = pk(h.x, h.y);
 #pragma unroll
-        for (int j = 0; j < kRunV2; ++j) {
-          const int t = i - j;
-          if (t >= 0 && t < kTaps) {
-            fab[j] = fma2(a.g2[t], u, fab[j]);
-            fc[j] = fmaf(a.g[t], z, fc[j]);
-          }
+        for (int t = 0; t < kTaps - 1; t++) {
+          sab[r + t] = fma2(a.g2[t], u, sab[r + t]);
+          sc[r + t] = fmaf(a.g[t], h.z, sc[r + t]);
+        }
+        sab[r + kTaps - 1] = mul2(a.g2[kTaps - 1], u);
+        sc[r + kTaps - 1] = a.g[kTaps - 1] * h.z;
+        const int gyo = y0 - 4 * kR + i0 + r;
+        if (gyo >= y0 && gyo < y1 && gxo < W) {
+          int s = base + r - 2 * kR;  // the ring's oldest rows
+          s += s < 0 ? kRing : 0;
+          const float2 v = rch[s * kInStride + pad8(col + 2 * kR)];
+          const float2 f = unpk(sab[r]);
+          const float diff = v.x - v.y;
+          const float dssim = f.x + 2.f * (v.x - kShift) * f.y + (v.y - kShift) * sc[r];
+          a.dimg[(vw.off + (long long)gyo * W + gxo) * 3 + ch] = 2.f * w_l2 * diff - w_ssim * dssim;
+          acc += w_l2 * diff * diff;
         }
       }
-      const int gx = x0 + q;
 #pragma unroll
-      for (int j = 0; j < kRunV2; ++j) {
-        const int r = r0 + j, gy = y0 + r;
-        if (gy < H && gx < W) {
-          const float2 v = sxy[(r + 2 * kR) * kSI + q + 2 * kR];
-          const float2 f = unpk(fab[j]);
-          const float dssim = f.x + 2.f * v.x * f.y + v.y * fc[j];
-          a.dimg[(base + (size_t)gy * W + gx) * 3 + c] = 2.f * w_l2 * (v.x - v.y) - w_ssim * dssim;
-        }
+      for (int k = 0; k < 2 * kR; k++) {
+        fab[k] = sab[kRows + k];
+        fc[k] = sc[kRows + k];
       }
     }
     __syncthreads();
+    base += kRows;
+    base -= base >= kRing ? kRing : 0;
   }
 
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
@@ -332,6 +375,28 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_l2_dssim_grad(const __grid_
     for (int k = 0; k < kLossThreads / 32; ++k) t += s_red[k];
     atomicAdd(a.loss, t);
   }
+}
+
+// Output rows per CTA of a launch over views[0, n): the length whose waves of
+// CTAs (two per SM) take the fewest rows each, 4 kR rows of halo included; a multiple of
+// kRows less the halo, so that the last group is full.
+int loss_segment(const LossView *views, int n, int slots) {
+  int best = 0;
+  long long best_cost = 0;
+  for (int seg = 2 * kRows - 4; seg <= 1020; seg += kRows) {
+    long long ctas = 0;
+    int rows = 0;
+    for (int v = 0; v < n; ++v) {
+      ctas += (long long)views[v].strips * ((views[v].H + seg - 1) / seg);
+      rows = std::max(rows, std::min(views[v].H, seg) + 4 * kR);
+    }
+    const long long cost = (ctas + slots - 1) / slots * rows;
+    if (!best || cost < best_cost) {
+      best = seg;
+      best_cost = cost;
+    }
+  }
+  return best;
 }
 
 }  // namespace
@@ -356,11 +421,13 @@ int launch_l2_dssim_grad(const float *img, const float *gt, int n_views, const i
     a.g2[t] = ((unsigned long long)bits << 32) | bits;
   }
   cudaFuncSetAttribute(k_l2_dssim_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, kLossSmem);
+  int sms = 0, dev = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   int launches = 0;
   long long off = 0;
   for (int v0 = 0; v0 < n_views; v0 += kMaxLossViews) {
     a.n_views = 0;
-    int tiles = 0;
     for (int v = v0; v < n_views && v < v0 + kMaxLossViews; ++v) {
       const int W = sizes[2 * v], H = sizes[2 * v + 1];
       const long long npx = (long long)W * H;
@@ -369,16 +436,21 @@ int launch_l2_dssim_grad(const float *img, const float *gt, int n_views, const i
         r.off = off;
         r.W = W;
         r.H = H;
-        r.tiles_x = (W + kTW - 1) / kTW;
-        r.tile0 = tiles;
-        tiles += r.tiles_x * ((H + kTH - 1) / kTH);
+        r.strips = (W + kOutW - 1) / kOutW;
         const double n = 3.0 * (double)npx;
         r.w_l2 = (float)((double)scale * (1.0 - (double)lambda) / n);
         r.w_ssim = (float)((double)scale * (double)lambda / n);
       }
       off += npx;
     }
-    if (tiles == 0) continue;
+    if (a.n_views == 0) continue;
+    a.seg = loss_segment(a.view, a.n_views, 2 * (sms > 0 ? sms : 152));
+    int tiles = 0;
+    for (int v = 0; v < a.n_views; ++v) {
+      LossView &r = a.view[v];
+      r.tile0 = tiles;
+      tiles += r.strips * ((r.H + a.seg - 1) / a.seg);
+    }
     k_l2_dssim_grad<<<tiles, kLossThreads, kLossSmem, st>>>(a);
     ++launches;
   }
