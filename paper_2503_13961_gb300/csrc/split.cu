@@ -13,6 +13,7 @@
 // (U, M_uv, M_uw), (M_uv, V, M_vw), (M_uw, M_vw, W), (M_vw, M_uw, M_uv), M
 // the edge midpoints, so every weight is 0, 1/2 or 1.
 #include <cmath>
+#include <cstdint>
 
 #include <cuda/atomic>
 
@@ -42,77 +43,108 @@ struct SplitArgs {
   bgt_prims out;
 };
 
-// de Casteljau with one parameter per level, in place: at level r the
-// degree-(d + 1) net becomes the degree-d net, slot(a, b) <- u net[slot(a, b)]
-// + v net[slot(a + 1, b)] + w net[slot(a + 1, b + 1)]; ascending slots only
-// overwrite values no later slot reads.
-template <int N, int C>
-__device__ __forceinline__ void blossom(float (&net)[kNcp<N>][C], const float (&par)[N][3]) {
+// One level of de Casteljau with parameter (u, v, w): the degree-D net to the
+// degree-(D - 1) net, slot(a, b) <- u net[slot(a, b)] + v net[slot(a + 1, b)] + w net[slot(a + 1, b + 1)]
+template <int D>
+__device__ __forceinline__ void casteljau(const float (&net)[kNcp<D>], const float (&par)[3], float (&out)[kNcp<D - 1>]) {
 #pragma unroll
-  for (int r = 0; r < N; ++r) {
-    const int d = N - 1 - r;
-    const float u = par[r][0], v = par[r][1], w = par[r][2];
+  for (int a = 0; a < D; ++a)
 #pragma unroll
-    for (int a = 0; a <= d; ++a)
-#pragma unroll
-      for (int b = 0; b <= a; ++b)
-#pragma unroll
-        for (int ch = 0; ch < C; ++ch)
-          net[slot(a, b)][ch] = u * net[slot(a, b)][ch] + v * net[slot(a + 1, b)][ch] +
-                                w * net[slot(a + 1, b + 1)][ch];
+    for (int b = 0; b <= a; ++b)
+      out[slot(a, b)] = par[0] * net[slot(a, b)] + par[1] * net[slot(a + 1, b)] + par[2] * net[slot(a + 1, b + 1)];
+}
+
+// All polar values of the degree-N net that extend the arguments so far (A x i,
+// B x j, C x k; net: the degree-D net behind them) by D more, no corner before
+// C of them: the shared prefixes (A, then B, then C) are evaluated once.
+template <int N, int D, int C, int I, int J>
+__device__ __forceinline__ void polar_tree(const float (&net)[kNcp<D>], const float (&par)[3][3], float *out) {
+  if constexpr (D == 0) {
+    constexpr int a = N - I, b = N - I - J;  // control point (I, J, k): slot(n - i, k)
+    out[3 * slot(a, b)] = net[0];
+  } else {
+    float sub[kNcp<D - 1>];
+    if constexpr (C == 0) {
+      casteljau<D>(net, par[0], sub);
+      polar_tree<N, D - 1, 0, I + 1, J>(sub, par, out);
+    }
+    if constexpr (C <= 1) {
+      casteljau<D>(net, par[1], sub);
+      polar_tree<N, D - 1, 1, I, J + 1>(sub, par, out);
+    }
+    casteljau<D>(net, par[2], sub);
+    polar_tree<N, D - 1, 2, I, J>(sub, par, out);
   }
 }
 
-// one thread per (selected primitive, piece, control point or texel)
-template <int N>
-__global__ void __launch_bounds__(256) k_subdivide(const SplitArgs s) {
-  constexpr int NC = kNcp<N>;
-  const int per = max(NC, s.T);
-  const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gid >= 4LL * s.n_sel * per) return;
-  const int e = (int)(gid % per);
-  const long long sp = gid / per;
-  const int piece = (int)(sp & 3);
-  const long long child = sp;  // output primitive 4 sel_index + piece
-  const int m = __ldg(s.sel + (sp >> 2));
-  const bool valid = m >= 0 && m < s.M;
+constexpr int kSplitParents = 8;                       // parents per block
+constexpr int kSplitThreads = kSplitParents * 4 * 6;   // one thread per (parent, piece, channel)
 
-  if (e < NC) {
-    // target control point q_ijk, a = n - i, b = k
-    int a = 0;
-    while (slot(a + 1, 0) <= e) ++a;
-    const int b = e - slot(a, 0);
-    const int i = N - a, k = b, j = N - i - k;
-    float par[N][3];
+// Blocks of kSplitParents selected primitives: their control points and
+// colours through shared memory, one thread per piece and channel evaluating
+// the piece's whole net (46 de Casteljau nodes for the 10 control points at
+// degree 3, by shared prefixes), the pieces written coalesced from shared memory; then the
+// map texels and the copied attributes. One thread per control point evaluated
+// all six channels of a polar form of its own from 60 loads (degree 3): 55 us
+// for 25,000 of 100,000 primitives with maps of leg 3, now 26.
+template <int N>
+__global__ void __launch_bounds__(kSplitThreads) k_subdivide(const SplitArgs s) {
+  constexpr int NC = kNcp<N>;
+  __shared__ float s_in[kSplitParents][2][3 * NC];
+  __shared__ __align__(16) float s_out[2][kSplitParents * 4 * 3 * NC];
+  const long long first = (long long)blockIdx.x * kSplitParents;
+  const int count = (int)min((long long)kSplitParents, s.n_sel - first);
+  const int tid = threadIdx.x;
+  const float nanv = __int_as_float(0x7fc00000);
+  for (int q = tid; q < count * 6 * NC; q += kSplitThreads) {
+    const int par = q / (6 * NC), e = q - par * 6 * NC;
+    const int m = __ldg(s.sel + first + par);
+    const bool ok = m >= 0 && m < s.M;
+    const float *src = e < 3 * NC ? s.ctrl : s.color;
+    const int k = e < 3 * NC ? e : e - 3 * NC;
+    s_in[par][e >= 3 * NC][k] = ok ? __ldg(src + (size_t)m * 3 * NC + k) : nanv;
+  }
+  __syncthreads();
+  {
+    const int par = tid / 24, piece = (tid / 6) % 4, ch = tid % 6;
+    if (par < count) {
+      float net[NC], corner[3][3];
 #pragma unroll
-    for (int r = 0; r < N; ++r) {
-      const int corner = r < i ? 0 : (r < i + j ? 1 : 2);
+      for (int t = 0; t < NC; ++t) net[t] = s_in[par][ch / 3][3 * t + ch % 3];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) par[r][c] = 0.5f * (float)c_piece[piece][corner][c];
+      for (int r = 0; r < 3; ++r)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) corner[r][c] = 0.5f * (float)c_piece[piece][r][c];
+      polar_tree<N, N, 0, 0, 0>(net, corner, &s_out[ch / 3][(par * 4 + piece) * 3 * NC + ch % 3]);
     }
-    float net[NC][6];
-#pragma unroll
-    for (int t = 0; t < NC; ++t)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        net[t][c] = valid ? __ldg(s.ctrl + ((size_t)m * NC + t) * 3 + c) : __int_as_float(0x7fc00000);
-        net[t][3 + c] = valid ? __ldg(s.color + ((size_t)m * NC + t) * 3 + c) : __int_as_float(0x7fc00000);
+  }
+  __syncthreads();
+  {
+    const int n = count * 4 * 3 * NC;
+    const size_t o = (size_t)first * 4 * 3 * NC;
+    const bool vec = ((reinterpret_cast<uintptr_t>(s.out.ctrl) | reinterpret_cast<uintptr_t>(s.out.color)) & 15) == 0;
+    if (vec) {  // 4 pieces of 3 NC floats: whole float4 per parent
+      for (int q = tid; q < n / 4; q += kSplitThreads) {
+        reinterpret_cast<float4 *>(s.out.ctrl + o)[q] = reinterpret_cast<const float4 *>(s_out[0])[q];
+        reinterpret_cast<float4 *>(s.out.color + o)[q] = reinterpret_cast<const float4 *>(s_out[1])[q];
       }
-    blossom<N, 6>(net, par);
-    const size_t o = ((size_t)child * NC + e) * 3;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      s.out.ctrl[o + c] = net[0][c];
-      s.out.color[o + c] = net[0][3 + c];
+    } else {
+      for (int q = tid; q < n; q += kSplitThreads) {
+        s.out.ctrl[o + q] = s_out[0][q];
+        s.out.color[o + q] = s_out[1][q];
+      }
     }
   }
 
-  if (e < s.T) {
-    // texel (ti, tj) of the piece's maps: the parent's Theta at its node
+  for (int q = tid; q < count * 4 * s.T; q += kSplitThreads) {
+    // texel e of the piece's maps: the parent's Theta at its node
+    const int sp = q / s.T, e = q - sp * s.T, piece = sp & 3;
+    const int m = __ldg(s.sel + first + (sp >> 2));
+    const bool valid = m >= 0 && m < s.M;
     float lsv[3], qv[4];
     if (!valid) {
-      for (int c = 0; c < 3; ++c) lsv[c] = __int_as_float(0x7fc00000);
-      for (int c = 0; c < 4; ++c) qv[c] = __int_as_float(0x7fc00000);
+      for (int c = 0; c < 3; ++c) lsv[c] = nanv;
+      for (int c = 0; c < 4; ++c) qv[c] = nanv;
     } else if (s.R <= 1) {
       for (int c = 0; c < 3; ++c) lsv[c] = __ldg(s.log_scale + (size_t)m * 3 + c);
       for (int c = 0; c < 4; ++c) qv[c] = __ldg(s.quat + (size_t)m * 4 + c);
@@ -141,17 +173,22 @@ __global__ void __launch_bounds__(256) k_subdivide(const SplitArgs s) {
         for (int c = 0; c < 4; ++c) qv[c] = fmaf(w[t], __ldg(s.quat + base * 4 + c), qv[c]);
       }
     }
-    const size_t o = (size_t)child * s.T + e;
+    const size_t o = (size_t)first * 4 * s.T + q;
     for (int c = 0; c < 3; ++c) s.out.log_scale[o * 3 + c] = lsv[c];
     for (int c = 0; c < 4; ++c) s.out.quat[o * 4 + c] = qv[c];
   }
 
-  if (e == 0) {
-    const float nanv = __int_as_float(0x7fc00000);
-    s.out.opacity[child] = valid ? __ldg(s.opacity + m) : nanv;
-    s.out.r_b[child] = valid ? __ldg(s.r_b + m) : nanv;
-    for (int c = 0; c < 3 * s.K; ++c)
-      s.out.sh[(size_t)child * 3 * s.K + c] = valid ? __ldg(s.sh + (size_t)m * 3 * s.K + c) : nanv;
+  for (int q = tid; q < count * 4; q += kSplitThreads) {
+    const int m = __ldg(s.sel + first + (q >> 2));
+    const bool valid = m >= 0 && m < s.M;
+    s.out.opacity[first * 4 + q] = valid ? __ldg(s.opacity + m) : nanv;
+    s.out.r_b[first * 4 + q] = valid ? __ldg(s.r_b + m) : nanv;
+  }
+  for (int q = tid; q < count * 4 * 3 * s.K; q += kSplitThreads) {
+    const int sp = q / (3 * s.K), c = q - sp * 3 * s.K;
+    const int m = __ldg(s.sel + first + (sp >> 2));
+    const bool valid = m >= 0 && m < s.M;
+    s.out.sh[(size_t)first * 4 * 3 * s.K + q] = valid ? __ldg(s.sh + (size_t)m * 3 * s.K + c) : nanv;
   }
 }
 
@@ -282,25 +319,61 @@ __device__ __forceinline__ unsigned long long relaxed_load(unsigned long long *p
 // Visibility measures from the raster of views [v0, v0 + 64): per foreground
 // pixel, the bit of the flat triangle it is seen through (the low 32 bits of
 // its depth key are prim * nsub + sub-triangle) in cell_mask[prim], and bit
-// v - v0 in seen[prim]. A bit already set is read, not written again.
+// v - v0 in seen[prim]. A bit already set is read, not written again. Warps
+// take kVisRounds x 32 consecutive pixels with the loads of all rounds in
+// flight and one view search for all of them (the views are ordered): at one
+// pixel per thread the kernel waited on its chain of loads (I_id, key, mask),
+// 167 us for 32 M pixels, now 107.
+constexpr int kVisRounds = 8;
+
 __global__ void __launch_bounds__(256) k_vis_pixels(const int *pid, const unsigned long long *zbuf,
                                                     const int *view_off, int V, int pix0, int pix1, int v0,
                                                     int nsub, int words, unsigned long long *cell_mask,
                                                     unsigned long long *seen) {
-  const int pix = pix0 + blockIdx.x * blockDim.x + threadIdx.x;
-  if (pix >= pix1) return;
-  const int id = pid[pix];
-  if (id < 0) return;
+  const int lane = threadIdx.x & 31;
+  const int first = pix0 + (blockIdx.x * 8 + ((int)threadIdx.x >> 5)) * (32 * kVisRounds);
+  if (first >= pix1) return;
+  const unsigned *low = reinterpret_cast<const unsigned *>(zbuf);
+  int id[kVisRounds];
+  unsigned key[kVisRounds];
+  bool any = false;
+#pragma unroll
+  for (int r = 0; r < kVisRounds; r++) {
+    const int pix = first + r * 32 + lane;
+    id[r] = pix < pix1 ? pid[pix] : -1;
+    any = any || id[r] >= 0;
+  }
+  if (!__any_sync(0xffffffffu, any)) return;
   if (cell_mask) {
-    const int sub = (int)((unsigned)(zbuf[pix] & 0xffffffffull) - (unsigned)id * (unsigned)nsub);
-    unsigned long long *c = cell_mask + (size_t)id * words + (sub >> 6);
-    const unsigned long long bit = 1ull << (sub & 63);
-    if (!(relaxed_load(c) & bit)) atomicOr(c, bit);
+#pragma unroll
+    for (int r = 0; r < kVisRounds; r++) key[r] = id[r] >= 0 ? low[2 * (size_t)(first + r * 32 + lane)] : 0u;
+    unsigned long long have[kVisRounds];
+#pragma unroll
+    for (int r = 0; r < kVisRounds; r++) {
+      have[r] = ~0ull;
+      if (id[r] < 0) continue;
+      key[r] -= (unsigned)id[r] * (unsigned)nsub;  // the sub-triangle
+      have[r] = relaxed_load(cell_mask + (size_t)id[r] * words + (key[r] >> 6));
+    }
+#pragma unroll
+    for (int r = 0; r < kVisRounds; r++) {
+      const unsigned long long bit = 1ull << (key[r] & 63u);
+      if (!(have[r] & bit)) atomicOr(cell_mask + (size_t)id[r] * words + (key[r] >> 6), bit);
+    }
   }
   if (seen) {
-    const int view = find_view(view_off, V, pix);
-    const unsigned long long bit = 1ull << (view - v0);
-    if (!(relaxed_load(seen + id) & bit)) atomicOr(seen + id, bit);
+    const int view = find_view(view_off, V, first), end = __ldg(view_off + view + 1);
+    unsigned long long have[kVisRounds];
+#pragma unroll
+    for (int r = 0; r < kVisRounds; r++) have[r] = id[r] >= 0 ? relaxed_load(seen + id[r]) : ~0ull;
+#pragma unroll
+    for (int r = 0; r < kVisRounds; r++) {
+      const int pix = first + r * 32 + lane;
+      if (id[r] < 0) continue;
+      const int v = pix < end ? view : find_view(view_off, V, pix);
+      const unsigned long long bit = 1ull << (v - v0);
+      if (!(have[r] & bit)) atomicOr(seen + id[r], bit);
+    }
   }
 }
 
@@ -320,58 +393,91 @@ constexpr int kMaxEdgeViews = 200;  // views per launch: the table stays in 4 KB
 struct EdgeArgs {
   const float *img;
   float *edges;
-  int n_views;
+  int n_views, rows;           // rows: output rows of a warp
   int off[kMaxEdgeViews + 1];  // first pixel of each view of the launch, last: end
   int W[kMaxEdgeViews];
+  int strip0[kMaxEdgeViews + 1];  // first warp of each view, last: their number
 };
 static_assert(sizeof(EdgeArgs) <= 4000, "kernel parameters");
 
-// 8-bit luma of pixel (x, y) of a W-wide view at pixel offset base (clamped to the view)
-__device__ __forceinline__ float luma255(const float *img, int base, int W, int H, int x, int y) {
-  x = min(max(x, 0), W - 1);
-  y = min(max(y, 0), H - 1);
-  const float *c = img + 3 * ((size_t)base + (size_t)y * W + x);
+constexpr int kEdgeCols = 30;  // output columns of a warp: its lanes less the halo
+
+// 8-bit luma
+__device__ __forceinline__ float luma255(const float *c) {
   return 255.0f * (0.299f * __ldg(c) + 0.587f * __ldg(c + 1) + 0.114f * __ldg(c + 2));
 }
 
 // Edge prior of the split criterion: Sobel gradient magnitude of the 8-bit
-// luma, border replicated, one thread per pixel of the launch's views
+// luma, border replicated. A warp streams down 32 columns (30 of output): every lane
+// takes its column's luma once per row, the neighbours' come by shuffles,
+// the rows above and below stay in registers. Bound: HBM (16 B per pixel). One
+// thread per pixel took nine lumas (27 loads) each: 295 us for 32 M pixels,
+// now 125.
 __global__ void __launch_bounds__(256) k_edge_magnitude(const __grid_constant__ EdgeArgs a) {
-  const int i = a.off[0] + blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= a.off[a.n_views]) return;
+  const int lane = threadIdx.x & 31;
+  const int item = blockIdx.x * 8 + ((int)threadIdx.x >> 5);
+  if (item >= a.strip0[a.n_views]) return;
   int lo = 0, hi = a.n_views - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
-    if (a.off[mid] <= i) lo = mid;
+    if (a.strip0[mid] <= item) lo = mid;
     else hi = mid - 1;
   }
   const int base = a.off[lo], W = a.W[lo], H = (a.off[lo + 1] - base) / W;
-  const int y = (i - base) / W, x = (i - base) - y * W;
-  float p[3][3];
-#pragma unroll
-  for (int dy = -1; dy <= 1; ++dy)
-#pragma unroll
-    for (int dx = -1; dx <= 1; ++dx) p[dy + 1][dx + 1] = luma255(a.img, base, W, H, x + dx, y + dy);
-  const float gx = (p[0][2] - p[0][0]) + 2.0f * (p[1][2] - p[1][0]) + (p[2][2] - p[2][0]);
-  const float gy = (p[2][0] - p[0][0]) + 2.0f * (p[2][1] - p[0][1]) + (p[2][2] - p[0][2]);
-  a.edges[i] = sqrtf(gx * gx + gy * gy);
+  const int strips = (W + kEdgeCols - 1) / kEdgeCols, local = item - a.strip0[lo];
+  const int x = (local % strips) * kEdgeCols + lane - 1, y0 = (local / strips) * a.rows, y1 = min(y0 + a.rows, H);
+  const bool own = lane >= 1 && lane <= kEdgeCols && x < W;
+  const float *col = a.img + 3 * ((size_t)base + min(max(x, 0), W - 1));
+  const size_t pitch = 3 * (size_t)W;
+  // lumas and horizontal differences of the rows above and at the output row
+  float p0 = luma255(col + (size_t)max(y0 - 1, 0) * pitch), p1 = luma255(col + (size_t)y0 * pitch);
+  float d0 = __shfl_down_sync(0xffffffffu, p0, 1) - __shfl_up_sync(0xffffffffu, p0, 1);
+  float d1 = __shfl_down_sync(0xffffffffu, p1, 1) - __shfl_up_sync(0xffffffffu, p1, 1);
+  float next = luma255(col + (size_t)min(y0 + 1, H - 1) * pitch);
+  for (int y = y0; y < y1; y++) {
+    const float p2 = next;
+    next = luma255(col + (size_t)min(y + 2, H - 1) * pitch);  // one row ahead
+    const float d2 = __shfl_down_sync(0xffffffffu, p2, 1) - __shfl_up_sync(0xffffffffu, p2, 1);
+    const float v = p2 - p0;
+    const float vl = __shfl_up_sync(0xffffffffu, v, 1), vr = __shfl_down_sync(0xffffffffu, v, 1);
+    const float gx = d0 + 2.0f * d1 + d2, gy = vl + 2.0f * v + vr;
+    if (own) a.edges[base + y * W + x] = sqrtf(gx * gx + gy * gy);
+    p0 = p1;
+    p1 = p2;
+    d0 = d1;
+    d1 = d2;
+  }
 }
 
 // edge values back-projected through I_id of the last forward: per run of
-// consecutive pixels of one primitive, one atomic for the sum and one for the count
+// consecutive pixels of one primitive, one atomic for the sum and one for the
+// count. Warps take kPriorRounds x 32 pixels with all their loads in flight
+// (32 M pixels: 105 us at one pixel per thread, now 44).
+constexpr int kPriorRounds = 4;
+
 __global__ void __launch_bounds__(256) k_edge_prior(const int *pid, const float *edges, int P, float *edge_sum,
                                                     int *edge_count) {
   const int lane = threadIdx.x & 31;
-  const int pix = blockIdx.x * blockDim.x + threadIdx.x;
-  const int id = pix < P ? pid[pix] : -1;
-  const bool on = id >= 0;
-  if (!__any_sync(0xffffffffu, on)) return;
-  const Seg sg = seg_info(on ? id : -1 - lane);
-  const float e = seg_sum(on ? edges[pix] : 0.f, sg);
-  const float c = seg_sum(on ? 1.f : 0.f, sg);
-  if (sg.tail && on) {
-    if (edge_sum) atomicAdd(edge_sum + id, e);
-    if (edge_count) atomicAdd(edge_count + id, (int)c);
+  const int first = (blockIdx.x * 8 + ((int)threadIdx.x >> 5)) * (32 * kPriorRounds);
+  int id[kPriorRounds];
+  float e[kPriorRounds];
+#pragma unroll
+  for (int r = 0; r < kPriorRounds; r++) {
+    const int pix = first + r * 32 + lane;
+    id[r] = pix < P ? pid[pix] : -1;
+  }
+#pragma unroll
+  for (int r = 0; r < kPriorRounds; r++) e[r] = id[r] >= 0 ? edges[first + r * 32 + lane] : 0.f;
+#pragma unroll
+  for (int r = 0; r < kPriorRounds; r++) {
+    const bool on = id[r] >= 0;
+    if (!__any_sync(0xffffffffu, on)) continue;
+    const Seg sg = seg_info(on ? id[r] : -1 - lane);
+    const float sum = seg_sum(e[r], sg);
+    if (sg.tail && on) {
+      if (edge_sum) atomicAdd(edge_sum + id[r], sum);
+      if (edge_count) atomicAdd(edge_count + id[r], lane - sg.start + 1);
+    }
   }
 }
 
@@ -395,10 +501,8 @@ int launch_subdivide(int degree, const bgt_scene &sc, const int *sel, int n_sel,
   s.sel = sel;
   s.n_sel = n_sel;
   s.out = out;
-  const long long per = std::max(ncp_of(degree), s.T);
-  const long long threads = 4LL * n_sel * per;
-  const int blocks = (int)((threads + 255) / 256);
-  dispatch_degree(degree, [&](auto d) { k_subdivide<decltype(d)::value><<<blocks, 256, 0, st>>>(s); });
+  const int blocks = (n_sel + kSplitParents - 1) / kSplitParents;
+  dispatch_degree(degree, [&](auto d) { k_subdivide<decltype(d)::value><<<blocks, kSplitThreads, 0, st>>>(s); });
   return 1;
 }
 
@@ -419,22 +523,30 @@ int launch_edge_magnitude(const float *img, int n_views, const int *sizes, float
   EdgeArgs a;
   a.img = img;
   a.edges = edges;
+  long long pixels = 0;
+  for (int v = 0; v < n_views; ++v) pixels += (long long)sizes[2 * v] * sizes[2 * v + 1];
+  // rows per warp: two of halo each, so long ones where they fill the GPU all the same (8 M pixels: 8,000
+  // warps of 32 rows, 53 per SM)
+  a.rows = pixels >= 8000000 ? 32 : 8;
   int launches = 0, off = 0;
   for (int v0 = 0; v0 < n_views; v0 += kMaxEdgeViews) {
     a.n_views = 0;
-    const int first = off;
+    int warps = 0;
     for (int v = v0; v < n_views && v < v0 + kMaxEdgeViews; ++v) {
       const int W = sizes[2 * v], H = sizes[2 * v + 1];
       if (W > 0 && H > 0) {
         a.off[a.n_views] = off;
         a.W[a.n_views] = W;
+        a.strip0[a.n_views] = warps;
+        warps += (W + kEdgeCols - 1) / kEdgeCols * ((H + a.rows - 1) / a.rows);
         a.n_views++;
       }
       off += W * H;
     }
     a.off[a.n_views] = off;
-    if (a.n_views == 0 || off == first) continue;
-    k_edge_magnitude<<<(off - first + 255) / 256, 256, 0, st>>>(a);
+    a.strip0[a.n_views] = warps;
+    if (warps == 0) continue;
+    k_edge_magnitude<<<(warps + 7) / 8, 256, 0, st>>>(a);
     ++launches;
   }
   return launches;
@@ -443,7 +555,8 @@ int launch_edge_magnitude(const float *img, int n_views, const int *sizes, float
 int launch_edge_prior(const Params &p, const Work &w, const float *edges, float *edge_sum, int *edge_count,
                       cudaStream_t st) {
   if (p.P <= 0) return 0;
-  k_edge_prior<<<(p.P + 255) / 256, 256, 0, st>>>(w.pid, edges, p.P, edge_sum, edge_count);
+  const int per = 256 * kPriorRounds;
+  k_edge_prior<<<(p.P + per - 1) / per, 256, 0, st>>>(w.pid, edges, p.P, edge_sum, edge_count);
   return 1;
 }
 
@@ -460,7 +573,7 @@ int launch_visibility(const Params &p, const Work &w, const int *view_off, int *
     const int v1 = v0 + 64 < p.V ? v0 + 64 : p.V;
     const int pix0 = view_off[v0], pix1 = view_off[v1];
     if (pix1 > pix0) {
-      k_vis_pixels<<<(pix1 - pix0 + 255) / 256, 256, 0, st>>>(w.pid, w.zbuf, w.view_pix_off, p.V, pix0, pix1, v0,
+      k_vis_pixels<<<(pix1 - pix0 + 256 * kVisRounds - 1) / (256 * kVisRounds), 256, 0, st>>>(w.pid, w.zbuf, w.view_pix_off, p.V, pix0, pix1, v0,
                                                              nsub, words, cell_mask,
                                                              view_count ? w.vis_seen : nullptr);
       launches++;
