@@ -93,7 +93,7 @@ void carve(bgt_handle *h, char *base, size_t *total) {
   const long long id_blocks = (P + bgt::kIdPixels - 1) / bgt::kIdPixels;
   w.pix_mask = c.take<uint2>(id_blocks * (bgt::kIdPixels / 32));
   w.blk_off = c.take<int2>(id_blocks);
-  w.counters = c.take<int>(16);
+  w.counters = c.take<int>(bgt::kCounters);
   w.stats = c.take<unsigned long long>(8);
   w.status = c.take<int>(1);
   w.gA = c.take<float4>(F);
@@ -122,6 +122,7 @@ void carve(bgt_handle *h, char *base, size_t *total) {
   w.b_tstart = c.take<long long>(T + 1);
   w.b_tfill = c.take<int>(T + 1);
   w.big_list = c.take<int>(2 * (long long)T + 2);
+  w.tile_order = c.take<int>(bgt::kTileClasses * (long long)T);
   w.tile_desc = c.take<int4>(2 * (long long)T + 2);
   // headers 3/4 of the capacity, fill units 1/64 (fills are per primitive-cache miss: ~1 in 13
   // headers on the 64-view scene, ~1 in 200 on dense tiles)
@@ -398,7 +399,7 @@ bgt_status bgt_create(const bgt_config *cfg, bgt_handle **out) {
   if (e == cudaSuccess) e = cudaMallocHost(&h->h_status, sizeof(int) * 16);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->staged, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaMemset(h->w.status, 0, sizeof(int));
-  if (e == cudaSuccess) e = cudaMemset(h->w.counters, 0, 16 * sizeof(int));
+  if (e == cudaSuccess) e = cudaMemset(h->w.counters, 0, bgt::kCounters * sizeof(int));
   if (e == cudaSuccess) e = bgt::configure_composite();
   if (e == cudaSuccess) e = bgt::configure_binning();
   if (e != cudaSuccess) {
@@ -911,7 +912,7 @@ bgt_status bgt_bin_sort(bgt_handle *h, int width, int height, int count, const i
   cudaMemsetAsync(w.g_tfill, 0, tb, st);
   cudaMemsetAsync(w.b_tcount, 0, tb, st);
   cudaMemsetAsync(w.b_tfill, 0, tb, st);
-  cudaMemsetAsync(w.counters, 0, 16 * sizeof(int), st);
+  cudaMemsetAsync(w.counters, 0, bgt::kCounters * sizeof(int), st);
   if (count > 0)
     k_load_gaussians<<<(count + 255) / 256, 256, 0, st>>>(p, w, count, qxy, off, conic, opacity, depth);
   cudaMemcpyAsync(w.counters + bgt::kF, &count, sizeof(int), cudaMemcpyHostToDevice, st);

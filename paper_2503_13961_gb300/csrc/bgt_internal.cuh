@@ -30,6 +30,10 @@ constexpr int kStatusNonFinite = 8;
 constexpr int kStatusBadPrim = 16;
 constexpr int kStatusBlendOverflow = 32;  // reserved (blend-record overflow falls back to a tile-list walk)
 
+// classes of tiles by the length of their Gaussian list, in which the blending
+// kernels take them: 0 empty, then below 128, 384, 768 entries, and longer ones
+constexpr int kTileClasses = 5;
+
 // blend records (forward -> backward): headers in chunks of kRecChunk per warp
 // block, fill records in chunks of kFillChunk per warp
 constexpr int kRecChunk = 32;
@@ -113,7 +117,7 @@ struct Work {
   uint2 *pix_mask;            // [P / 32] foreground and boundary bits of 32 consecutive pixels
   int2 *blk_off;              // [P / kIdPixels] foreground / boundary pixels of each block of k_ids, then
                               // their exclusive prefix sums
-  int *counters;              // [16] F, Nb, K, Kb, queue heads...
+  int *counters;              // [kCounters] F, Nb, K, Kb, queue heads, tiles per class...
   int *status;                // [1]
   // per primitive
   // gaussians
@@ -138,6 +142,7 @@ struct Work {
   int *b_tcount, *b_tfill;
   long long *g_tstart, *b_tstart;  // [tiles + 1] exclusive prefix sums (64-bit: no wrap)
   int *big_list;              // [2 tiles] segments too long for one warp to sort
+  int *tile_order;            // [kTileClasses][tiles] tiles by class (see kTileClasses), counters[kTileClass + c] of them
   int4 *tile_desc;            // [2 tiles] (view, x0 | y0 << 16, W | H << 16, view pixel offset),
                               // (Gaussian list start, length, boundary list start, length)
   // Blend records written by the forward pass for the backward pass. A fill
@@ -190,7 +195,9 @@ constexpr int kIndexBits = 27;  // Gaussian index field of a pair key (<= 134M G
 constexpr unsigned long long kIndexMask = (1ull << kIndexBits) - 1ull;
 
 enum Counter { kF = 0, kNb = 1, kK = 2, kKb = 3, kQueueFwd = 4, kQueueBwd = 5, kQueueSort = 6, kBigCount = 7,
-               kRecChunks = 8, kFillChunks = 9, kWalkCount = 10, kQueueWalk = 11, kIdsDone = 12 };
+               kRecChunks = 8, kFillChunks = 9, kWalkCount = 10, kQueueWalk = 11, kIdsDone = 12,
+               kQueueEmpty = 13, kTileClass = 16 };
+constexpr int kCounters = 24;
 
 // ---------------------------------------------------------------------------
 // small helpers

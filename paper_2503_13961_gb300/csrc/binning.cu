@@ -629,6 +629,17 @@ __global__ void __launch_bounds__(kSortThreads, 6) k_tile_sort(Params p, Work w,
       if (bnd ? b_over : g_over) s1 = s0;  // unwritten slots: nothing to sort
     }
     const int n_lane = (int)(s1 - s0);
+    // the tile into its class's list (a list that overflowed counts as empty)
+    const int cls = lane < grab && item < p.tiles ? (n_lane > 0) + (n_lane >= 128) + (n_lane >= 384) + (n_lane >= 768) : -1;
+#pragma unroll
+    for (int c = 0; c < kTileClasses; c++) {
+      const unsigned m = __ballot_sync(0xffffffffu, cls == c);
+      if (!m) continue;
+      int at = 0;
+      if (lane == 0) at = atomicAdd(w.counters + kTileClass + c, __popc(m));
+      at = __shfl_sync(0xffffffffu, at, 0);
+      if (cls == c) w.tile_order[(size_t)c * p.tiles + at + __popc(m & ((1u << lane) - 1u))] = item;
+    }
     if (n_lane > kWarpSortCap) big_list[atomicAdd(w.counters + kBigCount, 1)] = item;
     unsigned todo = __ballot_sync(0xffffffffu, n_lane > 0 && n_lane <= kWarpSortCap);
     while (todo) {

@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(kGenThreads) k_ids(Params p, Scene s, Work w, 
     w.g_tfill[t] = 0;
     w.b_tfill[t] = 0;
   }
-  if (gtid >= kQueueFwd && gtid < kIdsDone) w.counters[gtid] = 0;
+  if (gtid >= kQueueFwd && gtid < kCounters && gtid != kIdsDone) w.counters[gtid] = 0;
   if (p.attr_res == 1)
     for (int m = gtid; m < p.M; m += gthreads) prim_cov(s, w, m);
   if (blockIdx.x < npb) {
