@@ -26,10 +26,9 @@ struct bgt_handle {
   void *arena = nullptr;
   size_t arena_bytes = 0;
   bgt::Work w{};
+  // the call's views, their pixel offsets and their tile offsets, one after the other: one upload per call
   View *d_views = nullptr;
-  int *d_offs = nullptr;
   View *h_views = nullptr;  // pinned staging
-  int *h_offs = nullptr;    // pinned staging
   int *h_status = nullptr;  // pinned
   cudaEvent_t staged = nullptr;
   int tile = 16;
@@ -66,6 +65,9 @@ bgt_status cuda_fail(bgt_handle *h, cudaError_t e, const char *where) {
 
 size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
 
+// bytes of n views with their pixel and tile offsets (n + 1 each)
+size_t view_bytes(int n) { return sizeof(View) * (size_t)n + 2 * sizeof(int) * ((size_t)n + 1); }
+
 struct Carver {
   char *base;
   size_t off = 0;
@@ -82,8 +84,7 @@ void carve(bgt_handle *h, char *base, size_t *total) {
   bgt::Work &w = h->w;
   const long long P = h->Pcap, F = h->Fcap, K = h->Kcap, Kb = h->Kbcap;
   const int T = h->Tcap;
-  h->d_views = c.take<View>(h->Vcap);
-  h->d_offs = c.take<int>(2 * (h->Vcap + 1));
+  h->d_views = reinterpret_cast<View *>(c.take<char>((long long)view_bytes(h->Vcap)));
   w.zbuf = c.take<unsigned long long>(P);
   w.pid = c.take<int>(P);
   w.vis_seen = c.take<unsigned long long>(h->Mcap);
@@ -149,8 +150,6 @@ void carve(bgt_handle *h, char *base, size_t *total) {
   w.pb_rec = c.take<float4>(2 * F);
   w.Fcap = F;
   w.views = h->d_views;
-  w.view_pix_off = h->d_offs;
-  w.view_tile_off = h->d_offs + (h->Vcap + 1);
   *total = c.off;
 }
 
@@ -186,6 +185,7 @@ bgt_status setup_call(bgt_handle *h, const bgt_scene *sc, const bgt_camera *cams
   cudaError_t e = cudaEventSynchronize(h->staged);  // previous upload has left the staging buffer
   if (e != cudaSuccess) return cuda_fail(h, e, "cudaEventSynchronize");
   long long P = 0, tiles = 0;
+  int *pix_off = reinterpret_cast<int *>(h->h_views + n), *tile_off = pix_off + n + 1;
   for (int v = 0; v < n; v++) {
     const bgt_camera &c = cams[v];
     if (c.width < 1 || c.height < 1 || c.width > 32768 || c.height > 32768)
@@ -204,20 +204,18 @@ bgt_status setup_call(bgt_handle *h, const bgt_scene *sc, const bgt_camera *cams
     vw.tiles_y = (c.height + t - 1) / t;
     vw.pix_off = (int)P;
     vw.tile_off = (int)tiles;
-    h->h_offs[v] = (int)P;
-    h->h_offs[h->Vcap + 1 + v] = (int)tiles;
+    pix_off[v] = (int)P;
+    tile_off[v] = (int)tiles;
     P += (long long)c.width * c.height;
     tiles += (long long)vw.tiles_x * vw.tiles_y;
     if (P > h->Pcap) return fail(h, BGT_ERR_CAPACITY, "total pixels exceed max_pixels");
     if (tiles > h->Tcap) return fail(h, BGT_ERR_CAPACITY, "total tiles exceed capacity");
   }
-  h->h_offs[n] = (int)P;
-  h->h_offs[h->Vcap + 1 + n] = (int)tiles;
-  e = cudaMemcpyAsync(h->d_views, h->h_views, sizeof(View) * n, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(h->d_offs, h->h_offs, sizeof(int) * (n + 1), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(h->d_offs + h->Vcap + 1, h->h_offs + h->Vcap + 1, sizeof(int) * (n + 1),
-                        cudaMemcpyHostToDevice, st);
+  pix_off[n] = (int)P;
+  tile_off[n] = (int)tiles;
+  h->w.view_pix_off = reinterpret_cast<const int *>(h->d_views + n);
+  h->w.view_tile_off = h->w.view_pix_off + n + 1;
+  e = cudaMemcpyAsync(h->d_views, h->h_views, view_bytes(n), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaEventRecord(h->staged, st);
   if (e != cudaSuccess) return cuda_fail(h, e, "view upload");
   const bgt_config &c = h->cfg;
@@ -394,8 +392,7 @@ bgt_status bgt_create(const bgt_config *cfg, bgt_handle **out) {
   }
   h->arena_bytes = total;
   carve(h, static_cast<char *>(h->arena), &total);
-  e = cudaMallocHost(&h->h_views, sizeof(View) * h->Vcap);
-  if (e == cudaSuccess) e = cudaMallocHost(&h->h_offs, sizeof(int) * 2 * (h->Vcap + 1));
+  e = cudaMallocHost(&h->h_views, view_bytes(h->Vcap));
   if (e == cudaSuccess) e = cudaMallocHost(&h->h_status, sizeof(int) * 16);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->staged, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaMemset(h->w.status, 0, sizeof(int));
@@ -419,7 +416,6 @@ void bgt_destroy(bgt_handle *h) {
   if (h->g_bwd) cudaGraphExecDestroy(h->g_bwd);
   if (h->staged) cudaEventDestroy(h->staged);
   if (h->h_views) cudaFreeHost(h->h_views);
-  if (h->h_offs) cudaFreeHost(h->h_offs);
   if (h->h_status) cudaFreeHost(h->h_status);
   if (h->arena) cudaFree(h->arena);
   delete h;

@@ -144,6 +144,7 @@ __device__ inline longlong2 scan_both(const int *in0, long long *out0, const int
 template <int CL>
 __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(kScanThreads)
     k_scan_pair(int *in0, long long *out0, int *in1, long long *out1, int n, bool clear) {
+  chained();
   scan_both<CL>(in0, out0, in1, out1, n);
   if (!clear) return;
   // every count of the block's range was last read before its last block barrier, but for the final chunk's
@@ -157,6 +158,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(kScanThreads)
 // capacity check, by the block that holds the last tile
 template <int CL>
 __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(kScanThreads) k_tile_scan(Params p, Work w) {
+  chained();
   const longlong2 total = scan_both<CL>(w.g_tcount, w.g_tstart, w.b_tcount, w.b_tstart, p.tiles);
   const int chunks = (p.tiles + kScanChunk - 1) / kScanChunk, per = (chunks + CL - 1) / CL * kScanChunk;
   if ((int)blockIdx.x == (p.tiles - 1) / per && threadIdx.x == 0) {
@@ -212,6 +214,7 @@ __device__ inline void emit_rect(unsigned long long *keys, int *fill, const long
 // the pair keys, unsorted, into the second halves of the key arrays (the sort
 // writes the first), and the tiles' descriptors
 __global__ void k_emit(Params p, Work w) {
+  chained();
   const int F = w.counters[kF], Nb = w.counters[kNb];
   const int stride = gridDim.x * blockDim.x;
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < p.tiles; t += stride) tile_descriptor(p, w, t);
@@ -611,6 +614,7 @@ __device__ __forceinline__ bool warp_sort_segment(const Work &w, const unsigned 
 // words with up to 32 per lane 21 us and 0.58 ms, with the runs of 16 per lane
 // and the merge 20 us and 0.48 ms.
 __global__ void __launch_bounds__(kSortThreads, 6) k_tile_sort(Params p, Work w, int *big_list, int grab) {
+  chained();
   __shared__ unsigned s_sort[2 * kSortWarps * kWarpWords];
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   const bool g_over = w.g_tstart[p.tiles] > p.max_pairs, b_over = w.b_tstart[p.tiles] > p.max_bpairs;
@@ -771,6 +775,7 @@ __device__ __forceinline__ bool block_sort_words(const Work &w, const unsigned l
 // a bitonic network of the block over 64-bit keys in shared memory took 1.62
 // ms, quarters sorted by the warps and merged on 32-bit words 0.78 ms.
 __global__ void __launch_bounds__(kSortThreads, 4) k_tile_sort_big(Params p, Work w, const int *big_list) {
+  chained();
   extern __shared__ __align__(16) unsigned long long s_keys[];
   __shared__ KeyRange s_range[kSortWarps];
   const int nbig = w.counters[kBigCount];
@@ -801,9 +806,10 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_tile_sort_big(Params p, Wor
 
 }  // namespace
 
-int launch_scan_pair(int *in0, long long *out0, int *in1, long long *out1, int n, bool clear, cudaStream_t st) {
-  if (n <= kScanOne) k_scan_pair<1><<<1, kScanThreads, 0, st>>>(in0, out0, in1, out1, n, clear);
-  else k_scan_pair<kScanCluster><<<kScanCluster, kScanThreads, 0, st>>>(in0, out0, in1, out1, n, clear);
+int launch_scan_pair(int *in0, long long *out0, int *in1, long long *out1, int n, bool clear, bool overlap,
+                     cudaStream_t st) {
+  if (n <= kScanOne) chain_launch(overlap, k_scan_pair<1>, 1, kScanThreads, 0, st, in0, out0, in1, out1, n, clear);
+  else chain_launch(overlap, k_scan_pair<kScanCluster>, kScanCluster, kScanThreads, 0, st, in0, out0, in1, out1, n, clear);
   return 1;
 }
 
@@ -813,14 +819,14 @@ cudaError_t configure_binning() {
 
 int launch_binning(const Params &p, const Work &w, cudaStream_t st) {
   if (p.tiles <= 0) return 0;
-  if (p.tiles <= kScanOne) k_tile_scan<1><<<1, kScanThreads, 0, st>>>(p, w);
-  else k_tile_scan<kScanCluster><<<kScanCluster, kScanThreads, 0, st>>>(p, w);
-  k_emit<<<16 * 152, 256, 0, st>>>(p, w);
+  if (p.tiles <= kScanOne) chain_launch(p.P <= kOverlapPixels, k_tile_scan<1>, 1, kScanThreads, 0, st, p, w);
+  else chain_launch(p.P <= kOverlapPixels, k_tile_scan<kScanCluster>, kScanCluster, kScanThreads, 0, st, p, w);
+  chain_launch(p.P <= kOverlapPixels, k_emit, 16 * 152, 256, 0, st, p, w);
   // segments per dequeue: enough dequeues for every resident warp to take a few, so that long segments
   // spread, and few enough that the queue's one counter is no bottleneck
   const int blocks = 6 * 152, grab = std::max(1, std::min(32, 2 * p.tiles / (blocks * kSortWarps * 4)));
-  k_tile_sort<<<blocks, kSortThreads, 0, st>>>(p, w, w.big_list, grab);
-  k_tile_sort_big<<<4 * 152, kSortThreads, kSortBigSmem, st>>>(p, w, w.big_list);
+  chain_launch(p.P <= kOverlapPixels, k_tile_sort, blocks, kSortThreads, 0, st, p, w, w.big_list, grab);
+  chain_launch(p.P <= kOverlapPixels, k_tile_sort_big, 4 * 152, kSortThreads, kSortBigSmem, st, p, w, w.big_list);
   return 4;
 }
 

@@ -243,6 +243,7 @@ __device__ __forceinline__ void chain_gauss(const Params &p, const Scene &s, con
 // the control points with the Bernstein weights (Eq. 3).
 template <int N>
 __global__ void __launch_bounds__(256) k_chain_sh(Params p, Scene s, Work w, Grads out) {
+  chained();
   __shared__ float s_rows[kChainWarps][32 * ((3 * SurfPoint<N>::M) | 1)];
   float *sw = s_rows[threadIdx.x >> 5];
   const int F = w.counters[kF];
@@ -351,6 +352,7 @@ __device__ __forceinline__ void chain_bnd(const Params &p, const Scene &s, const
 // in one launch: the boundary points fill in where the Gaussians run out
 template <int N>
 __global__ void __launch_bounds__(256) k_chain(Params p, Scene s, Work w, Grads out) {
+  chained();
   __shared__ View s_views[kStagedViews];
   const int F = w.counters[kF], Nb = w.counters[kNb];
   const int ng = (F + 31) >> 5, groups = ng + ((Nb + 31) >> 5);
@@ -381,6 +383,7 @@ __device__ __forceinline__ void clear_floats(float *p, long long n) {
 // (nine or more memsets, 2-3 us each in the serial chain of a small call). With maps
 // of leg resolution 1 the map gradients are written whole at the end.
 __global__ void __launch_bounds__(256) k_clear_grads(Params p, Work w, Grads g) {
+  chained();
   const long long M = p.M;
   clear_floats(g.ctrl, M * p.ncp * 3);
   clear_floats(g.color, M * p.ncp * 3);
@@ -430,6 +433,7 @@ __device__ __forceinline__ SumChunks sum_chunks(int F, int Nb) {
 // run's sum with one atomic when the primitive changes and at the chunk's end.
 template <int N>
 __global__ void __launch_bounds__(256, 3) k_prim_sum_rows(Work w, Grads out, int with_cov) {
+  chained();
   constexpr int m = SurfPoint<N>::M;
   constexpr int RS = (kSumCols + m) | 1;  // row stride (odd: conflict-free row writes)
   constexpr int NO = 6 * m + 8;           // outputs
@@ -579,6 +583,7 @@ __global__ void __launch_bounds__(256, 3) k_prim_sum_rows(Work w, Grads out, int
 // per round (~8 instructions per record).
 template <int N>
 __global__ void __launch_bounds__(256, 2) k_prim_sum_regs(Work w, Grads out) {
+  chained();
   constexpr int m = SurfPoint<N>::M;
   constexpr int NO = 6 * m + 8;
   static_assert(NO <= 64, "outputs beyond two per lane");
@@ -691,6 +696,7 @@ __device__ __forceinline__ float l1_sign(float diff, float scale) {
 // values per thread and load when the three arrays are 16-byte aligned (vec)
 __global__ void k_l1_grad(const float *img, const float *tgt, long long n, float scale, float *d, float *loss,
                           int vec) {
+  chained();
   float acc = 0.f;
   const long long stride = (long long)gridDim.x * blockDim.x;
   const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -722,6 +728,7 @@ __global__ void k_l1_grad(const float *img, const float *tgt, long long n, float
 // taken to its one rotation and scaling texel (linear in dl/dSigma3D, so the
 // sum of the per-Gaussian terms)
 __global__ void k_prim_attr_grad(Params p, Scene s, Work w, Grads out) {
+  chained();
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= p.M) return;
   const float *gc = w.prim_gcov + 6 * (size_t)m;
@@ -751,35 +758,32 @@ constexpr long long kSumRegsFrom = 160;  // pixels per primitive
 
 int launch_clear_grads(const Params &p, const Work &w, const Grads &g, cudaStream_t st) {
   const long long most = std::max(1ll, (long long)p.M * (3 * p.ncp + 3 * p.sh_k));  // floats, about
-  k_clear_grads<<<(int)std::min(most / 1024 + 1, 152ll * 8), 256, 0, st>>>(p, w, g);
+  chain_launch(p.P <= kOverlapPixels, k_clear_grads, (int)std::min(most / 1024 + 1, 152ll * 8), 256, 0, st, p, w, g);
   return 1;
 }
 
 int launch_chain(const Params &p, const Scene &s, const Work &w, const Grads &g, cudaStream_t st) {
-  int sms = 0, dev = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (sms <= 0) sms = 152;
+  const int sms = num_sms();
   const int grid = sms * p.chain_bps;
   int k = 0;
   const int with_cov = p.attr_res == 1 && (g.log_scale || g.quat);
   if (p.M == 0) return 0;
   // segments of the per-primitive records from their counts (taken by the blending backward)
-  k += launch_scan_pair(w.prim_gcnt, w.prim_gseg, w.prim_bcnt, w.prim_bseg, p.M, true, st);
+  k += launch_scan_pair(w.prim_gcnt, w.prim_gseg, w.prim_bcnt, w.prim_bseg, p.M, true, p.P <= kOverlapPixels, st);
   dispatch_degree(p.n, [&](auto d) {
     constexpr int N = decltype(d)::value;
-    k_chain<N><<<grid, 256, 0, st>>>(p, s, w, g);
+    chain_launch(p.P <= kOverlapPixels, k_chain<N>, grid, 256, 0, st, p, s, w, g);
     bool regs = false;
     if constexpr (SurfPoint<N>::M <= 6) {
       regs = p.P > kSumRegsFrom * (long long)p.M;
-      if (regs) k_prim_sum_regs<N><<<sms * 2, 256, 0, st>>>(w, g);
+      if (regs) chain_launch(p.P <= kOverlapPixels, k_prim_sum_regs<N>, sms * 2, 256, 0, st, w, g);
     }
-    if (!regs) k_prim_sum_rows<N><<<sms * 4, 256, 0, st>>>(w, g, with_cov);
-    if (p.sh_deg > 0) k_chain_sh<N><<<grid, 256, 0, st>>>(p, s, w, g);
+    if (!regs) chain_launch(p.P <= kOverlapPixels, k_prim_sum_rows<N>, sms * 4, 256, 0, st, w, g, with_cov);
+    if (p.sh_deg > 0) chain_launch(p.P <= kOverlapPixels, k_chain_sh<N>, grid, 256, 0, st, p, s, w, g);
   });
   k += p.sh_deg > 0 ? 3 : 2;
   if (with_cov) {
-    k_prim_attr_grad<<<(p.M + 255) / 256, 256, 0, st>>>(p, s, w, g);
+    chain_launch(p.P <= kOverlapPixels, k_prim_attr_grad, (p.M + 255) / 256, 256, 0, st, p, s, w, g);
     k++;
   }
   return k;
@@ -793,7 +797,7 @@ int launch_l1_grad(const float *img, const float *target, long long n, float sca
   long long blocks = ((vec ? n / 4 : n) + 255) / 256;
   if (blocks > 152 * 16) blocks = 152 * 16;
   if (blocks < 1) blocks = 1;
-  k_l1_grad<<<(int)blocks, 256, 0, st>>>(img, target, n, scale, dimg, loss, vec);
+  chain_launch(n <= 3 * kOverlapPixels, k_l1_grad, (int)blocks, 256, 0, st, img, target, n, scale, dimg, loss, vec);
   return 1;
 }
 

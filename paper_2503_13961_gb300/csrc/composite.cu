@@ -441,6 +441,7 @@ struct RecWriter {
 // launched only when profiling, so the production kernel carries no counters)
 template <int T, bool STATS>
 __global__ void __launch_bounds__(TileCfg<T>::NT, TileCfg<T>::MINB_FWD) k_composite_fwd(Params p, Work w, float *image) {
+  chained();
   using Cfg = TileCfg<T>;
   constexpr int NT = Cfg::NT, PPT = Cfg::PPT, S = Cfg::SLOTS_FWD;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -743,6 +744,7 @@ __device__ __forceinline__ float w_from_candidate(const float4 *brec, int bi, fl
 // primitive) in a cache slot and flushed on eviction and at the block's end.
 template <int T, bool STATS>
 __global__ void __launch_bounds__(TileCfg<T>::NT, TileCfg<T>::MINB_BWD) k_composite_bwd(Params p, Work w, const float *dimage) {
+  chained();
   using Cfg = TileCfg<T>;
   constexpr int PPT = Cfg::PPT, S = Cfg::SLOTS_BWD, NW = Cfg::NW;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -979,6 +981,7 @@ __device__ __forceinline__ void count_prim_records(const Work &w) {
 // of the pair's search).
 template <int T>
 __global__ void __launch_bounds__(TileCfg<T>::NT) k_composite_bwd_walk(Params p, Work w, const float *dimage) {
+  chained();
   using Cfg = TileCfg<T>;
   constexpr int PPT = Cfg::PPT, NW = Cfg::NW;
   constexpr int kWalkSlots = PPT == 1 ? 8 : 2;  // primitive cache slots per warp (static shared memory)
@@ -1122,8 +1125,8 @@ template <int T>
 int launch_fwd_t(const Params &p, const Work &w, float *image, cudaStream_t st, int sms) {
   const int grid = std::min(p.tiles, sms * TileCfg<T>::RES_FWD);
   if (grid > 0) {
-    if (p.stats) k_composite_fwd<T, true><<<grid, TileCfg<T>::NT, sizeof(FwdShared<T>), st>>>(p, w, image);
-    else k_composite_fwd<T, false><<<grid, TileCfg<T>::NT, sizeof(FwdShared<T>), st>>>(p, w, image);
+    if (p.stats) chain_launch(p.P <= kOverlapPixels, k_composite_fwd<T, true>, grid, TileCfg<T>::NT, sizeof(FwdShared<T>), st, p, w, image);
+    else chain_launch(p.P <= kOverlapPixels, k_composite_fwd<T, false>, grid, TileCfg<T>::NT, sizeof(FwdShared<T>), st, p, w, image);
   }
   return grid > 0 ? 1 : 0;
 }
@@ -1132,10 +1135,10 @@ template <int T>
 int launch_bwd_t(const Params &p, const Work &w, const float *dimage, cudaStream_t st, int sms) {
   const int grid = std::min(p.tiles, sms * TileCfg<T>::RES_BWD);
   if (grid > 0) {
-    if (p.stats) k_composite_bwd<T, true><<<grid, TileCfg<T>::NT, sizeof(BwdShared<T>), st>>>(p, w, dimage);
-    else k_composite_bwd<T, false><<<grid, TileCfg<T>::NT, sizeof(BwdShared<T>), st>>>(p, w, dimage);
+    if (p.stats) chain_launch(p.P <= kOverlapPixels, k_composite_bwd<T, true>, grid, TileCfg<T>::NT, sizeof(BwdShared<T>), st, p, w, dimage);
+    else chain_launch(p.P <= kOverlapPixels, k_composite_bwd<T, false>, grid, TileCfg<T>::NT, sizeof(BwdShared<T>), st, p, w, dimage);
     // the records per primitive, and the warp blocks whose blend records overflowed (none in the common case)
-    k_composite_bwd_walk<T><<<sms * 3, TileCfg<T>::NT, 0, st>>>(p, w, dimage);  // 3 blocks per SM by registers
+    chain_launch(p.P <= kOverlapPixels, k_composite_bwd_walk<T>, sms * 3, TileCfg<T>::NT, 0, st, p, w, dimage);  // 3 blocks per SM by registers
   }
   return grid > 0 ? 2 : 0;
 }
@@ -1154,17 +1157,6 @@ template <int T>
 cudaError_t configure_t() {
   cudaError_t e = configure_ts<T, false>();
   return e == cudaSuccess ? configure_ts<T, true>() : e;
-}
-
-int num_sms() {
-  static int sms = 0;
-  if (!sms) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (sms <= 0) sms = 152;
-  }
-  return sms;
 }
 
 }  // namespace

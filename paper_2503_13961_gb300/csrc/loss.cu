@@ -117,6 +117,7 @@ struct LossArgs {
 static_assert(sizeof(LossArgs) <= 4000, "kernel parameters");
 
 __global__ void __launch_bounds__(kLossThreads, 2) k_l2_dssim_grad(const __grid_constant__ LossArgs a) {
+  chained();
   extern __shared__ float4 sm4[];
   float4 *part = sm4;                                             // [3][kRows][kPartStride] rows of moments / partials
   float2 *ring = reinterpret_cast<float2 *>(sm4 + 3 * kPartPlane);  // [3][kRing][kInStride] (x, y)
@@ -421,9 +422,6 @@ int launch_l2_dssim_grad(const float *img, const float *gt, int n_views, const i
     a.g2[t] = ((unsigned long long)bits << 32) | bits;
   }
   cudaFuncSetAttribute(k_l2_dssim_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, kLossSmem);
-  int sms = 0, dev = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   int launches = 0;
   long long off = 0;
   for (int v0 = 0; v0 < n_views; v0 += kMaxLossViews) {
@@ -444,14 +442,14 @@ int launch_l2_dssim_grad(const float *img, const float *gt, int n_views, const i
       off += npx;
     }
     if (a.n_views == 0) continue;
-    a.seg = loss_segment(a.view, a.n_views, 2 * (sms > 0 ? sms : 152));
+    a.seg = loss_segment(a.view, a.n_views, 2 * num_sms());
     int tiles = 0;
     for (int v = 0; v < a.n_views; ++v) {
       LossView &r = a.view[v];
       r.tile0 = tiles;
       tiles += r.strips * ((r.H + a.seg - 1) / a.seg);
     }
-    k_l2_dssim_grad<<<tiles, kLossThreads, kLossSmem, st>>>(a);
+    chain_launch(off <= kOverlapPixels, k_l2_dssim_grad, tiles, kLossThreads, kLossSmem, st, a);
     ++launches;
   }
   return launches;

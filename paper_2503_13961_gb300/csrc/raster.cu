@@ -22,6 +22,7 @@
 // below 2^30) and in 64-bit ones otherwise. Every operation that decides
 // coverage or the depth order is an explicit IEEE-rounded intrinsic, so the
 // result is reproducible bit for bit.
+#include <algorithm>
 #include <climits>
 
 #include "bgt_internal.cuh"
@@ -128,6 +129,7 @@ __global__ void __launch_bounds__(kRasterWarps * 32, N <= 2 ? 8 : 6) k_raster(Pa
     s_tri[ti] = make_int2(vslot(va[0], vb[0], L) | (vslot(va[1], vb[1], L) << 8) | (vslot(va[2], vb[2], L) << 16), sid);
   }
   __syncthreads();
+  chained();
   // the block row's camera in shared memory, its fields read where used
   // (held in registers it costs spills at the 64-register budget)
   __shared__ View s_view;
@@ -203,10 +205,13 @@ __global__ void __launch_bounds__(kRasterWarps * 32, N <= 2 ? 8 : 6) k_raster(Pa
 
 int launch_raster(const Params &p, const Scene &s, const Work &w, cudaStream_t st) {
   if (p.V == 0 || p.M == 0) return 0;
-  // each warp rasterizes p.raster_prims primitives per block (amortises the tables)
-  const int per_block = kRasterWarps * p.raster_prims;
+  // each warp rasterizes p.raster_prims primitives per block (amortises the tables), fewer where that
+  // leaves SMs without blocks (2,000 primitives in one view: 500 blocks, not 63)
+  const long long warps = 4ll * kRasterWarps * num_sms();
+  const int prims = (int)std::min<long long>(p.raster_prims, std::max<long long>(1, (long long)p.M * p.V / warps));
+  const int per_block = kRasterWarps * prims;
   const dim3 grid((unsigned)((p.M + per_block - 1) / per_block), (unsigned)p.V);
-  dispatch_degree(p.n, [&](auto d) { k_raster<decltype(d)::value><<<grid, kRasterWarps * 32, 0, st>>>(p, s, w); });
+  dispatch_degree(p.n, [&](auto d) { chain_launch(p.P <= kOverlapPixels, k_raster<decltype(d)::value>, grid, kRasterWarps * 32, 0, st, p, s, w); });
   return 1;
 }
 

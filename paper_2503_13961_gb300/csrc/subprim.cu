@@ -91,8 +91,11 @@ __device__ inline void prim_cov(const Scene &s, const Work &w, int m) {
 // the last block to finish scans the counts and stores F and Nb. The same
 // launch clears the tile counters and the queue heads of the passes behind it
 // and takes the primitives' Sigma3D, so that none of them is a launch. Bound:
-// HBM (8 B read and 4 B written per pixel).
+// HBM (8 B read and 4 B written per pixel) and the loads' latency; loading every pixel's
+// or every foreground pixel's rows above and below ahead of all rounds costs more
+// registers than it hides (64 mixed views: 0.24 and 0.21 ms against 0.18).
 __global__ void __launch_bounds__(kGenThreads) k_ids(Params p, Scene s, Work w, int npb) {
+  chained();
   __shared__ int s_cnt[kGenWarps];  // foreground | boundary << 16
   __shared__ int2 s_sum[kGenWarps];
   __shared__ bool s_last;
@@ -288,6 +291,7 @@ __device__ inline uint2 tile_rect(float cx, float cy, float rx, float ry, const 
 // pixel order (the Gaussian and boundary indices): the block's offset plus
 // the set bits of the block's mask words before the pixel
 __global__ void __launch_bounds__(kGenThreads) k_compact(Params p, Work w) {
+  chained();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint2 *words = w.pix_mask + blockIdx.x * kIdWords;
   const uint2 m0 = words[lane], m1 = words[32 + lane];
@@ -367,10 +371,10 @@ __device__ inline float2 pixel_uv(const float *sB, const float *cp, int sid, int
 template <int N>
 __global__ void __launch_bounds__(kGenThreads, N <= 3 ? 4 : 3) k_generate(Params p, Scene s, Work w) {
   __shared__ float sB[kMaxVerts * SurfPoint<N>::M];
-  const int F = w.counters[kF];
-  if ((int)blockIdx.x * kGenThreads >= F) return;
   tabulate_lattice<N>(p.L, sB);
   __syncthreads();
+  chained();
+  const int F = w.counters[kF];
   for (int g0 = blockIdx.x * kGenThreads; g0 < F; g0 += gridDim.x * kGenThreads) {
     // lanes past the last Gaussian repeat it without storing (the tile counts are taken by whole warps)
     const bool live = g0 + (int)threadIdx.x < F;
@@ -501,6 +505,7 @@ __global__ void __launch_bounds__(kGenThreads, N <= 3 ? 4 : 3) k_generate(Params
 // (R^T t in world coordinates, t the camera-space point of Eq. 3)
 template <int N>
 __global__ void __launch_bounds__(256) k_sh_color(Params p, Scene s, Work w) {
+  chained();
   const int F = w.counters[kF];
   constexpr int m = SurfPoint<N>::M;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < F; i += gridDim.x * blockDim.x) {
@@ -547,33 +552,22 @@ void launch_scatter_uv(const Params &p, const Work &w, int F, cudaStream_t st) {
   if (F > 0) k_scatter_uv<<<(F + 255) / 256, 256, 0, st>>>(w, F, p.P);
 }
 
-namespace {
-
-int num_sms() {
-  int sms = 0, dev = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return sms > 0 ? sms : 152;
-}
-
-}  // namespace
-
 int launch_ids(const Params &p, const Scene &s, const Work &w, cudaStream_t st) {
   const int npb = (p.P + kIdPixels - 1) / kIdPixels;
   // small views of many primitives: more blocks for Sigma3D than the pixels give
   const int blocks = std::max(npb, std::min((p.M + kGenThreads - 1) / kGenThreads, num_sms()));
-  k_ids<<<blocks, kGenThreads, 0, st>>>(p, s, w, npb);
+  chain_launch(p.P <= kOverlapPixels, k_ids, blocks, kGenThreads, 0, st, p, s, w, npb);
   return 1;
 }
 
 int launch_generate(const Params &p, const Scene &s, const Work &w, cudaStream_t st) {
-  k_compact<<<(p.P + kIdPixels - 1) / kIdPixels, kGenThreads, 0, st>>>(p, w);
+  chain_launch(p.P <= kOverlapPixels, k_compact, (p.P + kIdPixels - 1) / kIdPixels, kGenThreads, 0, st, p, w);
   // one thread per Gaussian over a persistent grid (F is known on the device only)
   const int gblocks = std::min((p.P + kGenThreads - 1) / kGenThreads, num_sms() * 8);
-  dispatch_degree(p.n, [&](auto d) { k_generate<decltype(d)::value><<<gblocks, kGenThreads, 0, st>>>(p, s, w); });
+  dispatch_degree(p.n, [&](auto d) { chain_launch(p.P <= kOverlapPixels, k_generate<decltype(d)::value>, gblocks, kGenThreads, 0, st, p, s, w); });
   int k = 2;
   if (p.sh_deg > 0) {
-    dispatch_degree(p.n, [&](auto d) { k_sh_color<decltype(d)::value><<<152 * 8, 256, 0, st>>>(p, s, w); });
+    dispatch_degree(p.n, [&](auto d) { chain_launch(p.P <= kOverlapPixels, k_sh_color<decltype(d)::value>, 152 * 8, 256, 0, st, p, s, w); });
     k++;
   }
   return k;
