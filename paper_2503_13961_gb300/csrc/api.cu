@@ -131,7 +131,7 @@ void carve(bgt_handle *h, char *base, size_t *total) {
   w.fill_unit_cap = (int)(h->Bcap / 64 + bgt::kFillChunk * 4 * 1024);
   w.rec_hdr = c.take<uint4>((long long)w.rec_chunk_cap * bgt::kRecChunk);
   w.rec_prev = c.take<int>(w.rec_chunk_cap);
-  w.rec_fill = c.take<int>((long long)w.fill_unit_cap * 32);
+  w.rec_fill = c.take<int2>((long long)w.fill_unit_cap * 32);
   w.blk_rec = c.take<int2>(8 * (long long)T + 8);  // warp blocks: at most 8 per tile at any tile size
   w.walk_list = c.take<int>(8 * (long long)T + 8);
   w.gkeys = c.take<unsigned long long>(2 * K);   // second half: sort scratch

@@ -147,14 +147,14 @@ struct Work {
                               // (Gaussian list start, length, boundary list start, length)
   // Blend records written by the forward pass for the backward pass. A fill
   // record is written when a warp's primitive cache takes in primitive g: per
-  // pixel plane k and lane, the index of the pixel's most influential boundary
-  // point of g in the tile's boundary list, or -1 (w follows from it). A
+  // pixel plane k and lane, w and the index of the pixel's most influential
+  // boundary point of g in the tile's boundary list, or -1. A
   // header is written per (warp visit of a listed Gaussian, plane k) with at
   // least one composited pixel: (Gaussian index, lane mask of the composited
   // pixels, first unit of the fill record of its primitive, k).
   uint4 *rec_hdr;             // [rec_chunk_cap * kRecChunk]
   int *rec_prev;              // [rec_chunk_cap] previous header chunk of the same warp block, -1
-  int *rec_fill;              // [fill_unit_cap * 32] one unit = one plane of one fill record
+  int2 *rec_fill;             // [fill_unit_cap * 32] one unit = one plane of one fill record
   int2 *blk_rec;              // [warp blocks] last header chunk (-1 none, -2 overflow), records in it
   int *walk_list;             // [warp blocks] blocks whose records overflowed (counters[kWalkCount] of them):
                               // the backward re-walks their tile lists instead of replaying records

@@ -14,12 +14,11 @@
 // skipped; blending stops before the pair that would take T below t_stop.
 // Every composited (warp visit, Gaussian) is recorded for the backward pass:
 // a header (Gaussian, lane mask of the composited pixels, fill record) and,
-// per cache fill, each pixel's most influential boundary point.
+// per cache fill, each pixel's w and most influential boundary point.
 //
 // Backward: warps take warp blocks from a queue and replay the block's
-// records back to front: w is rebuilt from the recorded boundary point with
-// the forward's operations, alpha recomputed bit for bit, T_i recovered as
-// T_{i+1} / (1 - alpha_i); per-Gaussian gradients (mean, conic, opacity,
+// records back to front: w is the recorded one, alpha recomputed bit for bit,
+// T_i recovered as T_{i+1} / (1 - alpha_i); per-Gaussian gradients (mean, conic, opacity,
 // colour) are reduced over the warp before the atomics, per-boundary-point
 // gradients (position, radius) summed per (pixel, primitive) in the cache.
 #include <algorithm>
@@ -45,8 +44,8 @@ struct TileCfg {
   static constexpr int WY = (T == 32) ? 8 : 4;
   static constexpr int WPR = T / WX;         // warp blocks per tile row
   // primitive cache per warp (fully associative, FIFO): slot keys one per lane
-  static constexpr int SLOTS_FWD = (PPT == 1) ? 16 : 8;
-  static constexpr int SLOTS_BWD = (PPT == 1) ? 6 : 4;
+  static constexpr int SLOTS_FWD = (PPT == 1) ? 22 : 8;
+  static constexpr int SLOTS_BWD = (PPT == 1) ? 12 : 4;
   // resident blocks per SM the kernels are compiled for (their shared memory
   // allows this many; the register budget follows)
   static constexpr int MINB_FWD = (T == 8) ? 6 : (T == 16) ? 4 : 2;
@@ -66,6 +65,20 @@ __device__ __forceinline__ float ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
+}
+
+// q - mu from the negated staged mean (pixel centre, offset): packed additions (sm_100+), each lane
+// rounded like a subtraction; the first difference is exact
+__device__ __forceinline__ float2 mean_offset(float2 q, const float4 &Pn) {
+  unsigned long long a, b, c;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(a) : "f"(q.x), "f"(q.y));
+  asm("mov.b64 %0, {%1, %2};" : "=l"(b) : "f"(Pn.x), "f"(Pn.y));
+  asm("mov.b64 %0, {%1, %2};" : "=l"(c) : "f"(Pn.z), "f"(Pn.w));
+  asm("add.rn.f32x2 %0, %0, %1;" : "+l"(a) : "l"(b));
+  asm("add.rn.f32x2 %0, %0, %1;" : "+l"(a) : "l"(c));
+  float2 d;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(a));
+  return d;
 }
 
 // Conic (a, b, c) and opacity o of a Gaussian record, with the conic scaled
@@ -245,7 +258,7 @@ __device__ __forceinline__ BList load_boundary(const TileInfo &ti, const Work &w
 
 // Stage this warp's hits of a chunk of 32 entries of the tile's list (this
 // lane's sort key, prefetched, if valid):
-// P = (pixel x, y of the Gaussian as exact floats, offset x, y of its mean),
+// P = (pixel x, y of the Gaussian as exact floats, offset x, y of its mean), all negated,
 // Q = (conic a, b, c, opacity), C = (colour, bits(prim)). The warp block is
 // [bx0, bx1] x [by0, by1] in pixel coordinates. Returns the ballot of hits.
 __device__ __forceinline__ unsigned stage_chunk(const Work &w, unsigned long long key, bool valid, float bx0,
@@ -261,7 +274,7 @@ __device__ __forceinline__ unsigned stage_chunk(const Work &w, unsigned long lon
     const float cx = gx + A.x, cy = gy + A.y, r = A.w;
     hit = r >= 0.f && cx + r >= bx0 && cx - r <= bx1 && cy + r >= by0 && cy - r <= by1;
     if (hit) {
-      sP[lane] = make_float4(gx, gy, A.x, A.y);
+      sP[lane] = make_float4(-gx, -gy, -A.x, -A.y);
       sQ[lane] = scaled_conic(w.gB[gi]);
       sC[lane] = w.gC[gi];
       if (sG) sG[lane] = (int)gi;
@@ -345,9 +358,9 @@ struct BwdShared {
   float s_cw[Cfg::NW][S][Cfg::PPT][32];  // w of the slot's primitive per pixel
   int s_cb[Cfg::NW][S][Cfg::PPT][32];    // the slot's boundary candidate per pixel (-1: none)
   float s_cacc[Cfg::NW][S][Cfg::PPT][32];  // sum of dl/dw over the slot's Gaussians per pixel
-  // one pixel per lane: per-pair values of the last 16 records (row = record,
+  // one pixel per lane: per-pair values of the last 8 records (row = record,
   // column = pixel, stride 33) and dl/dC of the warp block's pixels
-  static constexpr int TR = (Cfg::PPT == 1) ? 16 : 1;
+  static constexpr int TR = (Cfg::PPT == 1) ? 8 : 1;
   float s_sg[Cfg::NW][TR][33];  // s = dl/dalpha w G of the pair (0 if not composited or clamped)
   float s_ta[Cfg::NW][TR][33];  // T alpha of the pair
   float4 s_dc[Cfg::NW][(Cfg::PPT == 1) ? 32 : 1];
@@ -513,9 +526,8 @@ __global__ void __launch_bounds__(TileCfg<T>::NT, TileCfg<T>::MINB_FWD) k_compos
         bool anyc = false;
 #pragma unroll
         for (int k = 0; k < PPT; k++) {
-          // q - mu: the first difference is exact
-          const float dx = __fsub_rn(__fsub_rn(pxf[k], P.x), P.z), dy = __fsub_rn(__fsub_rn(pyf[k], P.y), P.w);
-          og[k] = __fmul_rn(Q.w, gauss(dx, dy, Q));
+          const float2 d = mean_offset(make_float2(pxf[k], pyf[k]), P);
+          og[k] = __fmul_rn(Q.w, gauss(d.x, d.y, Q));
           cand[k] = !done[k] && og[k] >= p.alpha_min;  // w <= 1: else alpha < alpha_min
           anyc = anyc || cand[k];
         }
@@ -537,9 +549,9 @@ __global__ void __launch_bounds__(TileCfg<T>::NT, TileCfg<T>::MINB_FWD) k_compos
 #pragma unroll
           for (int k = 0; k < PPT; k++) {
             int best = -1;
-            cw[(slot * PPT + k) * 32 + lane] = p.use_boundary
-                ? w_search<2>(bl, lo, hi, pxr[k], pyr[k], idq[k] == g, best, n_cand) : 1.0f;
-            if (f >= 0) w.rec_fill[(size_t)(f + k) * 32 + lane] = best;
+            const float wk = p.use_boundary ? w_search<2>(bl, lo, hi, pxr[k], pyr[k], idq[k] == g, best, n_cand) : 1.0f;
+            cw[(slot * PPT + k) * 32 + lane] = wk;
+            if (f >= 0) w.rec_fill[(size_t)(f + k) * 32 + lane] = make_int2(__float_as_int(wk), best);
           }
           if (lane == slot) {
             ckey = g;
@@ -724,17 +736,6 @@ __device__ __forceinline__ void flush_boundary(const float4 *brec, const unsigne
                   cy);
 }
 
-// w (Eq. 6-7) at the cell-relative pixel (pxr, pyr) for the primitive whose
-// most influential boundary point is candidate bi of the tile's list (-1: none
-// within rho < 1), with the operations of the forward search, so the value is
-// bit-identical
-__device__ __forceinline__ float w_from_candidate(const float4 *brec, int bi, float pxr, float pyr, int cx, int cy,
-                                                  bool inside) {
-  if (bi < 0) return inside ? 1.0f : 0.0f;
-  const float gamma = gamma_of(rec_r2(cell_record(brec[bi], cx, cy), pxr, pyr));
-  return inside ? gamma : __fsub_rn(1.0f, gamma);
-}
-
 // Backward pass over the forward pass's blend records. Every warp takes warp
 // blocks (tile, block) from a queue and replays the block's records back to
 // front: T_i = T_{i+1} / (1 - alpha_i) with alpha_i recomputed from the
@@ -817,7 +818,7 @@ __global__ void __launch_bounds__(TileCfg<T>::NT, TileCfg<T>::MINB_BWD) k_compos
           const float4 A = w.gA[h.x];
           const unsigned qxy = __float_as_uint(A.z);
           sH[lane] = h;
-          sP[lane] = make_float4((float)(int)(qxy & 0xffffu), (float)(int)(qxy >> 16), A.x, A.y);
+          sP[lane] = make_float4(-(float)(int)(qxy & 0xffffu), -(float)(int)(qxy >> 16), -A.x, -A.y);
           sQ[lane] = scaled_conic(w.gB[h.x]);
           sC[lane] = w.gC[h.x];
         }
@@ -842,24 +843,28 @@ __global__ void __launch_bounds__(TileCfg<T>::NT, TileCfg<T>::MINB_BWD) k_compos
                                     pyr, cx, cy);
 #pragma unroll
               for (int k = 0; k < PPT; k++) {
-                const int bi = (int)h.z >= 0 ? w.rec_fill[(size_t)((int)h.z + k) * 32 + lane] : -1;
-                s_cw[slot][k][lane] = w_from_candidate(brec, bi, pxr[k], pyr[k], cx, cy, idq[k] == g);
-                s_cb[slot][k][lane] = bi;
+                // no fill: a primitive without boundary points in the tile
+                int2 fill = make_int2(__float_as_int(idq[k] == g ? 1.0f : 0.0f), -1);
+                if ((int)h.z >= 0) fill = w.rec_fill[(size_t)((int)h.z + k) * 32 + lane];
+                s_cw[slot][k][lane] = __int_as_float(fill.x);
+                s_cb[slot][k][lane] = fill.y;
                 s_cacc[slot][k][lane] = 0.f;
               }
               if (lane == slot) ckey = g;
             }
           }
           if constexpr (PPT == 1) {
-            // the pair's values go to row r % 16 of the warp's transposition rows;
-            // every 16 records, lane i (and i + 16, for the other half of the
-            // pixels) sums record i's values over the block's pixels: the
-            // per-Gaussian sums without a warp reduction per record
+            // the pair's values go to row r % 8 of the warp's transposition rows;
+            // every 8 records, the lanes 8 q + i sum record i's values over
+            // pixel row q of the block and the four rows' sums are reduce-scattered: the
+            // per-Gaussian sums without a warp reduction per record. Rows of 8 records, not 16,
+            // leave the shared memory for 12 cache slots instead of 6 (an
+            // evicted slot costs its boundary gradients' atomics and the next miss a fill)
             float sg = 0.f, ta = 0.f, dl_dw = 0.f;
             if (mine) {
               if constexpr (STATS) n_comp++;
-              const float dx = __fsub_rn(__fsub_rn(pxf[0], P.x), P.z), dy = __fsub_rn(__fsub_rn(pyf[0], P.y), P.w);
-              const float G = gauss(dx, dy, Q);
+              const float2 d = mean_offset(make_float2(pxf[0], pyf[0]), P);
+              const float G = gauss(d.x, d.y, Q);
               const float og = __fmul_rn(Q.w, G);
               const float wv = p.use_boundary ? s_cw[slot][0][lane] : 1.0f;
               const float raw = __fmul_rn(og, wv);
@@ -867,33 +872,54 @@ __global__ void __launch_bounds__(TileCfg<T>::NT, TileCfg<T>::MINB_BWD) k_compos
               dl_dw = pair_values(G, og, wv, raw, alpha, p.alpha_max, Cc, dC[0], Tr[0], R[0], sg, ta);
               if (p.use_boundary) s_cacc[slot][0][lane] += dl_dw;
             }
-            sh.s_sg[warp][r & 15][lane] = sg;
-            sh.s_ta[warp][r & 15][lane] = ta;
-            if ((r & 15) == 0) {
+            sh.s_sg[warp][r & 7][lane] = sg;
+            sh.s_ta[warp][r & 7][lane] = ta;
+            if ((r & 7) == 0) {
               __syncwarp();
-              const int i = lane & 15, half = lane >> 4, rec = r + i;
-              float acc[9];
+              const int i = lane & 7, row = lane >> 3, rec = r + i;
+              float v[9];
 #pragma unroll
-              for (int q = 0; q < 9; q++) acc[q] = 0.f;
+              for (int q = 0; q < 9; q++) v[q] = 0.f;
               if (rec < n) {
                 const float4 Pm = sP[rec];
-                const float bxm = __fsub_rn(__fsub_rn(wx0, Pm.x), Pm.z), bym = __fsub_rn(__fsub_rn(wy0, Pm.y), Pm.w);
+                const float2 d0 = mean_offset(make_float2(wx0, wy0 + (float)row), Pm);
+                // along the row dy is constant: its factors are taken once
 #pragma unroll
-                for (int j = 0; j < 16; j++) {
-                  const int l = half * 16 + j;
+                for (int j = 0; j < 8; j++) {
+                  const int l = row * 8 + j;
                   const float4 dc = sh.s_dc[warp][l];
-                  const float dcv[3] = {dc.x, dc.y, dc.z};
-                  add_pair_sums(sh.s_sg[warp][i][l], sh.s_ta[warp][i][l], bxm + (float)(l & 7), bym + (float)(l >> 3),
-                                dcv, acc);
+                  const float sgv = sh.s_sg[warp][i][l], tav = sh.s_ta[warp][i][l];
+                  const float dx = d0.x + (float)j, a = sgv * dx;
+                  v[0] += a;
+                  v[2] = fmaf(a, dx, v[2]);
+                  v[5] += sgv;
+                  v[6] = fmaf(tav, dc.x, v[6]);
+                  v[7] = fmaf(tav, dc.y, v[7]);
+                  v[8] = fmaf(tav, dc.z, v[8]);
                 }
+                v[1] = v[5] * d0.y;
+                v[3] = v[0] * d0.y;
+                v[4] = v[1] * d0.y;
+              }
+              // reduce-scatter over the rows: row 0 keeps sums 0-2, 1: 5-7, 2: 3-4, 3: 8
+              const bool r1 = row & 1, r2 = row & 2;
+              float u[5], t[3];
+#pragma unroll
+              for (int q = 0; q < 5; q++) {
+                const float hi = q < 4 ? v[5 + q] : 0.f;
+                u[q] = (r1 ? hi : v[q]) + __shfl_xor_sync(0xffffffffu, r1 ? v[q] : hi, 8);
               }
 #pragma unroll
-              for (int q = 0; q < 9; q++) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], 16);
-              if (rec < n && half == 0) {
-                float *gg = w.gg + 12 * (size_t)sH[rec].x;
+              for (int q = 0; q < 3; q++) {
+                const float hi = q < 2 ? u[3 + q] : 0.f;
+                t[q] = (r2 ? hi : u[q]) + __shfl_xor_sync(0xffffffffu, r2 ? u[q] : hi, 16);
+              }
+              if (rec < n) {
+                float *gg = w.gg + 12 * (size_t)sH[rec].x + (r1 ? 5 : 0) + (r2 ? 3 : 0);
+                const int m = r2 ? (r1 ? 1 : 2) : 3;
 #pragma unroll
-                for (int q = 0; q < 9; q++)
-                  if (acc[q] != 0.f) atomicAdd(gg + q, acc[q]);
+                for (int q = 0; q < 3; q++)
+                  if (q < m && t[q] != 0.f) atomicAdd(gg + q, t[q]);
               }
               __syncwarp();
             }
@@ -906,13 +932,13 @@ __global__ void __launch_bounds__(TileCfg<T>::NT, TileCfg<T>::MINB_BWD) k_compos
             for (int k = 0; k < PPT; k++) {
               if (k != rk || !mine) continue;
               if constexpr (STATS) n_comp++;
-              const float dx = __fsub_rn(__fsub_rn(pxf[k], P.x), P.z), dy = __fsub_rn(__fsub_rn(pyf[k], P.y), P.w);
-              const float G = gauss(dx, dy, Q);
+              const float2 d = mean_offset(make_float2(pxf[k], pyf[k]), P);
+              const float G = gauss(d.x, d.y, Q);
               const float og = __fmul_rn(Q.w, G);
               const float wv = p.use_boundary ? s_cw[slot][k][lane] : 1.0f;
               const float raw = __fmul_rn(og, wv);
               const float alpha = fminf(p.alpha_max, raw);
-              dl_dw = pair_backward(dx, dy, G, og, wv, raw, alpha, p.alpha_max, Cc, dC[k], Tr[k], R[k], acc);
+              dl_dw = pair_backward(d.x, d.y, G, og, wv, raw, alpha, p.alpha_max, Cc, dC[k], Tr[k], R[k], acc);
             }
             if (p.use_boundary && mine) s_cacc[slot][rk][lane] += dl_dw;
             // per-Gaussian sums (see pair_backward); slots 0-7 by reduce-scatter
@@ -1066,8 +1092,8 @@ __global__ void __launch_bounds__(TileCfg<T>::NT) k_composite_bwd_walk(Params p,
       bool anyc = false;
 #pragma unroll
       for (int k = 0; k < PPT; k++) {
-        const float dx = __fsub_rn(__fsub_rn(pxf[k], P.x), P.z), dy = __fsub_rn(__fsub_rn(pyf[k], P.y), P.w);
-        Gk[k] = gauss(dx, dy, Q);
+        const float2 d = mean_offset(make_float2(pxf[k], pyf[k]), P);
+        Gk[k] = gauss(d.x, d.y, Q);
         og[k] = __fmul_rn(Q.w, Gk[k]);
         cand[k] = e < nlast[k] && og[k] >= p.alpha_min;
         anyc = anyc || cand[k];
@@ -1104,8 +1130,8 @@ __global__ void __launch_bounds__(TileCfg<T>::NT) k_composite_bwd_walk(Params p,
         const float raw = __fmul_rn(og[k], wv);
         const float alpha = fminf(p.alpha_max, raw);
         if (alpha < p.alpha_min) continue;
-        const float dx = __fsub_rn(__fsub_rn(pxf[k], P.x), P.z), dy = __fsub_rn(__fsub_rn(pyf[k], P.y), P.w);
-        const float dl_dw = pair_backward(dx, dy, Gk[k], og[k], wv, raw, alpha, p.alpha_max, Cc, dC[k], Tr[k], R[k], acc);
+        const float2 d = mean_offset(make_float2(pxf[k], pyf[k]), P);
+        const float dl_dw = pair_backward(d.x, d.y, Gk[k], og[k], wv, raw, alpha, p.alpha_max, Cc, dC[k], Tr[k], R[k], acc);
         if (p.use_boundary)
           boundary_grad(brec, bkeys, w.bg_grad, best, dl_dw, idq[k] == g, pxr[k], pyr[k], bl.cx, bl.cy);
       }
