@@ -98,9 +98,10 @@ SMS, FP32_LANES = 152, 128
 
 LAMBDA = 0.2      # weight of the D-SSIM term of Eq. 9
 # Algorithmic FP32 operations per pixel and channel of the fused loss: the
-# separable 11-tap window over five moments (2 x 5 x 11 FMA) and over three
-# SSIM partials (2 x 3 x 11 FMA), SSIM and its partials (~20), the gradient (6)
-LOSS_FLOPS_PER_VALUE = 2 * (2 * 5 * 11 + 2 * 3 * 11) + 26
+# separable 11-tap window over four moments (x, y, xy and x^2 + y^2, which is all
+# that SSIM needs of the two squares: 2 x 4 x 11 FMA) and over three SSIM
+# partials (2 x 3 x 11 FMA), SSIM and its partials (~20), the gradient (6)
+LOSS_FLOPS_PER_VALUE = 2 * (2 * 4 * 11 + 2 * 3 * 11) + 26
 
 # Algorithmic FP32 operations per work unit of the blending kernels (FMA = 2,
 # exp / sqrt / divide = 1): a pair inside a Gaussian's support needs the offset,
@@ -176,10 +177,13 @@ def stage_bytes(stage, c, M, ncp, V):
     return {
         # control points per view + one 64-bit depth key per pixel
         "raster": 12 * ncp * M * V + 8 * P,
-        # depth key read, I_id + I_uv write
+        # depth key read, I_id + I_uv write: a pass that resolves both for every pixel
         "resolve": 8 * P + 12 * P,
-        # I_id (+ neighbours) and I_uv read, Gaussian (48 B) and boundary (16 B) records written
-        "generate": 4 * P + 8 * F + 48 * F + 16 * Nb,
+        # what the stage timed as "resolve" does: depth key read, I_id write (I_uv is part of "generate";
+        # the foreground and boundary masks are 0.25 B per pixel)
+        "ids": 8 * P + 4 * P,
+        # depth key of each foreground pixel read, Gaussian (48 B) and boundary (16 B) records written
+        "generate": 8 * F + 48 * F + 16 * Nb,
         # pair keys written once, read + written by the per-tile sort
         "binning": 3 * 8 * K + 3 * 8 * Kb + 20 * Kb,
         # per tile: keys + 48-B records of its pairs, 20-B boundary entries; image, T, n, I_id per pixel
@@ -195,9 +199,9 @@ def stage_bytes(stage, c, M, ncp, V):
 # DRAM bytes (read + write) per composited pair of the blending kernels, from one
 # ncu capture of four 1024^2 views (profiles/composite_blend_views1024x4.md),
 # valid only for the kernel source they were measured on (else traffic: null)
-BLEND_TRAFFIC = {"source_sha256": "31926f2fd2cc1a5d3a82528a9d09ede5a53636275ce296cf8d2a83e72afeef5b",
-                 "composite_fwd": (131572480 + 153608192) / 50625814,
-                 "composite_bwd": (292371712 + 40375552) / 50625814}
+BLEND_TRAFFIC = {"source_sha256": "298302ccb3235284a55777b2fcf56451ed88b334cc4becc896df1fae19e0310d",
+                 "composite_fwd": (123715584 + 178526720) / 50625814,
+                 "composite_bwd": (332592896 + 46526208) / 50625814}
 
 
 # Warp instructions per warp visit of the blending kernels (a visit: one warp,
@@ -205,7 +209,7 @@ BLEND_TRAFFIC = {"source_sha256": "31926f2fd2cc1a5d3a82528a9d09ede5a53636275ce29
 # capture; the forward keeps the issue slots ~80 % busy, so issue is the
 # ceiling that binds it; same source check as the traffic
 BLEND_ISSUE = {"source_sha256": BLEND_TRAFFIC["source_sha256"],
-               "composite_fwd": 681557800 / 5419084, "composite_bwd": 552831143 / 4948871}
+               "composite_fwd": 672020532 / 5419084, "composite_bwd": 518734525 / 4948871}
 
 
 def _blend_source_matches():
@@ -518,7 +522,7 @@ def run_ours(args):
         fp32_peak = SMS * FP32_LANES * 2 * sm_mhz * 1e6 / 1e12
         per_stage = {}
         for s_name, s_ms in stage_ms.items():
-            b = stage_bytes(s_name, counts, M, ncp, V)
+            b = stage_bytes("ids" if s_name == "resolve" else s_name, counts, M, ncp, V)
             per_stage[s_name] = {"ms": round(s_ms, 4), "alg_bytes": int(b),
                                  "GBps": round(b / (s_ms * 1e-3) / 1e9, 1) if s_ms > 0 else None,
                                  "hbm_frac": round(b / (s_ms * 1e-3) / 1e9 / peak, 4) if s_ms > 0 else None}
@@ -527,7 +531,7 @@ def run_ours(args):
                 per_stage[s_name]["alg_flops"] = int(fl)
                 per_stage[s_name]["TFLOPs"] = round(fl / (s_ms * 1e-3) / 1e12, 3)
                 per_stage[s_name]["alu_frac"] = round(fl / (s_ms * 1e-3) / 1e12 / fp32_peak, 4)
-        dom_bytes = stage_bytes(dom, counts, M, ncp, V)
+        dom_bytes = per_stage[dom]["alg_bytes"]
         achieved = dom_bytes / (stage_ms[dom] * 1e-3) / 1e9
         out = {
             "metric": METRIC, "value": round(value, 2), "unit": "renders/s", "n_gpus": world,

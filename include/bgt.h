@@ -184,7 +184,8 @@ int bgt_get_tile_size(const bgt_handle *h);
  * counting, on = 0 turns profiling off (BGT_ERR_INVALID_ARG otherwise). bgt_get_profile
  * waits for the last backward and returns device milliseconds of the last
  * forward + backward: ms[0] clears + per-primitive prep, [1] tessellation +
- * raster, [2] resolve, [3] sub-primitive generation, [4] binning + sort,
+ * raster, [2] I_id, boundary set and foreground counts, [3] compaction and
+ * sub-primitive generation (I_uv included), [4] binning + sort,
  * [5] forward blending, [6] backward blending, [7] chain to parameters;
  * *kernels_fwd / *kernels_bwd receive the kernels each pass enqueues.
  * units (nullable) receives the work units the blending kernels counted:
