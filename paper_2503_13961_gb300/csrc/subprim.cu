@@ -283,7 +283,8 @@ __device__ inline uint2 tile_rect(float cx, float cy, float rx, float ry, const 
   x0 = max(x0, 0); y0 = max(y0, 0);
   x1 = min(x1, vw.W - 1); y1 = min(y1, vw.H - 1);
   if (x0 > x1 || y0 > y1) return make_uint2(1u, 0u);  // x0 = 1 > x1 = 0: empty
-  x0 /= t; x1 /= t; y0 /= t; y1 /= t;
+  const int sh = 31 - __clz(t);  // 8, 16 or 32; no coordinate is negative here
+  x0 >>= sh; x1 >>= sh; y0 >>= sh; y1 >>= sh;
   return make_uint2((unsigned)x0 | ((unsigned)y0 << 16), (unsigned)x1 | ((unsigned)y1 << 16));
 }
 
