@@ -244,6 +244,7 @@ constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kRunCap = 512;                    // keys one warp sorts in registers (16 per lane)
 constexpr int kWarpSortCap = 2 * kRunCap;       // keys one warp sorts: two such runs, merged
 constexpr int kSortCap = kSortWarps * kWarpSortCap;  // keys one block sorts in shared memory
+constexpr int kLongCap = 8 * kSortCap;               // keys one block sorts as runs of kSortCap, merged
 constexpr int kFullKeys = 1 << 30;              // flag of a listed segment: its order needs all key bits
 
 // position of key i in shared memory: one key of padding per 16, so that lanes
@@ -476,7 +477,7 @@ __device__ __forceinline__ WordForm word_form(const KeyRange &r, bool bnd, int p
 __device__ __forceinline__ unsigned key_word(const WordForm &f, bool bnd, unsigned long long key, int pos,
                                              int pos_bits) {
   const unsigned hi = (unsigned)(key >> 32) - f.hi0, lo = (unsigned)key;
-  // boundary shift is below 32 (both ranges within 31 bits), pos_bits between 5 and 13
+  // boundary shift is below 32 (both ranges within 31 bits), pos_bits between 5 and 16
   return bnd ? (hi << f.shift) | (lo - f.lo0)
              : ((((hi << 5) | (lo >> kIndexBits)) >> f.shift) << pos_bits) | (unsigned)pos;
 }
@@ -490,20 +491,24 @@ __device__ __forceinline__ unsigned long long word_key(const WordForm &f, bool b
 
 constexpr int kFixPasses = 8;  // rounds of neighbour exchanges before a list is sorted on all bits
 
+struct Padded {
+  __device__ int operator()(int i) const { return padded(i); }
+};
+
 // One round of exchanges (even, then odd neighbours) among the sorted words of a
 // Gaussian list that agree above their position bits, by the full keys; true
-// if any moved. SYNC separates the two halves and ends the round.
-template <class Sync>
-__device__ __forceinline__ bool exchange_ties(const unsigned long long *keys, unsigned *s, int n, int pos_bits, int first,
-                                              int step, Sync sync) {
+// if any moved. SYNC separates the two halves and ends the round. Word i is at s[at(i)].
+template <class At, class Sync>
+__device__ __forceinline__ bool exchange_ties(const unsigned long long *keys, unsigned *s, At at, int n, int pos_bits,
+                                              int first, int step, Sync sync) {
   const unsigned mask = (1u << pos_bits) - 1u;
   bool moved = false;
   for (int odd = 0; odd < 2; odd++) {
     for (int i = 2 * first + odd; i + 1 < n; i += 2 * step) {
-      const unsigned a = s[padded(i)], b = s[padded(i + 1)];
+      const unsigned a = s[at(i)], b = s[at(i + 1)];
       if (((a ^ b) >> pos_bits) == 0u && keys[b & mask] < keys[a & mask]) {
-        s[padded(i)] = b;
-        s[padded(i + 1)] = a;
+        s[at(i)] = b;
+        s[at(i + 1)] = a;
         moved = true;
       }
     }
@@ -594,7 +599,7 @@ __device__ __forceinline__ bool warp_sort_segment(const Work &w, const unsigned 
   unsigned *s = warp_sort_words(keys, sk, sk + kWarpWords, f, bnd, 0, n, pos_bits);
   if (!bnd) {
     int pass = 0;
-    while (__any_sync(0xffffffffu, exchange_ties(keys, s, n, pos_bits, lane, 32, [] { __syncwarp(); })))
+    while (__any_sync(0xffffffffu, exchange_ties(keys, s, Padded(), n, pos_bits, lane, 32, [] { __syncwarp(); })))
       if (++pass == kFixPasses) return false;
   }
   for (int i = lane; i < n; i += 32) store_sorted(w, bnd, s0 + i, word_key(f, bnd, keys, s[padded(i)], pos_bits));
@@ -717,14 +722,10 @@ __device__ __forceinline__ void block_sort_full(const Work &w, const unsigned lo
   for (int i = threadIdx.x; i < n; i += kSortThreads) store_sorted(w, bnd, s0 + i, s[padded(i)]);
 }
 
-// a segment of n <= kSortCap keys as 32-bit words: a quarter of them per warp,
-// then two merges by the block; false: it needs all key bits
-__device__ __forceinline__ bool block_sort_words(const Work &w, const unsigned long long *keys, unsigned *s,
-                                                 KeyRange *s_range, bool bnd, long long s0, int n) {
-  static_assert(kSortWarps == 4, "two merge levels");
-  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, pos_bits = position_bits(n);
+// the key range of a segment, by the block
+__device__ __forceinline__ KeyRange block_key_range(const unsigned long long *keys, int n, KeyRange *s_range) {
   KeyRange r = key_range(keys, n, threadIdx.x, kSortThreads);
-  if (lane == 0) s_range[wp] = r;
+  if ((threadIdx.x & 31) == 0) s_range[threadIdx.x >> 5] = r;
   __syncthreads();
   for (int q = 0; q < kSortWarps; q++) {
     r.hi0 = min(r.hi0, s_range[q].hi0);
@@ -732,8 +733,15 @@ __device__ __forceinline__ bool block_sort_words(const Work &w, const unsigned l
     r.lo0 = min(r.lo0, s_range[q].lo0);
     r.lo1 = max(r.lo1, s_range[q].lo1);
   }
-  const WordForm f = word_form(r, bnd, pos_bits);
-  if (!f.ok) return false;
+  return r;
+}
+
+// The words of keys[0, n), n <= kSortCap, positions from 0 on, sorted by the block: a quarter of them per
+// warp, then two merges. s: both buffers; returned: the one that holds the result, behind a block barrier.
+__device__ __forceinline__ unsigned *block_sort_run(const unsigned long long *keys, unsigned *s, const WordForm &f,
+                                                    bool bnd, int n, int pos_bits) {
+  static_assert(kSortWarps == 4, "two merge levels");
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   unsigned *t = s + kSortWarps * kWarpWords;
   const int q = (n + kSortWarps - 1) / kSortWarps;  // <= kWarpSortCap, and all quarters on one side of kRunCap
   const int c[5] = {0, min(q, n), min(2 * q, n), min(3 * q, n), n};
@@ -759,9 +767,20 @@ __device__ __forceinline__ bool block_sort_words(const Work &w, const unsigned l
     merge_part(t, 0, c[2], c[2], n - c[2], s, 0, min(d, n), min(d + part, n));
   }
   __syncthreads();
+  return s;
+}
+
+// a segment of n <= kSortCap keys as 32-bit words; false: it needs all key bits
+__device__ __forceinline__ bool block_sort_words(const Work &w, const unsigned long long *keys, unsigned *s,
+                                                 KeyRange *s_range, bool bnd, long long s0, int n) {
+  const int pos_bits = position_bits(n);
+  const WordForm f = word_form(block_key_range(keys, n, s_range), bnd, pos_bits);
+  if (!f.ok) return false;
+  s = block_sort_run(keys, s, f, bnd, n, pos_bits);
   if (!bnd) {
     int pass = 0;
-    while (__syncthreads_or(exchange_ties(keys, s, n, pos_bits, threadIdx.x, kSortThreads, [] { __syncthreads(); })))
+    while (__syncthreads_or(
+        exchange_ties(keys, s, Padded(), n, pos_bits, threadIdx.x, kSortThreads, [] { __syncthreads(); })))
       if (++pass == kFixPasses) return false;
   }
   for (int i = threadIdx.x; i < n; i += kSortThreads)
@@ -769,15 +788,107 @@ __device__ __forceinline__ bool block_sort_words(const Work &w, const unsigned l
   return true;
 }
 
+// How many of the first d outputs of the merge of a[0, na) and b[0, nb) (distinct words, global memory)
+// come from a: the warp tests 32 points of the diagonal at a time.
+__device__ __forceinline__ int merge_split(const unsigned *a, int na, const unsigned *b, int nb, int d) {
+  const int lane = threadIdx.x & 31;
+  int lo = max(0, d - nb), hi = min(d, na);
+  while (lo < hi) {
+    const int step = (hi - lo + 31) >> 5, mid = lo + lane * step;
+    const bool below = mid < hi && a[mid] < b[d - 1 - mid];
+    const int cnt = __popc(__ballot_sync(0xffffffffu, below));
+    hi = min(hi, lo + cnt * step);
+    if (cnt > 0) lo += (cnt - 1) * step + 1;
+  }
+  return lo;
+}
+
+// src[0, n) in sorted runs of len words merged in pairs into dst, kSortCap outputs at a time: their inputs
+// are two contiguous pieces, merged in shared memory (s: both buffers).
+__device__ __forceinline__ void merge_runs(const unsigned *src, unsigned *dst, int n, int len, unsigned *s, int *s_split) {
+  unsigned *t = s + kSortWarps * kWarpWords;
+  const int wp = threadIdx.x >> 5;
+  for (int r = 0; r < n; r += 2 * len) {
+    const int na = min(len, n - r), nb = min(len, n - r - na);
+    const unsigned *a = src + r, *b = a + na;
+    for (int d0 = 0; d0 < na + nb; d0 += kSortCap) {
+      const int d1 = min(d0 + kSortCap, na + nb), m = d1 - d0;
+      if (wp < 2) s_split[wp] = merge_split(a, na, b, nb, wp ? d1 : d0);
+      __syncthreads();
+      const int i0 = s_split[0], ni = s_split[1] - i0, j0 = d0 - i0;
+      for (int k = threadIdx.x; k < m; k += kSortThreads) s[padded(k)] = k < ni ? a[i0 + k] : b[j0 + k - ni];
+      __syncthreads();
+      const int part = (m + kSortThreads - 1) / kSortThreads, d = (int)threadIdx.x * part;
+      merge_part(s, 0, ni, ni, m - ni, t, 0, min(d, m), min(d + part, m));
+      __syncthreads();
+      for (int k = threadIdx.x; k < m; k += kSortThreads) dst[r + d0 + k] = t[padded(k)];
+    }
+  }
+  __syncthreads();
+}
+
+// A segment of kSortCap < n <= kLongCap keys as 32-bit words: equal runs of at most kSortCap sorted in shared
+// memory, the runs merged between the two halves of the list's own place (8 bytes per key hold two words
+// per key), ending in the upper half. False: it needs all key bits.
+__device__ __forceinline__ bool block_sort_long(const Work &w, const unsigned long long *keys, unsigned *s,
+                                                KeyRange *s_range, int *s_split, bool bnd, long long s0, int n) {
+  const int pos_bits = position_bits(n);
+  const WordForm f = word_form(block_key_range(keys, n, s_range), bnd, pos_bits);
+  if (!f.ok) return false;
+  const int runs = (n + kSortCap - 1) / kSortCap, len = (n + runs - 1) / runs;
+  unsigned *lower = reinterpret_cast<unsigned *>((bnd ? w.bkeys : w.gkeys) + s0), *upper = lower + n;
+  unsigned *cur = (32 - __clz(runs - 1)) & 1 ? lower : upper;  // an odd number of merge passes ends in the other half
+  for (int r = 0; r < n; r += len) {
+    const int m = min(len, n - r);
+    const unsigned *out = block_sort_run(keys + r, s, f, bnd, m, pos_bits);
+    for (int k = threadIdx.x; k < m; k += kSortThreads) cur[r + k] = out[padded(k)] + (bnd ? 0u : (unsigned)r);
+    __syncthreads();
+  }
+  for (int l = len; l < n; l *= 2) {
+    unsigned *next = cur == lower ? upper : lower;
+    merge_runs(cur, next, n, l, s, s_split);
+    cur = next;
+  }
+  if (!bnd) {
+    int pass = 0;
+    while (__syncthreads_or(exchange_ties(keys, upper, [](int i) { return i; }, n, pos_bits, threadIdx.x, kSortThreads,
+                                          [] { __syncthreads(); })))
+      if (++pass == kFixPasses) return false;
+  }
+  // keys [i, i + step) end at word 2 (i + step), at most n + i + step: no word is overwritten before it is read
+  constexpr int kEach = 8, step = kEach * kSortThreads;
+  for (int i = 0; i < n; i += step) {
+    unsigned word[kEach];
+#pragma unroll
+    for (int e = 0; e < kEach; e++) {
+      const int k = i + e * kSortThreads + (int)threadIdx.x;
+      word[e] = k < n ? upper[k] : 0u;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < kEach; e++) {
+      const int k = i + e * kSortThreads + (int)threadIdx.x;
+      if (k < n) store_sorted(w, bnd, s0 + k, word_key(f, bnd, keys, word[e], pos_bits));
+    }
+  }
+  return true;
+}
+
 // Segments longer than kWarpSortCap and those that need all key bits: one
-// block each, in shared memory up to kSortCap keys, by a stable radix sort in
-// global memory beyond. On eight 1600 x 1200 views of the room (dense tiles)
+// block each, in shared memory up to kSortCap keys, as merged runs of that many
+// up to kLongCap (from there on the words' depth bits, 32 less the position's, no
+// longer tell neighbours apart), by a stable radix sort in global memory beyond and where the
+// words do not resolve the order. On eight 1600 x 1200 views of a room
 // a bitonic network of the block over 64-bit keys in shared memory took 1.62
-// ms, quarters sorted by the warps and merged on 32-bit words 0.78 ms.
+// ms, quarters sorted by the warps and merged on 32-bit words 0.78 ms; with
+// larger Gaussians (150 M pairs, lists up to ~9,000 keys) the radix sort
+// of the lists beyond kSortCap (a pass per 8 key bits, three barriers per 128 keys) took
+// the kernel to 9.9 ms, the merged runs to 5.2.
 __global__ void __launch_bounds__(kSortThreads, 4) k_tile_sort_big(Params p, Work w, const int *big_list) {
   chained();
   extern __shared__ __align__(16) unsigned long long s_keys[];
   __shared__ KeyRange s_range[kSortWarps];
+  __shared__ int s_split[2];
   const int nbig = w.counters[kBigCount];
   for (int b = blockIdx.x; b < nbig; b += gridDim.x) {
     const int item = big_list[b];
@@ -792,7 +903,9 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_tile_sort_big(Params p, Wor
         __syncthreads();
         block_sort_full<kWarpSortCap / 32>(w, keys, s_keys, bnd, s0, n);
       }
-    } else {
+    } else if (n > kLongCap ||
+               !block_sort_long(w, keys, reinterpret_cast<unsigned *>(s_keys), s_range, s_split, bnd, s0, n)) {
+      __syncthreads();
       unsigned long long *s_red = s_keys;  // 2 per warp
       int *s_hist = reinterpret_cast<int *>(s_keys + 2 * kSortWarps), *s_base = s_hist + 256;
       unsigned long long *out = (bnd ? w.bkeys : w.gkeys) + s0;
