@@ -1,5 +1,6 @@
 """The per-tile sort at the sizes where it changes form (runs of 32, 64, 128, 256 and 512 words per
-warp, two merged runs, the block's quarters, the radix sort beyond 4096 keys) and on depths that need
+warp, two merged runs, the block's quarters, the block's merged runs beyond 4096 keys, the radix sort
+beyond 32768) and on depths that need
 each of its forms: spread depths, ties, depths closer than the words resolve, all equal (the index
 decides), and a range too wide for 32-bit words. Keys are integers: the list has to hold every Gaussian
 once, in ascending key order."""
