@@ -4,6 +4,7 @@
 #include <cstdio>
 #include <algorithm>
 #include <cstring>
+#include <initializer_list>
 #include <string>
 #include <vector>
 
@@ -311,6 +312,13 @@ std::string graph_key(const bgt::Params &p, const void *a, const void *b, const 
   return k;
 }
 
+// the other addresses a captured pass reads or writes, and the counting mode, for its key
+std::string key_of(const bgt_handle *h, std::initializer_list<const void *> addresses) {
+  std::string k;
+  for (const void *a : addresses) k += "|" + std::to_string((size_t)a);
+  return k + (h->profiling ? "|P" : "|-") + (h->count_units ? "U" : "-");
+}
+
 template <class F>
 cudaError_t run_graph(cudaGraphExec_t *exec, std::string *key_slot, const std::string &key, cudaStream_t st, F body) {
   if (*exec && *key_slot == key) return cudaGraphLaunch(*exec, st);
@@ -433,8 +441,7 @@ bgt_status bgt_render_fwd(bgt_handle *h, const bgt_scene *scene, const bgt_camer
   cudaError_t e;
   if ((h->cfg.flags & BGT_FLAG_GRAPH) && st != nullptr) {
     const std::string key = graph_key(p, scene->ctrl, scene->color, scene->opacity, scene->r_b, images, cams, n_views) +
-                            std::to_string((size_t)scene->quat) + std::to_string((size_t)scene->log_scale) +
-                            std::to_string((size_t)scene->sh) + (h->profiling ? "P" : "-") + (h->count_units ? "U" : "-");
+                            key_of(h, {scene->quat, scene->log_scale, scene->sh});
     e = run_graph(&h->g_fwd, &h->g_fwd_key, key, st, [&]() { return enqueue_fwd(h, p, sc, images, st); });
   } else {
     e = enqueue_fwd(h, p, sc, images, st);
@@ -473,10 +480,11 @@ bgt_status bgt_render_bwd(bgt_handle *h, const bgt_scene *scene, const bgt_camer
                      scene->sh_degree > 0 ? grads->sh : nullptr};
   cudaError_t e;
   if ((h->cfg.flags & BGT_FLAG_GRAPH) && st != nullptr) {
+    // the chain rule reads the rotation, scaling and SH arrays again
     const std::string key = graph_key(p, scene->ctrl, d_images, grads->ctrl, grads->color, grads->opacity, cams,
-                                      n_views) + std::to_string((size_t)grads->r_b) +
-                            std::to_string((size_t)grads->log_scale) + std::to_string((size_t)grads->quat) +
-                            std::to_string((size_t)grads->sh) + (h->profiling ? "P" : "-") + (h->count_units ? "U" : "-");
+                                      n_views) +
+                            key_of(h, {grads->r_b, grads->log_scale, grads->quat, grads->sh, scene->quat,
+                                       scene->log_scale, scene->sh});
     e = run_graph(&h->g_bwd, &h->g_bwd_key, key, st, [&]() { return enqueue_bwd(h, p, sc, d_images, g, st); });
   } else {
     e = enqueue_bwd(h, p, sc, d_images, g, st);
