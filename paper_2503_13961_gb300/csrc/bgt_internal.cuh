@@ -196,7 +196,7 @@ constexpr unsigned long long kIndexMask = (1ull << kIndexBits) - 1ull;
 
 enum Counter { kF = 0, kNb = 1, kK = 2, kKb = 3, kQueueFwd = 4, kQueueBwd = 5, kQueueSort = 6, kBigCount = 7,
                kRecChunks = 8, kFillChunks = 9, kWalkCount = 10, kQueueWalk = 11, kIdsDone = 12,
-               kQueueEmpty = 13, kTileClass = 16 };
+               kQueueEmpty = 13, kSumsUsed = 14, kTileClass = 16 };
 constexpr int kCounters = 24;
 
 // ---------------------------------------------------------------------------

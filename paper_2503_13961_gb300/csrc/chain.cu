@@ -378,10 +378,12 @@ __device__ __forceinline__ void clear_floats(float *p, long long n) {
   if (tail + t0 < n) p[tail + t0] = 0.f;
 }
 
-// Everything the backward pass adds into, cleared in one launch: the gradient
+// What the backward pass adds into, cleared in one launch: the gradient
 // arrays, the per-primitive record counters and dl/dSigma3D, the queue heads
 // (nine or more memsets, 2-3 us each in the serial chain of a small call). With maps
-// of leg resolution 1 the map gradients are written whole at the end.
+// of leg resolution 1 the map gradients are written whole at the end. The sums per
+// Gaussian and boundary point come cleared from the generation pass; a further
+// backward pass over the same forward (counters[kSumsUsed]) clears them here.
 __global__ void __launch_bounds__(256) k_clear_grads(Params p, Work w, Grads g) {
   chained();
   const long long M = p.M;
@@ -398,6 +400,10 @@ __global__ void __launch_bounds__(256) k_clear_grads(Params p, Work w, Grads g) 
   if (p.sh_k > 0) clear_floats(g.sh, 3 * M * p.sh_k);
   clear_floats(reinterpret_cast<float *>(w.prim_gcnt), M);
   clear_floats(reinterpret_cast<float *>(w.prim_bcnt), M);
+  if (w.counters[kSumsUsed]) {
+    clear_floats(w.gg, 12ll * w.counters[kF]);
+    clear_floats(reinterpret_cast<float *>(w.bg_grad), 4ll * w.counters[kNb]);
+  }
   if (blockIdx.x == 0 && threadIdx.x == 0) w.counters[kQueueBwd] = w.counters[kQueueWalk] = 0;
 }
 

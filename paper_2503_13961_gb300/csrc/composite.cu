@@ -1019,6 +1019,7 @@ __global__ void __launch_bounds__(TileCfg<T>::NT) k_composite_bwd_walk(Params p,
   float4 *sP = s_P[warp], *sQ = s_Q[warp], *sC = s_C[warp];
   int *sG = s_G[warp];
   count_prim_records(w);
+  if (blockIdx.x == 0 && threadIdx.x == 0) w.counters[kSumsUsed] = 1;  // cleared by the forward's I_id pass
   const int nwalk = w.counters[kWalkCount];
   for (;;) {
     int q = 0;

@@ -39,3 +39,42 @@ def test_graph_follows_swapped_attribute_arrays(scenes, attr_res, swapped):
         rd.sync_status(stream=s)
         for k, v in w.items():
             assert grad_rel(grads[k].cpu(), v.cpu()) < GRAD_TOL, k
+
+
+@pytest.mark.parametrize("graph", [False, True])
+@pytest.mark.parametrize("records", [0, 512])  # default capacity; 512: most blocks re-walk their tile lists
+def test_backward_twice_after_one_forward(scenes, graph, records):
+    """Two image gradients taken back through one forward: each backward overwrites the gradients with
+    its own, as after a forward of its own."""
+    import torch
+    from paper_2503_13961_gb300 import render as R
+    sc, cams = scenes.tiny_scene("ico1", noise=0.04, size=(96, 80), r_b=0.03)
+    sc = scenes.with_sh(sc, 1)
+    dev = R.scene_to_device(sc)
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    ds = [torch.randn((96 * 80, 3), generator=gen, device="cuda") for _ in range(2)]
+    plain = make_renderer(sc, cams)
+    want = [_step(plain, dev, cams, d, None)[0] for d in ds]
+    rd = make_renderer(sc, cams, graph=graph, max_blend_pairs=records)
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    for _ in range(2):  # graphs: captured, then replayed
+        rd.forward(dev, cams, stream=s)
+        for d, w in zip(ds + ds[:1], want + want[:1]):
+            got = rd.backward(dev, cams, d, stream=s)
+            s.synchronize()
+            rd.sync_status(stream=s)
+            for k, v in w.items():
+                assert grad_rel(got[k].cpu(), v.cpu()) < GRAD_TOL, k
+
+
+def test_autograd_of_a_retained_graph(scenes):
+    import torch
+    from paper_2503_13961_gb300 import render as R
+    sc, cams = scenes.tiny_scene("ico1", noise=0.04, size=(70, 50), r_b=0.03)
+    dev = R.scene_to_device(sc)
+    dev["ctrl"].requires_grad_(True)
+    img = R.render(make_renderer(sc, cams), dev, cams)
+    a = torch.autograd.grad(img.square().sum(), dev["ctrl"], retain_graph=True)[0]
+    b = torch.autograd.grad(img.square().sum(), dev["ctrl"])[0]
+    assert grad_rel(b.cpu(), a.cpu()) < GRAD_TOL
