@@ -148,7 +148,8 @@ bgt_status bgt_render_fwd(bgt_handle *h, const bgt_scene *scene, const bgt_camer
  * and sh when not NULL) with dl/dparameters summed over all views, holding
  * I_id, I_uv, B and the per-pixel survivor lists of the forward fixed
  * (supplementary "Backward Derivative"). The scene and cameras must be those
- * of the forward; BGT_ERR_STATE otherwise or without a forward. */
+ * of the forward (ctrl array, num_prims, attr_res, sh_degree, view sizes);
+ * BGT_ERR_STATE otherwise or without a forward. */
 bgt_status bgt_render_bwd(bgt_handle *h, const bgt_scene *scene, const bgt_camera *cams, int n_views,
                           const float *d_images, const bgt_grads *grads, void *stream);
 

@@ -469,10 +469,16 @@ bgt_status bgt_render_bwd(bgt_handle *h, const bgt_scene *scene, const bgt_camer
   if (scene->num_prims > 0 && (!grads->ctrl || !grads->color || !grads->opacity || !grads->r_b))
     return fail(h, BGT_ERR_INVALID_ARG, "null gradient array");
   if (!h->fwd_valid) return fail(h, BGT_ERR_STATE, "backward without a forward");
-  bool same = scene->ctrl == h->fwd_ctrl && n_views == h->fwd_views && scene->num_prims == h->last.M;
+  const int attr_res = scene->attr_res == 0 ? 1 : scene->attr_res;
+  bool same = scene->ctrl == h->fwd_ctrl && n_views == h->fwd_views && scene->num_prims == h->last.M &&
+              attr_res == h->last.attr_res && scene->sh_degree == h->last.sh_deg;
   for (int v = 0; same && v < n_views; v++)
     same = cams[v].width == h->fwd_shapes[2 * v] && cams[v].height == h->fwd_shapes[2 * v + 1];
   if (!same) return fail(h, BGT_ERR_STATE, "backward scene / views differ from the forward");
+  // the arrays that the chain rule reads again
+  const bool maps = attr_res > 1 || grads->log_scale || grads->quat;
+  if (scene->num_prims > 0 && ((maps && (!scene->log_scale || !scene->quat)) || (scene->sh_degree > 0 && !scene->sh)))
+    return fail(h, BGT_ERR_INVALID_ARG, "null scene array");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const bgt::Params p = h->last;
   const bgt::Scene sc = to_scene(scene);

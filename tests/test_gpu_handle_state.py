@@ -78,3 +78,29 @@ def test_autograd_of_a_retained_graph(scenes):
     a = torch.autograd.grad(img.square().sum(), dev["ctrl"], retain_graph=True)[0]
     b = torch.autograd.grad(img.square().sum(), dev["ctrl"])[0]
     assert grad_rel(b.cpu(), a.cpu()) < GRAD_TOL
+
+
+def test_backward_refuses_a_scene_of_another_form(scenes):
+    """The pass over the last forward's records reads maps and SH of the forward's sizes: a scene with the
+    same control points and another map resolution or SH degree is refused before any launch."""
+    import torch
+    from paper_2503_13961_gb300 import render as R
+    sc, cams = scenes.tiny_scene("ico1", size=(40, 30))
+    forms = [R.scene_to_device(sc), R.scene_to_device(scenes.with_attribute_maps(sc, 3)),
+             R.scene_to_device(scenes.with_sh(sc, 2))]
+    for f in forms:
+        f["ctrl"] = forms[0]["ctrl"]
+    rd = make_renderer(sc, cams)
+    d = torch.ones((40 * 30, 3), device="cuda")
+    for i, f in enumerate(forms):
+        rd.forward(f, cams)
+        want = rd.backward(f, cams, d)
+        for j, other in enumerate(forms):
+            if j != i:
+                with pytest.raises(RuntimeError, match="differ from the forward"):
+                    rd.backward(other, cams, d)
+        assert grad_rel(rd.backward(f, cams, d)["ctrl"].cpu(), want["ctrl"].cpu()) < GRAD_TOL
+    for attr_res in (0, 1):  # both name maps of one texel
+        rd.forward(dict(forms[0], attr_res=1 - attr_res), cams)
+        rd.backward(dict(forms[0], attr_res=attr_res), cams, d)
+    rd.sync_status()
