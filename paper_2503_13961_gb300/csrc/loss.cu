@@ -144,6 +144,8 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_l2_dssim_grad(const __grid_
 
   // loads: value e of an image row (pixel e / 3, channel e % 3) by thread e, the
   // kExtra values beyond one per thread spread over the threads
+  // (plain loads: the renderer may still write the image when this kernel's blocks start, and the
+  // read-only path of __ldg is for memory that nothing writes during the kernel)
   const long long pitch = 3ll * W;
   const long long origin = (vw.off + (long long)(y0 - 2 * kR) * W + x0 - 2 * kR) * 3;  // of the first image row's values
   const int gx = x0 - 2 * kR + tid / 3;
@@ -157,7 +159,7 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_l2_dssim_grad(const __grid_
       ld[r] = make_float2(0.f, 0.f);
       if (col_ok && gy >= 0 && gy < H) {
         const long long o = origin + (i0 + r) * pitch + tid;
-        ld[r] = make_float2(__ldg(a.img + o), __ldg(a.gt + o));
+        ld[r] = make_float2(a.img[o], a.gt[o]);
       }
     }
 #pragma unroll
@@ -167,7 +169,7 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_l2_dssim_grad(const __grid_
       lx[k] = make_float2(0.f, 0.f);
       if (r < kRows && x >= 0 && x < W && gy >= 0 && gy < H) {
         const long long o = origin + (i0 + r) * pitch + e;
-        lx[k] = make_float2(__ldg(a.img + o), __ldg(a.gt + o));
+        lx[k] = make_float2(a.img[o], a.gt[o]);
       }
     }
   };

@@ -104,3 +104,28 @@ def test_backward_refuses_a_scene_of_another_form(scenes):
         rd.forward(dict(forms[0], attr_res=1 - attr_res), cams)
         rd.backward(dict(forms[0], attr_res=attr_res), cams, d)
     rd.sync_status()
+
+
+def test_loss_right_behind_the_forward(scenes):
+    """The loss starts while the forward that writes its images drains: its gradient is that of the
+    finished images, two scenes in turn through one buffer."""
+    import torch
+    from paper_2503_13961_gb300 import render as R
+    sc, cams = scenes.tiny_scene("ico1", noise=0.04, size=(96, 80), r_b=0.03)
+    dark = dict(sc, color=sc["color"] * 0.25)
+    rd = make_renderer(sc, cams)
+    devs = [R.scene_to_device(x) for x in (sc, dark)]
+    gt = torch.rand((96 * 80, 3), generator=torch.Generator(device="cuda").manual_seed(5), device="cuda")
+    img, d = torch.empty_like(gt), [torch.empty_like(gt) for _ in range(40)]
+    want = []
+    for dev in devs:
+        rd.forward(dev, cams, images=img)
+        torch.cuda.synchronize()
+        want.append(rd.l2_dssim_loss_grad(img, gt, cams).clone())
+    torch.cuda.synchronize()
+    for i in range(40):
+        rd.forward(devs[i % 2], cams, images=img)
+        rd.l2_dssim_loss_grad(img, gt, cams, d_images=d[i])
+    torch.cuda.synchronize()
+    for i in range(40):
+        assert torch.equal(d[i], want[i % 2]), i
