@@ -421,21 +421,24 @@ __device__ __forceinline__ void store_sorted(const Work &w, bool bnd, long long 
 // How the 64-bit keys of one segment are sorted as 32-bit words, which one
 // compare-exchange of the network moves in two instructions instead of six (and
 // the network's code, a third of the size, stays in the instruction cache).
-//   Boundary keys: (primitive - least) << lo_bits | (index - least), the key
-//   itself shortened, when both ranges fit 31 bits together.
-//   Gaussian keys: the depth key less the least FP32 depth of the segment,
+//   Exact words: (primitive or depth key - least) << index bits | (index -
+//   least), the key itself shortened, when both ranges fit 31 bits together.
+//   Boundary keys have no other; of the Gaussian keys it is those of a surface at
+//   one depth, whose ties no position resolves: a wall that faces eight 1600 x
+//   1200 views (58 M pairs) took the binning 10.1 ms when its lists ended on all key bits, now 0.91.
+//   Gaussian keys otherwise: the depth key less the least FP32 depth of the segment,
 //   cut to its upper bits, with the key's position in the segment below them.
 //   Depths that differ only in the cut bits, and ties of depth, may leave
 //   neighbours out of order: words that agree above their positions are
 //   exchanged by their full keys (groups of up to 3 on the room's tiles).
 // Segments that fit neither are sorted on all key bits.
 struct WordForm {
-  unsigned hi0, lo0;  // least high word; boundary keys: least low word
-  int shift;          // Gaussian keys: bits cut off; boundary keys: lo_bits
-  bool ok;
+  unsigned hi0, lo0;   // least high word and index
+  int low, down, up;   // key bits below the primitive or depth key, its bits cut off, word bits below it
+  bool exact, ok;
 };
 
-// least and greatest high word of a segment; boundary keys: low words too
+// least and greatest high word and index of a segment
 struct KeyRange {
   unsigned hi0, hi1, lo0, lo1;
 };
@@ -444,7 +447,7 @@ __device__ __forceinline__ KeyRange key_range(const unsigned long long *keys, in
   KeyRange r{0xffffffffu, 0u, 0xffffffffu, 0u};
   for (int i = first; i < n; i += step) {
     const unsigned long long k = keys[i];
-    const unsigned hi = (unsigned)(k >> 32), lo = (unsigned)k;
+    const unsigned hi = (unsigned)(k >> 32), lo = (unsigned)(k & kIndexMask);
     r.hi0 = min(r.hi0, hi);
     r.hi1 = max(r.hi1, hi);
     r.lo0 = min(r.lo0, lo);
@@ -457,36 +460,33 @@ __device__ __forceinline__ KeyRange key_range(const unsigned long long *keys, in
   return r;
 }
 
-// pos_bits: bits of a position in the segment
-__device__ __forceinline__ WordForm word_form(const KeyRange &r, bool bnd, int pos_bits) {
+// n: keys of the segment
+__device__ __forceinline__ WordForm word_form(const KeyRange &r, bool bnd, int n) {
   WordForm f;
   f.hi0 = r.hi0;
   f.lo0 = r.lo0;
+  f.low = bnd ? 32 : kIndexBits;
   const unsigned span = r.hi1 - r.hi0;
-  if (bnd) {
-    f.shift = 32 - __clz((int)(r.lo1 - r.lo0));
-    f.ok = f.shift + 32 - __clz((int)span) <= 31;
-  } else {
-    f.ok = span < (1u << 27);  // depth key less (hi0 << 5) fits 32 bits
-    const int bits = 32 - __clz((int)((span << 5) | 31u));
-    f.shift = max(0, bits - (32 - pos_bits));
-  }
+  const bool narrow = span < (1u << 27);  // the depth key less (hi0 << 5) fits 32 bits
+  const int bits = bnd ? 32 - __clz((int)span) : narrow ? 32 - __clz((int)((span << 5) | 31u)) : 32;
+  const int index_bits = 32 - __clz((int)(r.lo1 - r.lo0));
+  const int pos_bits = max(5, 32 - __clz(n));  // one more position than keys for the padding word
+  f.exact = index_bits + bits <= 31;
+  f.ok = f.exact || (!bnd && narrow);
+  f.down = f.exact ? 0 : max(0, bits - (32 - pos_bits));
+  f.up = f.exact ? index_bits : pos_bits;
   return f;
 }
 
-__device__ __forceinline__ unsigned key_word(const WordForm &f, bool bnd, unsigned long long key, int pos,
-                                             int pos_bits) {
-  const unsigned hi = (unsigned)(key >> 32) - f.hi0, lo = (unsigned)key;
-  // boundary shift is below 32 (both ranges within 31 bits), pos_bits between 5 and 16
-  return bnd ? (hi << f.shift) | (lo - f.lo0)
-             : ((((hi << 5) | (lo >> kIndexBits)) >> f.shift) << pos_bits) | (unsigned)pos;
+__device__ __forceinline__ unsigned key_word(const WordForm &f, unsigned long long key, int pos) {
+  const unsigned rank = __funnelshift_rc((unsigned)key, (unsigned)(key >> 32) - f.hi0, f.low);
+  return ((rank >> f.down) << f.up) | (f.exact ? (unsigned)(key & kIndexMask) - f.lo0 : (unsigned)pos);
 }
 
-__device__ __forceinline__ unsigned long long word_key(const WordForm &f, bool bnd, const unsigned long long *keys,
-                                                       unsigned word, int pos_bits) {
-  if (!bnd) return keys[word & ((1u << pos_bits) - 1u)];
-  const unsigned lo = word & ((1u << f.shift) - 1u);
-  return ((unsigned long long)((word >> f.shift) + f.hi0) << 32) | (unsigned long long)(lo + f.lo0);
+__device__ __forceinline__ unsigned long long word_key(const WordForm &f, const unsigned long long *keys, unsigned word) {
+  const unsigned lo = word & ((1u << f.up) - 1u);
+  if (!f.exact) return keys[lo];
+  return ((unsigned long long)f.hi0 << 32) + ((unsigned long long)(word >> f.up) << f.low) + (lo + f.lo0);
 }
 
 constexpr int kFixPasses = 8;  // rounds of neighbour exchanges before a list is sorted on all bits
@@ -522,14 +522,13 @@ __device__ __forceinline__ bool exchange_ties(const unsigned long long *keys, un
 // code of a size, which has to stay in the instruction cache (a form of 32
 // words per lane beside it made the fetches the first stall).
 template <int E>
-__device__ __noinline__ void warp_sort_run(const unsigned long long *keys, unsigned *s, WordForm f, bool bnd, int first,
-                                           int n, int pos_bits) {
+__device__ __noinline__ void warp_sort_run(const unsigned long long *keys, unsigned *s, WordForm f, int first, int n) {
   const int lane = threadIdx.x & 31;
   unsigned k[E];
 #pragma unroll
   for (int e = 0; e < E; e++) {
     const int i = e * 32 + lane;
-    k[e] = i < n ? key_word(f, bnd, keys[i], first + i, pos_bits) : 0xffffffffu;  // padding: last in any order
+    k[e] = i < n ? key_word(f, keys[i], first + i) : 0xffffffffu;  // padding: last in any order
   }
   warp_sort_regs<E>(k, lane);
 #pragma unroll
@@ -537,13 +536,13 @@ __device__ __noinline__ void warp_sort_run(const unsigned long long *keys, unsig
     if (lane * E + e < n) s[padded(first + lane * E + e)] = k[e];
 }
 
-__device__ __forceinline__ void sort_run(const unsigned long long *keys, unsigned *s, const WordForm &f, bool bnd,
-                                         int first, int n, int pos_bits) {
-  if (n <= 32) warp_sort_run<1>(keys, s, f, bnd, first, n, pos_bits);
-  else if (n <= 64) warp_sort_run<2>(keys, s, f, bnd, first, n, pos_bits);
-  else if (n <= 128) warp_sort_run<4>(keys, s, f, bnd, first, n, pos_bits);
-  else if (n <= 256) warp_sort_run<8>(keys, s, f, bnd, first, n, pos_bits);
-  else warp_sort_run<16>(keys, s, f, bnd, first, n, pos_bits);
+__device__ __forceinline__ void sort_run(const unsigned long long *keys, unsigned *s, const WordForm &f, int first,
+                                         int n) {
+  if (n <= 32) warp_sort_run<1>(keys, s, f, first, n);
+  else if (n <= 64) warp_sort_run<2>(keys, s, f, first, n);
+  else if (n <= 128) warp_sort_run<4>(keys, s, f, first, n);
+  else if (n <= 256) warp_sort_run<8>(keys, s, f, first, n);
+  else warp_sort_run<16>(keys, s, f, first, n);
 }
 
 // Outputs [d0, d1) of the merge of the sorted runs s[a, a + na) and s[b, b + nb)
@@ -575,10 +574,10 @@ __device__ __forceinline__ void merge_part(const unsigned *s, int a, int na, int
 // The words of keys[0, n), n <= kWarpSortCap, positions from `first` on, sorted by one warp; the result
 // is in s or t (returned), padded positions from `first` on.
 __device__ __forceinline__ unsigned *warp_sort_words(const unsigned long long *keys, unsigned *s, unsigned *t,
-                                                     const WordForm &f, bool bnd, int first, int n, int pos_bits) {
+                                                     const WordForm &f, int first, int n) {
   const int n0 = min(n, kRunCap), n1 = n - n0;
-  sort_run(keys, s, f, bnd, first, n0, pos_bits);
-  if (n1 > 0) sort_run(keys + n0, s, f, bnd, first + n0, n1, pos_bits);
+  sort_run(keys, s, f, first, n0);
+  if (n1 > 0) sort_run(keys + n0, s, f, first + n0, n1);
   __syncwarp();
   if (n1 <= 0) return s;
   const int lane = threadIdx.x & 31, part = (n + 31) >> 5;
@@ -587,22 +586,18 @@ __device__ __forceinline__ unsigned *warp_sort_words(const unsigned long long *k
   return t;
 }
 
-// position bits of a segment of n keys: one more position than keys for the padding word
-__device__ __forceinline__ int position_bits(int n) { return max(5, 32 - __clz(n)); }
-
 // A segment of n <= kWarpSortCap keys, sorted by one warp. False: it needs all key bits.
 __device__ __forceinline__ bool warp_sort_segment(const Work &w, const unsigned long long *keys, unsigned *sk, bool bnd,
                                                   long long s0, int n, int lane) {
-  const int pos_bits = position_bits(n);
-  const WordForm f = word_form(key_range(keys, n, lane, 32), bnd, pos_bits);
+  const WordForm f = word_form(key_range(keys, n, lane, 32), bnd, n);
   if (!f.ok) return false;
-  unsigned *s = warp_sort_words(keys, sk, sk + kWarpWords, f, bnd, 0, n, pos_bits);
-  if (!bnd) {
+  unsigned *s = warp_sort_words(keys, sk, sk + kWarpWords, f, 0, n);
+  if (!f.exact) {
     int pass = 0;
-    while (__any_sync(0xffffffffu, exchange_ties(keys, s, Padded(), n, pos_bits, lane, 32, [] { __syncwarp(); })))
+    while (__any_sync(0xffffffffu, exchange_ties(keys, s, Padded(), n, f.up, lane, 32, [] { __syncwarp(); })))
       if (++pass == kFixPasses) return false;
   }
-  for (int i = lane; i < n; i += 32) store_sorted(w, bnd, s0 + i, word_key(f, bnd, keys, s[padded(i)], pos_bits));
+  for (int i = lane; i < n; i += 32) store_sorted(w, bnd, s0 + i, word_key(f, keys, s[padded(i)]));
   __syncwarp();
   return true;
 }
@@ -739,7 +734,7 @@ __device__ __forceinline__ KeyRange block_key_range(const unsigned long long *ke
 // The words of keys[0, n), n <= kSortCap, positions from 0 on, sorted by the block: a quarter of them per
 // warp, then two merges. s: both buffers; returned: the one that holds the result, behind a block barrier.
 __device__ __forceinline__ unsigned *block_sort_run(const unsigned long long *keys, unsigned *s, const WordForm &f,
-                                                    bool bnd, int n, int pos_bits) {
+                                                    int n) {
   static_assert(kSortWarps == 4, "two merge levels");
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   unsigned *t = s + kSortWarps * kWarpWords;
@@ -747,10 +742,10 @@ __device__ __forceinline__ unsigned *block_sort_run(const unsigned long long *ke
   const int c[5] = {0, min(q, n), min(2 * q, n), min(3 * q, n), n};
   const int first = min(wp * q, n), mine = min(q, n - first);
   // one or two runs per warp: which buffer holds the result is decided by q for all warps alike
-  sort_run(keys + first, s, f, bnd, first, min(mine, kRunCap), pos_bits);
+  sort_run(keys + first, s, f, first, min(mine, kRunCap));
   if (q > kRunCap) {
     const int n0 = min(mine, kRunCap), n1 = mine - n0, part = (mine + 31) >> 5;
-    if (n1 > 0) sort_run(keys + first + n0, s, f, bnd, first + n0, n1, pos_bits);
+    if (n1 > 0) sort_run(keys + first + n0, s, f, first + n0, n1);
     __syncwarp();
     merge_part(s, first, n0, first + n0, n1, t, first, min(lane * part, mine), min(lane * part + part, mine));
     unsigned *x = s; s = t; t = x;
@@ -773,18 +768,17 @@ __device__ __forceinline__ unsigned *block_sort_run(const unsigned long long *ke
 // a segment of n <= kSortCap keys as 32-bit words; false: it needs all key bits
 __device__ __forceinline__ bool block_sort_words(const Work &w, const unsigned long long *keys, unsigned *s,
                                                  KeyRange *s_range, bool bnd, long long s0, int n) {
-  const int pos_bits = position_bits(n);
-  const WordForm f = word_form(block_key_range(keys, n, s_range), bnd, pos_bits);
+  const WordForm f = word_form(block_key_range(keys, n, s_range), bnd, n);
   if (!f.ok) return false;
-  s = block_sort_run(keys, s, f, bnd, n, pos_bits);
-  if (!bnd) {
+  s = block_sort_run(keys, s, f, n);
+  if (!f.exact) {
     int pass = 0;
     while (__syncthreads_or(
-        exchange_ties(keys, s, Padded(), n, pos_bits, threadIdx.x, kSortThreads, [] { __syncthreads(); })))
+        exchange_ties(keys, s, Padded(), n, f.up, threadIdx.x, kSortThreads, [] { __syncthreads(); })))
       if (++pass == kFixPasses) return false;
   }
   for (int i = threadIdx.x; i < n; i += kSortThreads)
-    store_sorted(w, bnd, s0 + i, word_key(f, bnd, keys, s[padded(i)], pos_bits));
+    store_sorted(w, bnd, s0 + i, word_key(f, keys, s[padded(i)]));
   return true;
 }
 
@@ -832,16 +826,15 @@ __device__ __forceinline__ void merge_runs(const unsigned *src, unsigned *dst, i
 // per key), ending in the upper half. False: it needs all key bits.
 __device__ __forceinline__ bool block_sort_long(const Work &w, const unsigned long long *keys, unsigned *s,
                                                 KeyRange *s_range, int *s_split, bool bnd, long long s0, int n) {
-  const int pos_bits = position_bits(n);
-  const WordForm f = word_form(block_key_range(keys, n, s_range), bnd, pos_bits);
+  const WordForm f = word_form(block_key_range(keys, n, s_range), bnd, n);
   if (!f.ok) return false;
   const int runs = (n + kSortCap - 1) / kSortCap, len = (n + runs - 1) / runs;
   unsigned *lower = reinterpret_cast<unsigned *>((bnd ? w.bkeys : w.gkeys) + s0), *upper = lower + n;
   unsigned *cur = (32 - __clz(runs - 1)) & 1 ? lower : upper;  // an odd number of merge passes ends in the other half
   for (int r = 0; r < n; r += len) {
     const int m = min(len, n - r);
-    const unsigned *out = block_sort_run(keys + r, s, f, bnd, m, pos_bits);
-    for (int k = threadIdx.x; k < m; k += kSortThreads) cur[r + k] = out[padded(k)] + (bnd ? 0u : (unsigned)r);
+    const unsigned *out = block_sort_run(keys + r, s, f, m);
+    for (int k = threadIdx.x; k < m; k += kSortThreads) cur[r + k] = out[padded(k)] + (f.exact ? 0u : (unsigned)r);
     __syncthreads();
   }
   for (int l = len; l < n; l *= 2) {
@@ -849,9 +842,9 @@ __device__ __forceinline__ bool block_sort_long(const Work &w, const unsigned lo
     merge_runs(cur, next, n, l, s, s_split);
     cur = next;
   }
-  if (!bnd) {
+  if (!f.exact) {
     int pass = 0;
-    while (__syncthreads_or(exchange_ties(keys, upper, [](int i) { return i; }, n, pos_bits, threadIdx.x, kSortThreads,
+    while (__syncthreads_or(exchange_ties(keys, upper, [](int i) { return i; }, n, f.up, threadIdx.x, kSortThreads,
                                           [] { __syncthreads(); })))
       if (++pass == kFixPasses) return false;
   }
@@ -868,7 +861,7 @@ __device__ __forceinline__ bool block_sort_long(const Work &w, const unsigned lo
 #pragma unroll
     for (int e = 0; e < kEach; e++) {
       const int k = i + e * kSortThreads + (int)threadIdx.x;
-      if (k < n) store_sorted(w, bnd, s0 + k, word_key(f, bnd, keys, word[e], pos_bits));
+      if (k < n) store_sorted(w, bnd, s0 + k, word_key(f, keys, word[e]));
     }
   }
   return true;
@@ -883,7 +876,9 @@ __device__ __forceinline__ bool block_sort_long(const Work &w, const unsigned lo
 // ms, quarters sorted by the warps and merged on 32-bit words 0.78 ms; with
 // larger Gaussians (150 M pairs, lists up to ~9,000 keys) the radix sort
 // of the lists beyond kSortCap (a pass per 8 key bits, three barriers per 128 keys) took
-// the kernel to 9.9 ms, the merged runs to 5.2.
+// the kernel to 9.9 ms, the merged runs to 5.2. All key bits are sorted in as few registers as the list
+// fills: padded to kSortCap keys whatever its length, boundary lists of ~200 keys whose primitive and index
+// ranges exceed 31 bits (320,000 primitives in random order) took the binning of eight views 18.2 ms, now 1.6.
 __global__ void __launch_bounds__(kSortThreads, 4) k_tile_sort_big(Params p, Work w, const int *big_list) {
   chained();
   extern __shared__ __align__(16) unsigned long long s_keys[];
@@ -901,7 +896,11 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_tile_sort_big(Params p, Wor
     if (n <= kSortCap) {
       if (full || !block_sort_words(w, keys, reinterpret_cast<unsigned *>(s_keys), s_range, bnd, s0, n)) {
         __syncthreads();
-        block_sort_full<kWarpSortCap / 32>(w, keys, s_keys, bnd, s0, n);
+        if (n <= 128) block_sort_full<1>(w, keys, s_keys, bnd, s0, n);
+        else if (n <= 512) block_sort_full<4>(w, keys, s_keys, bnd, s0, n);
+        else if (n <= 1024) block_sort_full<8>(w, keys, s_keys, bnd, s0, n);
+        else if (n <= 2048) block_sort_full<16>(w, keys, s_keys, bnd, s0, n);
+        else block_sort_full<kWarpSortCap / 32>(w, keys, s_keys, bnd, s0, n);
       }
     } else if (n > kLongCap ||
                !block_sort_long(w, keys, reinterpret_cast<unsigned *>(s_keys), s_range, s_split, bnd, s0, n)) {
