@@ -8,7 +8,8 @@
 // window (sigma 1.5, zero outside the image), C1 = 0.01^2, C2 = 0.03^2,
 // averaged over pixels and channels; L2 is the mean of (C - C_gt)^2.
 //
-// One CTA owns a strip of kOutW columns and some rows of one view, all three
+// One CTA owns a strip of kOutW columns (the first and the last of a view kR more)
+// and some rows of one view, all three
 // channels (views of any size, the image layout of the renderer: concatenated
 // [H][W][3] blocks), and streams down it kRows rows at a time. The gradient
 // needs SSIM's partials a = ds/dmu_x, b = ds/d(F (x^2 + y^2)), c = ds/d(F xy)
@@ -23,12 +24,14 @@
 // c) with the symmetric window as its own adjoint. HBM traffic is the two
 // images read and the gradient written.
 //
-// Streaming leaves a halo to recompute only beside a strip (64 of 54 columns)
-// and above a segment of rows: ~180 window FMAs per value, the square sum
+// Streaming leaves a halo to recompute only beside a strip (64 of 54 columns, none beyond a
+// view's edge) and above a segment of rows (none above the view): ~180 window FMAs per value, the square sum
 // included, against 288 for 32 x 32 tiles that recompute it on all sides
 // (52 x 52 -> 42 x 42 -> 32 x 32). Bound: issue (55 % of the slots busy at 12
 // warps per SM) and the FP32 pipe. 64 mixed views (97 M values) took 2.01 ms,
-// now 1.30; one 800^2 view 53 us, now 41. Three CTAs per SM spill the sums
+// now 1.27; one 800^2 view 53 us, now 40; 64 and 112 views of 64^2 35 and 58 us while such a view took two
+// strips and a search of 24 us, now 21 and 32 (tiles: 22 and 35). Views narrower than a strip leave the
+// other columns idle: 112 views of 32^2 take 21 us, 13 as tiles. Three CTAs per SM spill the sums
 // (112 registers: 1.70 ms without loads in flight, 2.13 with).
 //
 // The moments are taken of x - 1/2 and y - 1/2 (pixels outside the image: -1/2):
@@ -47,7 +50,7 @@ namespace {
 constexpr int kR = 5;
 constexpr int kTaps = 2 * kR + 1;
 constexpr int kLossThreads = 192;                       // 3 channels x 64 columns
-constexpr int kOutW = 54, kPartW = kOutW + 2 * kR, kInW = kOutW + 4 * kR;  // columns: output, partials, image
+constexpr int kOutW = 54, kPartW = kOutW + 2 * kR, kInW = kOutW + 4 * kR;  // columns: step of strips, partials, image
 constexpr int kRows = 8;                                // rows per group
 constexpr int kRun = 8;                                 // columns a thread filters along a row
 constexpr int kRing = kRows + 2 * kR;                   // image rows held: an output row completes 10 rows behind
@@ -57,7 +60,9 @@ static_assert(kLossThreads == 3 * kPartW && kPartW == kRun * (kLossThreads / 3 /
 // warp reads 8 runs of 2 rows), its channels 12 (three channels stored together)
 __host__ __device__ constexpr int pad8(int i) { return i + (i >> 3); }
 constexpr int kInStride = 88, kInPlane = kRing * kInStride + 6;  // float2 (x, y)
-constexpr int kPartStride = pad8(kPartW), kPartPlane = kRows * kPartStride;  // float4
+// rows of partials hold 8 columns of padding before and 5 behind, zero: the window along a row reads kR beyond
+constexpr int kPartPad = 8, kPartAt = pad8(kPartPad);  // column c at pad8(c) + kPartAt
+constexpr int kPartStride = pad8(kPartPad + kPartW + kR - 1) + 1, kPartPlane = kRows * kPartStride;  // float4
 static_assert(pad8(kInW - 1) < kInStride && kInStride * 2 % 32 == 16, "ring row");
 constexpr int kLossSmem = (int)(sizeof(float2) * 3 * kInPlane + sizeof(float4) * 3 * kPartPlane);
 static_assert(2 * kLossSmem + 4096 <= 232448, "two CTAs per SM");
@@ -133,8 +138,10 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_l2_dssim_grad(const __grid_
   const LossView &vw = a.view[lo];
   const int W = vw.W, H = vw.H;
   const int tile = blockIdx.x - vw.tile0;
-  const int x0 = (tile % vw.strips) * kOutW, y0 = (tile / vw.strips) * a.seg;
+  const int strip = tile % vw.strips;
+  const int x0 = strip * kOutW, y0 = (tile / vw.strips) * a.seg;  // first column of partials, first output row
   const int y1 = min(y0 + a.seg, H);
+  const int skip = max(2 * kR - y0, 0), r0 = y0 - 2 * kR + skip;  // rows above the view, first image row
   const float w_l2 = vw.w_l2, w_ssim = vw.w_ssim;
   const int tid = threadIdx.x;
   const int ch = tid / kPartW, col = tid % kPartW;    // column phases: channel and column
@@ -147,17 +154,16 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_l2_dssim_grad(const __grid_
   // (plain loads: the renderer may still write the image when this kernel's blocks start, and the
   // read-only path of __ldg is for memory that nothing writes during the kernel)
   const long long pitch = 3ll * W;
-  const long long origin = (vw.off + (long long)(y0 - 2 * kR) * W + x0 - 2 * kR) * 3;  // of the first image row's values
-  const int gx = x0 - 2 * kR + tid / 3;
+  const long long origin = (vw.off + (long long)r0 * W + x0 - kR) * 3;  // of the first image row's values
+  const int gx = x0 - kR + tid / 3;
   const bool col_ok = gx >= 0 && gx < W;
   const int slot_e = (tid % 3) * kInPlane + pad8(tid / 3);
   float2 ld[kRows], lx[kExtraLoads];
   auto load = [&](int i0) {  // image rows i0 .. i0 + kRows - 1 of the strip into registers
 #pragma unroll
     for (int r = 0; r < kRows; r++) {
-      const int gy = y0 - 2 * kR + i0 + r;
       ld[r] = make_float2(0.f, 0.f);
-      if (col_ok && gy >= 0 && gy < H) {
+      if (col_ok && r0 + i0 + r < H) {
         const long long o = origin + (i0 + r) * pitch + tid;
         ld[r] = make_float2(a.img[o], a.gt[o]);
       }
@@ -165,9 +171,9 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_l2_dssim_grad(const __grid_
 #pragma unroll
     for (int k = 0; k < kExtraLoads; k++) {
       const int q = tid + k * kLossThreads, r = q / kExtra, e = kLossThreads + q % kExtra;
-      const int gy = y0 - 2 * kR + i0 + r, x = x0 - 2 * kR + e / 3;
+      const int x = x0 - kR + e / 3;
       lx[k] = make_float2(0.f, 0.f);
-      if (r < kRows && x >= 0 && x < W && gy >= 0 && gy < H) {
+      if (r < kRows && x >= 0 && x < W && r0 + i0 + r < H) {
         const long long o = origin + (i0 + r) * pitch + e;
         lx[k] = make_float2(a.img[o], a.gt[o]);
       }
@@ -182,8 +188,32 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_l2_dssim_grad(const __grid_
     m01[k] = m23[k] = fab[k] = 0ull;
     fc[k] = 0.f;
   }
+  if (skip > 0) {  // the rows above the view (x = y = 0), all of the same sums along the row
+    const f32x2 xy2 = pk(-kShift, -kShift), sp = pk(2.f * kShift * kShift, kShift * kShift);
+    f32x2 u = 0ull, v = 0ull;
+#pragma unroll
+    for (int t = 0; t < kTaps; t++) {
+      u = fma2(a.g2[t], xy2, u);
+      v = fma2(a.g2[t], sp, v);
+    }
+    for (int r = 0; r < skip; r++) {
+#pragma unroll
+      for (int k = 0; k + 1 < 2 * kR; k++) {
+        m01[k] = fma2(a.g2[k + 1], u, m01[k + 1]);
+        m23[k] = fma2(a.g2[k + 1], v, m23[k + 1]);
+      }
+      m01[2 * kR - 1] = mul2(a.g2[kTaps - 1], u);
+      m23[2 * kR - 1] = mul2(a.g2[kTaps - 1], v);
+    }
+  }
+  for (int k = tid; k < 3 * kRows * 2 * kR; k += kLossThreads) {  // the padding of the partials
+    const int c = k % (2 * kR) < kR ? k % (2 * kR) - kR : k % (2 * kR) - kR + kPartW;
+    part[k / (2 * kR) * kPartStride + pad8(c + kPartPad)] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
   float acc = 0.f;
-  const int n_rows = y1 - y0 + 4 * kR;
+  const int n_rows = y1 - r0 + 2 * kR;
+  // output columns of the strip: at the view's edges the window's other half holds no partials
+  const bool own = (strip == 0 || col >= kR) && (strip == vw.strips - 1 || col < kR + kOutW) && x0 + col < W;
   load(0);
   int base = 0;  // ring slot of image row i0
   for (int i0 = 0; i0 < n_rows; i0 += kRows) {
@@ -226,7 +256,7 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_l2_dssim_grad(const __grid_
           }
         }
       }
-      float4 *o = pch + hrow * kPartStride + hrun * (kRun + 1);
+      float4 *o = pch + hrow * kPartStride + hrun * (kRun + 1) + kPartAt;
 #pragma unroll
       for (int j = 0; j < kRun; j++) {
         const float2 u = unpk(h01[j]), v = unpk(h23[j]);
@@ -237,9 +267,7 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_l2_dssim_grad(const __grid_
 
     // along the columns: image row i0 + r completes the moments of row i0 + r - 5, in place
     {
-      const int gxp = x0 - kR + col;
-      const bool x_ok = gxp >= 0 && gxp < W;
-      const bool own = col >= kR && col < kR + kOutW;
+      const bool x_ok = x0 + col < W;
       f32x2 s01[kRows + 2 * kR], s23[kRows + 2 * kR];
 #pragma unroll
       for (int k = 0; k < 2 * kR; k++) {
@@ -248,7 +276,7 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_l2_dssim_grad(const __grid_
       }
 #pragma unroll
       for (int r = 0; r < kRows; r++) {
-        float4 *cell = pch + r * kPartStride + pad8(col);
+        float4 *cell = pch + r * kPartStride + pad8(col) + kPartAt;
         const float4 h = *cell;
         const f32x2 u = pk(h.x, h.y), v = pk(h.z, h.w);
 #pragma unroll
@@ -258,7 +286,7 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_l2_dssim_grad(const __grid_
         }
         s01[r + kTaps - 1] = mul2(a.g2[kTaps - 1], u);
         s23[r + kTaps - 1] = mul2(a.g2[kTaps - 1], v);
-        const int gyp = y0 - 3 * kR + i0 + r;  // its row in the view
+        const int gyp = r0 - kR + i0 + r;  // its row in the view
         float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
         if (x_ok && gyp >= 0 && gyp < H && gyp >= y0 - kR) {
           const float2 mu = unpk(s01[r]), sp = unpk(s23[r]);
@@ -286,11 +314,11 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_l2_dssim_grad(const __grid_
     }
     __syncthreads();
 
-    // along the rows of the partials (the last run's columns beyond kOutW read padding or the next
-    // row's values and are not used)
+    // along the rows of the partials (output columns that the strip does not own have a cut window)
     float4 h2[kRun];
     {
-      const float4 *in = pch + hrow * kPartStride + hrun * (kRun + 1);
+      const float4 *in = pch + hrow * kPartStride + hrun * (kRun + 1);  // column 8 hrun - 8
+      constexpr int kLead = kPartPad - kR;
       f32x2 hab[kRun];
       float hc[kRun];
 #pragma unroll
@@ -300,8 +328,7 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_l2_dssim_grad(const __grid_
       }
 #pragma unroll
       for (int i = 0; i < kRun + 2 * kR; i++) {
-        if (hrun * kRun + i >= kPartW) break;
-        const float4 d = in[i + (i >> 3)];
+        const float4 d = in[pad8(i + kLead)];
         const f32x2 u = pk(d.x, d.y);
 #pragma unroll
         for (int j = 0; j < kRun; j++) {
@@ -320,15 +347,14 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_l2_dssim_grad(const __grid_
     }
     __syncthreads();
     {
-      float4 *o = pch + hrow * kPartStride + hrun * (kRun + 1);
+      float4 *o = pch + hrow * kPartStride + hrun * (kRun + 1) + kPartAt;
 #pragma unroll
       for (int j = 0; j < kRun; j++) o[j] = h2[j];
     }
     __syncthreads();
 
-    // along the columns of the partials: row i0 + r completes output row i0 + r - 20
-    if (col < kOutW) {
-      const int gxo = x0 + col;
+    // along the columns of the partials: image row i0 + r completes output row i0 + r - 10
+    {
       f32x2 sab[kRows + 2 * kR];
       float sc[kRows + 2 * kR];
 #pragma unroll
@@ -338,7 +364,7 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_l2_dssim_grad(const __grid_
       }
 #pragma unroll
       for (int r = 0; r < kRows; r++) {
-        const float4 h = pch[r * kPartStride + pad8(col)];
+        const float4 h = pch[r * kPartStride + pad8(col) + kPartAt];
         const f32x2 u = pk(h.x, h.y);
 #pragma unroll
         for (int t = 0; t < kTaps - 1; t++) {
@@ -347,15 +373,15 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_l2_dssim_grad(const __grid_
         }
         sab[r + kTaps - 1] = mul2(a.g2[kTaps - 1], u);
         sc[r + kTaps - 1] = a.g[kTaps - 1] * h.z;
-        const int gyo = y0 - 4 * kR + i0 + r;
-        if (gyo >= y0 && gyo < y1 && gxo < W) {
+        const int gyo = r0 - 2 * kR + i0 + r;
+        if (own && gyo >= y0 && gyo < y1) {
           int s = base + r - 2 * kR;  // the ring's oldest rows
           s += s < 0 ? kRing : 0;
-          const float2 v = rch[s * kInStride + pad8(col + 2 * kR)];
+          const float2 v = rch[s * kInStride + pad8(col + kR)];
           const float2 f = unpk(sab[r]);
           const float diff = v.x - v.y;
           const float dssim = f.x + 2.f * (v.x - kShift) * f.y + (v.y - kShift) * sc[r];
-          a.dimg[(vw.off + (long long)gyo * W + gxo) * 3 + ch] = 2.f * w_l2 * diff - w_ssim * dssim;
+          a.dimg[(vw.off + (long long)gyo * W + x0 + col) * 3 + ch] = 2.f * w_l2 * diff - w_ssim * dssim;
           acc += w_l2 * diff * diff;
         }
       }
@@ -381,25 +407,67 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_l2_dssim_grad(const __grid_
 }
 
 // Output rows per CTA of a launch over views[0, n): the length whose waves of
-// CTAs (two per SM) take the fewest rows each, 4 kR rows of halo included; a multiple of
-// kRows less the halo, so that the last group is full.
+// CTAs take the fewest groups of rows, the halo's 4 kR rows included (half of it in a view's first rows).
+// One CTA per SM takes 3.4 us a group, two together 4.9, so a last wave that leaves half of the slots idle
+// counts 7 of 10. Lengths are tried where the rows alone, without the rounding to segments and
+// waves, could beat the best so far, and views of one height are counted
+// together: 127 lengths over every view took 24 us at 64 views and 37 at 112, now 1 to 2 (5 at 112
+// heights).
 int loss_segment(const LossView *views, int n, int slots) {
-  int best = 0;
-  long long best_cost = 0;
-  for (int seg = 2 * kRows - 4; seg <= 1020; seg += kRows) {
-    long long ctas = 0;
-    int rows = 0;
-    for (int v = 0; v < n; ++v) {
-      ctas += (long long)views[v].strips * ((views[v].H + seg - 1) / seg);
-      rows = std::max(rows, std::min(views[v].H, seg) + 4 * kR);
+  struct { unsigned H; long long strips; } of[kMaxLossViews];
+  int m = 0;
+  long long strips = 0, rows = 0;
+  unsigned tall = 0;
+  for (int v = 0; v < n; ++v) {
+    const unsigned H = views[v].H;
+    int k = m - 1;
+    while (k >= 0 && k >= m - 8 && of[k].H != H) --k;
+    if (k < 0 || k < m - 8) {
+      k = m++;
+      of[k].H = H;
+      of[k].strips = 0;
     }
-    const long long cost = (ctas + slots - 1) / slots * rows;
-    if (!best || cost < best_cost) {
+    of[k].strips += views[v].strips;
+    strips += views[v].strips;
+    rows += (long long)views[v].strips * H;
+    tall = std::max(tall, H);
+  }
+  const auto cost = [&](unsigned seg, long long ctas) {
+    const unsigned r = seg >= tall ? tall + 2 * kR : std::max(seg + 2 * kR, std::min(seg, tall - seg) + 4 * kR);
+    const long long rem = ctas % slots;
+    return (ctas / slots * 10 + (rem == 0 ? 0 : 2 * rem <= slots ? 7 : 10)) * ((r + kRows - 1) / kRows);
+  };
+  const auto bound = [&](unsigned seg) { return cost(seg, std::max(strips, (rows + seg - 1) / seg)); };
+  const auto exact = [&](unsigned seg) {
+    const unsigned long long inv = ((1ull << 32) + seg - 1) / seg;  // H / seg for H below 4 M, about beyond
+    long long ctas = 0;
+    for (int k = 0; k < m; ++k) ctas += of[k].strips * (long long)(((of[k].H - 1) * inv >> 32) + 1);
+    return cost(seg, ctas);
+  };
+  constexpr unsigned kFirst = 4, kLast = 1020, kMid = 124;
+  const unsigned step = m <= 16 ? 4 : 16;  // the more heights, the less one length fits all of them
+  const auto next = [&](unsigned seg) { return seg + (seg < kMid ? step : 2 * step); };
+  long long bounds[(kMid - kFirst) / 4 + (kLast - kMid) / 8 + 2];
+  unsigned best = kFirst;
+  int q = 0, q_low = 0;
+  for (unsigned seg = kFirst; seg <= kLast; seg = next(seg), ++q) {
+    bounds[q] = bound(seg);
+    if (bounds[q] < bounds[q_low]) {
+      q_low = q;
       best = seg;
-      best_cost = cost;
     }
   }
-  return best;
+  long long best_cost = exact(best);
+  q = 0;
+  for (unsigned seg = kFirst; seg <= kLast; seg = next(seg), ++q) {
+    if (bounds[q] >= best_cost) continue;
+    const long long c = exact(seg);
+    if (c < best_cost) {
+      best_cost = c;
+      best = seg;
+    }
+  }
+  return (int)best;
 }
 
 }  // namespace
@@ -436,7 +504,7 @@ int launch_l2_dssim_grad(const float *img, const float *gt, int n_views, const i
         r.off = off;
         r.W = W;
         r.H = H;
-        r.strips = (W + kOutW - 1) / kOutW;
+        r.strips = std::max(1, (W - 2 * kR + kOutW - 1) / kOutW);  // the first and the last own kR columns more
         const double n = 3.0 * (double)npx;
         r.w_l2 = (float)((double)scale * (1.0 - (double)lambda) / n);
         r.w_ssim = (float)((double)scale * (double)lambda / n);
