@@ -29,7 +29,7 @@
 // included, against 288 for 32 x 32 tiles that recompute it on all sides
 // (52 x 52 -> 42 x 42 -> 32 x 32). Bound: issue (55 % of the slots busy at 12
 // warps per SM) and the FP32 pipe. 64 mixed views (97 M values) took 2.01 ms,
-// now 1.27; one 800^2 view 53 us, now 40; 64 and 112 views of 64^2 35 and 58 us while such a view took two
+// now 1.27; one 800^2 view 53 us, now 40; 64 and 112 views of 64^2 34 and 57 us while such a view took two
 // strips and a search of 24 us, now 21 and 32 (tiles: 22 and 35). Views narrower than a strip leave the
 // other columns idle: 112 views of 32^2 take 21 us, 13 as tiles. Three CTAs per SM spill the sums
 // (112 registers: 1.70 ms without loads in flight, 2.13 with).
