@@ -755,12 +755,15 @@ __global__ void k_prim_attr_grad(Params p, Scene s, Work w, Grads out) {
 }
 
 // The form of the per-primitive sums at degrees 1 and 2: k_prim_sum_regs pays
-// per run of records of one primitive, k_prim_sum_rows per record. How many
-// records a primitive has is known on the device only; about 0.4 (an object) to
-// 1.1 (a room) per pixel are Gaussians and boundary points. 20,000 primitives:
-// 32 pixels per primitive 29 against 47 us (rows against registers), 52 46
-// against 70, 302 107 against 91, 1,600 337 against 184.
-constexpr long long kSumRegsFrom = 160;  // pixels per primitive
+// per run of records of one primitive, k_prim_sum_rows per record, and fills the GPU with fewer records.
+// How many records a primitive has is known on the device only; about 0.4 (an object) to
+// 1.4 (a surface that fills the view) per pixel are Gaussians and boundary points. Pixels per primitive from
+// which the registers are taken, with the backward chain's time (rows against registers, degree 2):
+//   one view of up to a few million pixels, an object: 32 29 against 47 us, 45 120 against 132, 100 87 against
+//   97, 154 81 against 81, 198 79 against 75 (a view-filling wall: 25 212 against 196, 154 163 against 136);
+//   batches, an object: 25 500 against 532 us, 45 411 against 402, 100 321 against 321, 410 238 against
+//   205; a wall: 25 1111 against 1025, 45 975 against 856, 155 781 against 638.
+constexpr long long kSumRegsFrom = 160, kSumRegsFromBatch = 36;
 
 int launch_clear_grads(const Params &p, const Work &w, const Grads &g, cudaStream_t st) {
   const long long most = std::max(1ll, (long long)p.M * (3 * p.ncp + 3 * p.sh_k));  // floats, about
@@ -781,7 +784,7 @@ int launch_chain(const Params &p, const Scene &s, const Work &w, const Grads &g,
     chain_launch(p.P <= kOverlapPixels, k_chain<N>, grid, 256, 0, st, p, s, w, g);
     bool regs = false;
     if constexpr (SurfPoint<N>::M <= 6) {
-      regs = p.P > kSumRegsFrom * (long long)p.M;
+      regs = p.P > (p.P <= kOverlapPixels ? kSumRegsFrom : kSumRegsFromBatch) * (long long)p.M;
       if (regs) chain_launch(p.P <= kOverlapPixels, k_prim_sum_regs<N>, sms * 2, 256, 0, st, w, g);
     }
     if (!regs) chain_launch(p.P <= kOverlapPixels, k_prim_sum_rows<N>, sms * 4, 256, 0, st, w, g, with_cov);
