@@ -445,6 +445,7 @@ int loss_segment(const LossView *views, int n, int slots) {
     return cost(seg, ctas);
   };
   constexpr unsigned kFirst = 4, kLast = 1020, kMid = 124;
+  if (exact(kFirst) <= cost(kFirst, 1)) return (int)kFirst;  // one CTA per SM at most: no length has fewer groups
   const unsigned step = m <= 16 ? 4 : 16;  // the more heights, the less one length fits all of them
   const auto next = [&](unsigned seg) { return seg + (seg < kMid ? step : 2 * step); };
   long long bounds[(kMid - kFirst) / 4 + (kLast - kMid) / 8 + 2];
