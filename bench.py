@@ -199,9 +199,9 @@ def stage_bytes(stage, c, M, ncp, V):
 # DRAM bytes (read + write) per composited pair of the blending kernels, from one
 # ncu capture of four 1024^2 views (profiles/composite_blend_views1024x4.md),
 # valid only for the kernel source they were measured on (else traffic: null)
-BLEND_TRAFFIC = {"source_sha256": "298302ccb3235284a55777b2fcf56451ed88b334cc4becc896df1fae19e0310d",
-                 "composite_fwd": (123715584 + 178526720) / 50625814,
-                 "composite_bwd": (332592896 + 46526208) / 50625814}
+BLEND_TRAFFIC = {"source_sha256": "11aee918e4da13440b843cd475f7c47345367552a9793f464d7ab5cc79da7192",
+                 "composite_fwd": (123853824 + 178640896) / 50625814,
+                 "composite_bwd": (332707840 + 46604544) / 50625814}
 
 
 # Warp instructions per warp visit of the blending kernels (a visit: one warp,
@@ -209,7 +209,7 @@ BLEND_TRAFFIC = {"source_sha256": "298302ccb3235284a55777b2fcf56451ed88b334cc4be
 # capture; the forward keeps the issue slots ~80 % busy, so issue is the
 # ceiling that binds it; same source check as the traffic
 BLEND_ISSUE = {"source_sha256": BLEND_TRAFFIC["source_sha256"],
-               "composite_fwd": 672020532 / 5419084, "composite_bwd": 518734525 / 4948871}
+               "composite_fwd": 666141753 / 5419084, "composite_bwd": 518734525 / 4948871}
 
 
 def _blend_source_matches():

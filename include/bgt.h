@@ -184,8 +184,8 @@ int bgt_get_tile_size(const bgt_handle *h);
  * slightly slower), on = 2 times the kernels of the normal step without
  * counting, on = 0 turns profiling off (BGT_ERR_INVALID_ARG otherwise). bgt_get_profile
  * waits for the last backward and returns device milliseconds of the last
- * forward + backward: ms[0] clears + per-primitive prep, [1] tessellation +
- * raster, [2] I_id, boundary set and foreground counts, [3] compaction and
+ * forward + backward: ms[0] clears, [1] tessellation +
+ * raster, [2] I_id, boundary set, foreground counts and Sigma3D per primitive, [3] compaction and
  * sub-primitive generation (I_uv included), [4] binning + sort,
  * [5] forward blending, [6] backward blending, [7] chain to parameters;
  * *kernels_fwd / *kernels_bwd receive the kernels each pass enqueues.
@@ -207,7 +207,9 @@ bgt_status bgt_get_profile(bgt_handle *h, float ms[8], int *kernels_fwd, int *ke
  * by the summation order of FP32 atomics. */
 typedef struct {
   int tile_size;           /* screen tile edge: 8, 16 or 32 pixels */
-  int raster_prims;        /* primitives each rasterizer warp takes per block, 1..64 (default 8) */
+  int raster_prims;        /* primitives each rasterizer warp takes per block, 1..64 (default 8); fewer, so
+                              without effect, in calls of less than 16 x SMs x raster_prims
+                              (view, primitive) pairs */
   int bwd_dequeue;         /* warp blocks a backward-blending warp takes per queue dequeue, 1..8 (default 1) */
   int chain_blocks_per_sm; /* persistent blocks per SM of the chain-rule kernels, 1..32 (default 8) */
 } bgt_tuning;

@@ -255,7 +255,7 @@ bgt::Scene to_scene(const bgt_scene *s) {
   return bgt::Scene{s->ctrl, s->color, s->opacity, s->r_b, s->log_scale, s->quat, s->sh_degree > 0 ? s->sh : nullptr};
 }
 
-// stage boundaries recorded when profiling: 0 fwd start, 1 after prep, 2 raster,
+// stage boundaries recorded when profiling: 0 fwd start, 1 after the clears, 2 raster,
 // 3 I_id pass, 4 generate, 5 binning, 6 composite fwd; 7 bwd start, 8 composite
 // bwd, 9 chain
 void mark(bgt_handle *h, int i, cudaStream_t st) {
