@@ -210,6 +210,7 @@ class Renderer:
         _abi.check(self.lib.bgt_create(ctypes.byref(cfg), ctypes.byref(h)))
         self.h = h
         self._last_pixels = 0
+        self._forwards = 0  # forward() calls: whose records the handle holds
 
     def close(self):
         if getattr(self, "h", None):
@@ -239,6 +240,7 @@ class Renderer:
         _device_f32(images, "images", 3 * P)
         cam_arr = _camera_array(cams)
         sc = self._scene(scene)
+        self._forwards += 1
         self._check(self.lib.bgt_render_fwd(self.h, ctypes.byref(sc), cam_arr, len(cams), _ptr(images),
                                             _stream(stream)))
         return images
@@ -447,11 +449,14 @@ class _RenderFn(torch.autograd.Function):
         if scene_meta.get("sh_degree", 0) > 0:
             scene["sh"] = sh
         img = renderer.forward(scene, cams)
-        ctx.renderer, ctx.cams, ctx.scene = renderer, cams, scene
+        ctx.renderer, ctx.cams, ctx.scene, ctx.call = renderer, cams, scene, renderer._forwards
         return img
 
     @staticmethod
     def backward(ctx, d_img):
+        if ctx.call != ctx.renderer._forwards:  # the handle holds a later forward's records
+            ctx.renderer.forward(ctx.scene, ctx.cams)
+            ctx.call = ctx.renderer._forwards
         g = ctx.renderer.backward(ctx.scene, ctx.cams, d_img.contiguous())
         return (None, None, None, g["ctrl"], g["color"], g["opacity"], g["r_b"], g["log_scale"], g["quat"],
                 g.get("sh"))
@@ -459,7 +464,9 @@ class _RenderFn(torch.autograd.Function):
 
 def render(renderer, scene, cams):
     """Differentiable render: images [sum W*H, 3]; gradients flow to
-    scene['ctrl'], ['color'], ['opacity'], ['r_b'], ['log_scale'], ['quat'] and ['sh']."""
+    scene['ctrl'], ['color'], ['opacity'], ['r_b'], ['log_scale'], ['quat'] and ['sh'].
+    A renderer holds the records of its last forward: the backward of an
+    earlier one renders its views again first."""
     meta = {"degree": scene["degree"], "bg": scene["bg"], "attr_res": scene.get("attr_res", 1),
             "sh_degree": scene.get("sh_degree", 0)}
     sh = scene.get("sh")

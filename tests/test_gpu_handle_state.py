@@ -129,3 +129,26 @@ def test_loss_right_behind_the_forward(scenes):
     torch.cuda.synchronize()
     for i in range(40):
         assert torch.equal(d[i], want[i % 2]), i
+
+
+def test_autograd_of_two_renders_through_one_renderer(scenes):
+    """Two views rendered one after the other, their losses added: every backward takes its own view's
+    records, whichever forward came last."""
+    import torch
+    from paper_2503_13961_gb300 import render as R
+    sc, _ = scenes.tiny_scene("ico1", noise=0.04, size=(70, 50), r_b=0.03)
+    cams = [[scenes.look_at_camera(eye, (0, 0, 0), 70, 50)] for eye in ((4.0, 0.0, 0.0), (0.0, 3.0, 1.0))]
+    dev = R.scene_to_device(sc)
+    dev["ctrl"].requires_grad_(True)
+    rd = make_renderer(sc, cams[0])
+    alone = [torch.autograd.grad(R.render(rd, dev, c).square().sum(), dev["ctrl"])[0].cpu() for c in cams]
+    assert grad_rel(alone[0], alone[1]) > 10 * GRAD_TOL
+    for order in ((0, 1), (1, 0)):
+        imgs = [R.render(rd, dev, c) for c in cams]
+        got = [None, None]
+        for k in order:
+            got[k] = torch.autograd.grad(imgs[k].square().sum(), dev["ctrl"])[0]
+        assert all(grad_rel(got[k].cpu(), alone[k]) < GRAD_TOL for k in range(2)), order
+    both = torch.autograd.grad(sum(R.render(rd, dev, c).square().sum() for c in cams), dev["ctrl"])[0]
+    assert grad_rel(both.cpu(), alone[0] + alone[1]) < GRAD_TOL
+    rd.sync_status()
